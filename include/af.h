@@ -335,7 +335,8 @@ af_status af_batch_get_tuning(af_batch *batch, af_batch_tuning *out);
  * The first call builds a single-precision view of the map (dense: 36 bytes
  * per voxel of the box; brick-sparse: 16 KB per brick near an observed one;
  * see af_soft_set_view; AF_ERR_CAPACITY if it cannot be allocated) and later
- * calls rebuild it when scans were integrated since; the map's updates must be
+ * calls bring it up to date when scans were integrated since (dense: the
+ * bricks they touched; brick-sparse: rebuilt); the map's updates must be
  * ordered before the call on `stream`. AF_ERR_STATE without a tool or when
  * no axis sample lies beyond r_s. Asynchronous on `stream`. Non-finite
  * inputs give NaN outputs.

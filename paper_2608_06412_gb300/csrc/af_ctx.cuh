@@ -35,6 +35,7 @@ struct af_ctx {
   // map has changed since)
   float* d_dense = nullptr;
   float4* d_cells = nullptr;
+  uint32_t* d_vlist = nullptr;   // bricks to update, then their count
   uint32_t* d_bgrid = nullptr;   // the brick-sparse view: slot per grid brick
   uint32_t* d_skeys = nullptr;   // grid brick of every slot
   uint32_t* d_nslots = nullptr;

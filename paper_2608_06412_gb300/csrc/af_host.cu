@@ -30,8 +30,8 @@ cudaError_t launch_score(const MapView& M, const ToolView& T, const float* d_pts
                          const ScoreSplit& S, int num_sms, cudaStream_t stream);
 cudaError_t launch_export_flags(const MapView& M, uint32_t count, uint8_t* d_flags,
                                 cudaStream_t stream);
-cudaError_t launch_views(const MapView& M, int num_sms, bool fill, float* dense, float4* cells,
-                         cudaStream_t stream);
+cudaError_t launch_views(const MapView& M, int num_sms, bool fill, bool all, uint32_t since,
+                         float* dense, float4* cells, uint32_t* list, cudaStream_t stream);
 cudaError_t launch_soft_seed(const float* d_nrm, uint32_t m, const float* d_table, uint32_t K,
                              float* d_u0, int num_sms, cudaStream_t stream);
 cudaError_t launch_soft(const SoftView& S, bool grad, const float* pts, uint32_t per_point,
@@ -310,6 +310,7 @@ static void free_all(af_ctx* c) {
   cudaFree(c->d_scount);
   cudaFree(c->d_dense);
   cudaFree(c->d_cells);
+  cudaFree(c->d_vlist);
   cudaFree(c->d_bgrid);
   cudaFree(c->d_skeys);
   cudaFree(c->d_nslots);
@@ -835,11 +836,14 @@ static af_status ensure_views(af_ctx* ctx, cudaStream_t s) {
       if (nc >= (1ull << 31))
         return fail(ctx, AF_ERR_CAPACITY, "soft clearance: the map box has too many cells for the dense SDF view");
       if (cudaMalloc(&ctx->d_dense, nd * sizeof(float)) != cudaSuccess ||
-          cudaMalloc(&ctx->d_cells, nc * 2 * sizeof(float4)) != cudaSuccess) {
+          cudaMalloc(&ctx->d_cells, nc * 2 * sizeof(float4)) != cudaSuccess ||
+          cudaMalloc(&ctx->d_vlist, ((size_t)M.pool_blocks + 1) * sizeof(uint32_t)) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(ctx->d_dense);
+        cudaFree(ctx->d_cells);
         ctx->d_dense = nullptr;
         ctx->d_cells = nullptr;
+        ctx->d_vlist = nullptr;
         return fail(ctx, AF_ERR_CAPACITY,
                     "soft clearance: cannot allocate the SDF views (%zu + %zu bytes) of the map box",
                     nd * sizeof(float), nc * 2 * sizeof(float4));
@@ -847,9 +851,17 @@ static af_status ensure_views(af_ctx* ctx, cudaStream_t s) {
       fill = true;
     }
     if (fill || stale) {
+      // scan stamps wrap at 2^32 - 2: then every brick is taken
+      const bool all = fill || !ctx->views_valid || ctx->frame < ctx->views_frame;
       AF_CUDA(ctx, timed(ctx, 4, s, [&] {
-        return af::launch_views(M, ctx->num_sms, fill, ctx->d_dense, ctx->d_cells, s);
+        return af::launch_views(M, ctx->num_sms, fill, all, ctx->views_frame, ctx->d_dense,
+                                ctx->d_cells, ctx->d_vlist, s);
       }));
+      // a captured update has not run yet: the next call updates from where
+      // the view is now
+      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+      if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+      if (!fill && cap != cudaStreamCaptureStatusNone) return AF_OK;
     }
   } else {
     const int gx = M.dim_vox[0] / 8 + 1, gy = M.dim_vox[1] / 8 + 1, gz = M.dim_vox[2] / 8 + 1;
@@ -1074,12 +1086,14 @@ extern "C" af_status af_soft_set_view(af_ctx* ctx, int32_t mode) {
   AF_CUDA(ctx, cudaDeviceSynchronize());
   cudaFree(ctx->d_dense);
   cudaFree(ctx->d_cells);
+  cudaFree(ctx->d_vlist);
   cudaFree(ctx->d_bgrid);
   cudaFree(ctx->d_skeys);
   cudaFree(ctx->d_nslots);
   cudaFree(ctx->d_scells);
   ctx->d_dense = nullptr;
   ctx->d_cells = nullptr;
+  ctx->d_vlist = nullptr;
   ctx->d_bgrid = nullptr;
   ctx->d_skeys = nullptr;
   ctx->d_nslots = nullptr;

@@ -11,8 +11,8 @@
 // interpolation of the TSDF (Sec. 3.2) over voxel centres, tau where
 // unobserved.
 //
-// Views. The hashed map is flattened twice, lazily and only when the map has
-// changed since the last build:
+// Views. The hashed map is flattened twice, lazily: all of it on the first
+// call, then only the bricks that scans have touched since the last one:
 //  * dense : one FP32 SDF per voxel of the map box, row-major (x fastest);
 //  * cells : for every interpolation cell (low corner from one voxel below
 //            the box to its last voxel) its 8 corner values as two float4,
@@ -43,18 +43,39 @@ namespace af {
 // View builds
 // ---------------------------------------------------------------------------
 
-__global__ void k_fill(float* __restrict__ out, size_t n, float value) {
+// Bound by the write bandwidth: 16-byte stores from a grid of resident CTAs.
+__global__ void __launch_bounds__(256) k_fill(float4* __restrict__ out, size_t n, float value) {
+  const float4 v = make_float4(value, value, value, value);
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (size_t)gridDim.x * blockDim.x)
-    out[i] = value;
+    out[i] = v;
 }
 
-// Dense SDF of every allocated brick: S / (w 2^20) divided in double and
-// rounded to single precision; tau where w = 0.
-__global__ void __launch_bounds__(256) k_dense_view(MapView M, float* __restrict__ dense) {
+// Lists the pool bricks whose voxels changed after scan `since` (every brick
+// with `all`): each scan stamps the hash slot of every brick it touches, so
+// the slots say what a view built at an earlier scan lacks, however many scans
+// ago that was. A brick stamped by a scan later than the caller's is listed
+// too, so a replayed launch covers the scans since.
+__global__ void __launch_bounds__(256) k_view_list(MapView M, uint32_t since, int all,
+                                                   uint32_t* __restrict__ list,
+                                                   uint32_t* __restrict__ nlist) {
   const uint32_t count = min(__ldcg(&M.ctl->pool_count), M.pool_blocks);
+  for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < count; b += gridDim.x * blockDim.x) {
+    uint32_t val, stamp = ~0u;
+    const bool found = all || find_slot(M, M.bkey[b], &val, &stamp) >= 0;
+    if (all || (found && stamp != ~0u && stamp > since)) list[atomicAdd(nlist, 1u)] = b;
+  }
+}
+
+// Dense SDF of the listed bricks: S / (w 2^20) divided in double and rounded to
+// single precision; tau where w = 0.
+__global__ void __launch_bounds__(256) k_dense_view(MapView M, const uint32_t* __restrict__ list,
+                                                    const uint32_t* __restrict__ nlist,
+                                                    float* __restrict__ dense) {
+  const uint32_t count = __ldcg(nlist);
   const size_t X = (size_t)M.dim_vox[0], Y = (size_t)M.dim_vox[1];
-  for (uint32_t b = blockIdx.x; b < count; b += gridDim.x) {
+  for (uint32_t k = blockIdx.x; k < count; k += gridDim.x) {
+    const uint32_t b = list[k];
     const uint64_t key = M.bkey[b];
     const size_t bx = (size_t)(key & 0x1FFFFF) * 8, by = (size_t)((key >> 21) & 0x1FFFFF) * 8,
                  bz = (size_t)(key >> 42) * 8;
@@ -68,25 +89,46 @@ __global__ void __launch_bounds__(256) k_dense_view(MapView M, float* __restrict
   }
 }
 
-__device__ inline float dense_at(const float* __restrict__ dense, int x, int y, int z, int X,
-                                 int Y, int Z, float tau) {
-  if (x < 0 || y < 0 || z < 0 || x >= X || y >= Y || z >= Z) return tau;
-  return dense[((size_t)z * Y + y) * X + x];
-}
+// Corner records of the cells that read a voxel of a listed brick: low corners
+// from one voxel below the brick to its last voxel, 9^3 cells, from the 10^3
+// voxels around it. One CTA per brick, the voxels staged in shared memory, the
+// records written in runs of nine (288 bytes). Neighbouring bricks of the list
+// write the cells they share twice, with the same values. Bound by the record
+// writes: a scan of the pine stream changes about 900 bricks, 21 MB of records.
+// Rebuilding all 3.7 GB of that box instead took 1.21 ms after each scan; a
+// step of scan, scoring and refinement of its 12k points went from 1.56 ms to
+// 0.35 ms.
+constexpr int kCellEdge = kBrick + 1, kCornerEdge = kBrick + 2;
 
-// Corner records of every cell whose low corner lies in [-1, dim) per axis.
-__global__ void __launch_bounds__(256) k_cell_view(const float* __restrict__ dense, int X, int Y,
-                                                   int Z, float tau, float4* __restrict__ cells) {
-  const size_t NX = (size_t)X + 1, NY = (size_t)Y + 1, n = NX * NY * ((size_t)Z + 1);
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const int x = (int)(i % NX) - 1, y = (int)((i / NX) % NY) - 1, z = (int)(i / (NX * NY)) - 1;
-    float c[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      c[k] = dense_at(dense, x + (k & 1), y + ((k >> 1) & 1), z + (k >> 2), X, Y, Z, tau);
-    cells[2 * i] = make_float4(c[0], c[1], c[2], c[3]);
-    cells[2 * i + 1] = make_float4(c[4], c[5], c[6], c[7]);
+__global__ void __launch_bounds__(256) k_cell_view(MapView M, const uint32_t* __restrict__ list,
+                                                   const uint32_t* __restrict__ nlist,
+                                                   const float* __restrict__ dense,
+                                                   float4* __restrict__ cells) {
+  __shared__ float s_d[kCornerEdge * kCornerEdge * kCornerEdge];
+  const uint32_t count = __ldcg(nlist);
+  const int X = M.dim_vox[0], Y = M.dim_vox[1], Z = M.dim_vox[2];
+  for (uint32_t k = blockIdx.x; k < count; k += gridDim.x) {
+    const uint64_t key = M.bkey[list[k]];
+    const int bx = (int)(key & 0x1FFFFF) * 8, by = (int)((key >> 21) & 0x1FFFFF) * 8,
+              bz = (int)(key >> 42) * 8;
+    __syncthreads();  // the previous brick's voxels are no longer read
+    for (int i = threadIdx.x; i < kCornerEdge * kCornerEdge * kCornerEdge; i += blockDim.x) {
+      const int x = bx - 1 + i % kCornerEdge, y = by - 1 + (i / kCornerEdge) % kCornerEdge,
+                z = bz - 1 + i / (kCornerEdge * kCornerEdge);
+      const bool in = (unsigned)x < (unsigned)X && (unsigned)y < (unsigned)Y && (unsigned)z < (unsigned)Z;
+      s_d[i] = in ? __ldcg(dense + ((size_t)z * Y + y) * X + x) : M.tau;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kCellEdge * kCellEdge * kCellEdge; i += blockDim.x) {
+      const int cx = i % kCellEdge, cy = (i / kCellEdge) % kCellEdge, cz = i / (kCellEdge * kCellEdge);
+      const float* c = s_d + (cz * kCornerEdge + cy) * kCornerEdge + cx;
+      // cell index = low corner + 1 on each axis (the lowest cells lie below the box)
+      float4* rec = cells + 2 * (((size_t)(bz + cz) * ((size_t)Y + 1) + (size_t)(by + cy)) * ((size_t)X + 1) +
+                                 (size_t)(bx + cx));
+      constexpr int sy = kCornerEdge, sz = kCornerEdge * kCornerEdge;
+      rec[0] = make_float4(c[0], c[1], c[sy], c[sy + 1]);
+      rec[1] = make_float4(c[sz], c[sz + 1], c[sz + sy], c[sz + sy + 1]);
+    }
   }
 }
 
@@ -676,14 +718,24 @@ cudaError_t launch_sview_fill(const MapView& M, int num_sms, const uint32_t* key
   return cudaGetLastError();
 }
 
-cudaError_t launch_views(const MapView& M, int num_sms, bool fill, float* dense, float4* cells,
-                         cudaStream_t stream) {
-  const size_t nd = (size_t)M.dim_vox[0] * M.dim_vox[1] * M.dim_vox[2];
-  if (fill) k_fill<<<grid_for(nd, 256, num_sms, 8), 256, 0, stream>>>(dense, nd, M.tau);
-  k_dense_view<<<(unsigned)num_sms * 8, 256, 0, stream>>>(M, dense);
+// Brings the dense view up to date with the map: the bricks changed after scan
+// `since`, or every brick (`all`); with `fill` the buffers are new and every
+// value starts as tau.
+cudaError_t launch_views(const MapView& M, int num_sms, bool fill, bool all, uint32_t since,
+                         float* dense, float4* cells, uint32_t* list, cudaStream_t stream) {
+  const size_t nd = (size_t)M.dim_vox[0] * M.dim_vox[1] * M.dim_vox[2];  // a multiple of 512
   const size_t nc = ((size_t)M.dim_vox[0] + 1) * (M.dim_vox[1] + 1) * (M.dim_vox[2] + 1);
-  k_cell_view<<<grid_for(nc, 256, num_sms, 8), 256, 0, stream>>>(dense, M.dim_vox[0], M.dim_vox[1],
-                                                                  M.dim_vox[2], M.tau, cells);
+  if (fill) {
+    k_fill<<<grid_for(nd / 4, 256, num_sms, 8), 256, 0, stream>>>(reinterpret_cast<float4*>(dense),
+                                                                   nd / 4, M.tau);
+    k_fill<<<grid_for(nc * 2, 256, num_sms, 8), 256, 0, stream>>>(cells, nc * 2, M.tau);
+  }
+  uint32_t* nlist = list + M.pool_blocks;
+  cudaError_t e = cudaMemsetAsync(nlist, 0, sizeof(uint32_t), stream);
+  if (e != cudaSuccess) return e;
+  k_view_list<<<grid_for(M.pool_blocks, 256, num_sms, 8), 256, 0, stream>>>(M, since, all ? 1 : 0, list, nlist);
+  k_dense_view<<<(unsigned)num_sms * 8, 256, 0, stream>>>(M, list, nlist, dense);
+  k_cell_view<<<(unsigned)num_sms * 8, 256, 0, stream>>>(M, list, nlist, dense, cells);
   return cudaGetLastError();
 }
 
