@@ -26,8 +26,8 @@ struct af_ctx {
   bool has_tool = false;
   af::ToolView T{};
   float* d_dirs = nullptr;
-  short4* d_runs = nullptr;
-  int2* d_fruns = nullptr;
+  int2* d_qent = nullptr;
+  uint4* d_qmask = nullptr;
   int4* d_dtab = nullptr;
   short4* d_arm = nullptr;
   af_tool tool{};

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <array>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdlib>
@@ -143,21 +144,27 @@ bool member(const af_tool& t, double v, const double u[3], int ox, int oy, int o
   return a > L && a <= L + (double)t.corr_length && rho2 <= r * r;
 }
 
-// Offsets of one kernel, enumerating the axis-aligned box that holds the
-// cylinder (with one voxel of margin), z-major.
-std::vector<Offset> rasterise(const af_tool& t, double v, const double u[3], int which) {
-  std::vector<Offset> out;
+// The axis-aligned box that holds the cylinder (with one voxel of margin);
+// false if the kernel is empty.
+bool kernel_box(const af_tool& t, double v, const double u[3], int which, int lo[3], int hi[3]) {
   const double a0 = which == AF_KERNEL_TOOL ? 0.0 : (double)t.length;
   const double a1 = which == AF_KERNEL_TOOL ? (double)t.length
                                             : (double)t.length + (double)t.corr_length;
   const double r = which == AF_KERNEL_TOOL ? (double)t.radius : (double)t.corr_radius;
-  if (which == AF_KERNEL_CORRIDOR && !(t.corr_length > 0.f)) return out;
-  int lo[3], hi[3];
+  if (which == AF_KERNEL_CORRIDOR && !(t.corr_length > 0.f)) return false;
   for (int k = 0; k < 3; ++k) {
     const double p = a0 * u[k], q = a1 * u[k];
     lo[k] = (int)std::floor((std::min(p, q) - r) / v) - 1;
     hi[k] = (int)std::ceil((std::max(p, q) + r) / v) + 1;
   }
+  return true;
+}
+
+// Offsets of one kernel, z-major.
+std::vector<Offset> rasterise(const af_tool& t, double v, const double u[3], int which) {
+  std::vector<Offset> out;
+  int lo[3], hi[3];
+  if (!kernel_box(t, v, u, which, lo, hi)) return out;
   for (int oz = lo[2]; oz <= hi[2]; ++oz)
     for (int oy = lo[1]; oy <= hi[1]; ++oy)
       for (int ox = lo[0]; ox <= hi[0]; ++ox)
@@ -165,46 +172,128 @@ std::vector<Offset> rasterise(const af_tool& t, double v, const double u[3], int
   return out;
 }
 
-// The axis a direction's runs follow: the one it is closest to (largest
+// The same as runs along `axis`: voxels [s, e) of the row (d1, d2), d1 along the
+// lower of the other two axes, and the axial distance of the run's nearer end.
+struct Run {
+  int d1, d2, s, e;
+  double a;
+};
+
+std::vector<Run> rasterise_runs(const af_tool& t, double v, const double u[3], int which, int axis) {
+  std::vector<Run> out;
+  int lo[3], hi[3], o[3];
+  if (!kernel_box(t, v, u, which, lo, hi)) return out;
+  const int o1 = axis == 0 ? 1 : 0, o2 = axis == 2 ? 1 : 2;
+  auto axial = [&](int k) {
+    o[axis] = k;
+    return ((double)o[0] * v * u[0] + (double)o[1] * v * u[1]) + (double)o[2] * v * u[2];
+  };
+  for (o[o2] = lo[o2]; o[o2] <= hi[o2]; ++o[o2])
+    for (o[o1] = lo[o1]; o[o1] <= hi[o1]; ++o[o1])
+      for (int k = lo[axis]; k <= hi[axis];) {
+        auto in = [&](int i) {
+          o[axis] = i;
+          return member(t, v, u, o[0], o[1], o[2], which);
+        };
+        if (!in(k)) {
+          ++k;
+          continue;
+        }
+        int e = k + 1;
+        while (e <= hi[axis] && in(e)) ++e;
+        out.push_back({o[o1], o[o2], k, e, std::min(axial(k), axial(e - 1))});
+        k = e + 1;
+      }
+  return out;
+}
+
+// The axis a direction's rows follow: the one it is closest to (largest
 // |u_k|, the lowest k on ties).
 int run_axis(const double u[3]) {
   int a = std::fabs(u[1]) > std::fabs(u[0]) ? 1 : 0;
   return std::fabs(u[2]) > std::fabs(u[a]) ? 2 : a;
 }
 
-// Groups offsets into runs of at most 64 voxels along `axis`, ordered by the
-// axial distance of their first voxel (near runs first: blocking geometry
-// next to the surface is met early). A run is (d_axis, len | axis << 8,
-// d_o1, d_o2), o1 < o2 the other two axes.
-void to_runs(const std::vector<Offset>& offs, double v, const double u[3], int axis,
-             std::vector<short4>* runs) {
-  struct R {
+// One entry of a direction's kernel (af_score.cuh): a 2 x 2 group of rows at
+// group offset (q1, q2) from the point's, the 32 - spare voxels from d0 on
+// along the rows' axis, one mask per row.
+struct Quad {
+  double a;  // axial distance of its nearest voxel, for the order
+  int q1, q2, d0, spare;
+  uint32_t mask[4];
+};
+
+// Groups a kernel's runs along one axis into quads, once per parity p of the
+// point's coordinates (o1, o2) across it (p = (o1 & 1) | (o2 & 1) << 1): out[p],
+// ordered by axial distance (near ones first: blocking geometry next to the
+// surface is met early).
+void to_quads(const std::vector<Run>& runs, std::vector<Quad> out[4]) {
+  struct Piece {
+    int q1, q2, s, e, row;
     double a;
-    short4 s;
   };
-  const int o1 = axis == 0 ? 1 : 0, o2 = axis == 2 ? 1 : 2;
-  std::vector<std::array<int, 3>> c(offs.size());
-  for (size_t k = 0; k < offs.size(); ++k) c[k] = {offs[k].x, offs[k].y, offs[k].z};
-  std::sort(c.begin(), c.end(), [&](const std::array<int, 3>& p, const std::array<int, 3>& q) {
-    if (p[o2] != q[o2]) return p[o2] < q[o2];
-    if (p[o1] != q[o1]) return p[o1] < q[o1];
-    return p[axis] < q[axis];
-  });
-  std::vector<R> rs;
-  size_t i = 0;
-  while (i < c.size()) {
-    size_t j = i + 1;
-    while (j < c.size() && c[j][o1] == c[i][o1] && c[j][o2] == c[i][o2] &&
-           c[j][axis] == c[j - 1][axis] + 1 && (int)(j - i) < 64)
-      ++j;
-    const std::array<int, 3>& o = c[i];
-    const double a = ((double)o[0] * v * u[0] + (double)o[1] * v * u[1]) + (double)o[2] * v * u[2];
-    rs.push_back({a, make_short4((short)o[axis], (short)((int)(j - i) | (axis << 8)), (short)o[o1],
-                                 (short)o[o2])});
-    i = j;
+  std::vector<Piece> pieces(runs.size());
+  for (int p = 0; p < 4; ++p) {
+    const int p1 = p & 1, p2 = p >> 1;
+    for (size_t k = 0; k < runs.size(); ++k) {
+      const Run& r = runs[k];
+      pieces[k] = {(p1 + r.d1) >> 1, (p2 + r.d2) >> 1, r.s, r.e,
+                   ((p1 + r.d1) & 1) | (((p2 + r.d2) & 1) << 1), r.a};
+    }
+    std::sort(pieces.begin(), pieces.end(), [](const Piece& x, const Piece& y) {
+      if (x.q2 != y.q2) return x.q2 < y.q2;
+      if (x.q1 != y.q1) return x.q1 < y.q1;
+      if (x.s != y.s) return x.s < y.s;
+      return x.row < y.row;
+    });
+    std::vector<Quad>& q = out[p];
+    for (size_t i = 0; i < pieces.size();) {
+      size_t j = i;
+      while (j < pieces.size() && pieces[j].q1 == pieces[i].q1 && pieces[j].q2 == pieces[i].q2) ++j;
+      // windows of 32 over the group's pieces, from the lowest voxel not yet taken
+      int from = pieces[i].s;
+      while (true) {
+        int lo = INT_MAX;
+        for (size_t k = i; k < j; ++k)
+          if (pieces[k].e > from) lo = std::min(lo, std::max(pieces[k].s, from));
+        if (lo == INT_MAX) break;
+        int hi = lo;
+        Quad w{1e300, pieces[i].q1, pieces[i].q2, lo, 0, {0, 0, 0, 0}};
+        for (size_t k = i; k < j; ++k) {
+          const int s = std::max(pieces[k].s, lo), e = std::min(pieces[k].e, lo + 32);
+          if (s >= e) continue;
+          w.mask[pieces[k].row] |= (uint32_t)(((1ull << (e - s)) - 1ull) << (s - lo));
+          w.a = std::min(w.a, pieces[k].a);
+          hi = std::max(hi, e);
+        }
+        w.spare = 32 - (hi - lo);
+        q.push_back(w);
+        from = lo + 32;
+      }
+      i = j;
+    }
+    std::stable_sort(q.begin(), q.end(), [](const Quad& x, const Quad& y) { return x.a < y.a; });
   }
-  std::stable_sort(rs.begin(), rs.end(), [](const R& p, const R& q) { return p.a < q.a; });
-  for (const R& r : rs) runs->push_back(r.s);
+}
+
+// Appends the four parities of one kernel to the tables, each as long as the
+// longest (a filler has empty masks); returns the entries per parity.
+int append_quads(const std::vector<Quad> quads[4], std::vector<int2>* ent, std::vector<uint4>* mask) {
+  size_t n = 0;
+  for (int p = 0; p < 4; ++p) n = std::max(n, quads[p].size());
+  for (int p = 0; p < 4; ++p)
+    for (size_t k = 0; k < n; ++k) {
+      if (k >= quads[p].size()) {
+        ent->push_back(make_int2(0, 31));
+        mask->push_back(make_uint4(0, 0, 0, 0));
+        continue;
+      }
+      const Quad& q = quads[p][k];
+      ent->push_back(make_int2((int)(((uint32_t)q.q1 & 0xFFFFu) | ((uint32_t)q.q2 << 16)),
+                               (int)(((uint32_t)q.d0 << 16) | (uint32_t)q.spare)));
+      mask->push_back(make_uint4(q.mask[0], q.mask[1], q.mask[2], q.mask[3]));
+    }
+  return (int)n;
 }
 
 void arm_offsets(double v, double tau, const double u[3], int out[9]) {
@@ -266,13 +355,13 @@ extern "C" af_status af_arm_offsets(float voxel_size, float truncation, const fl
 
 static void free_tool(af_ctx* c) {
   cudaFree(c->d_dirs);
-  cudaFree(c->d_runs);
-  cudaFree(c->d_fruns);
+  cudaFree(c->d_qent);
+  cudaFree(c->d_qmask);
   cudaFree(c->d_dtab);
   cudaFree(c->d_arm);
   c->d_dirs = nullptr;
-  c->d_runs = nullptr;
-  c->d_fruns = nullptr;
+  c->d_qent = nullptr;
+  c->d_qmask = nullptr;
   c->d_dtab = nullptr;
   c->d_arm = nullptr;
   c->has_tool = false;
@@ -386,12 +475,13 @@ extern "C" af_status af_create(const af_config* cfg, af_ctx** out) {
     M.dom_vox[k] = cfg->domain_min[k] * 8;
     M.dim_vox[k] = (int)cfg->domain_bricks[k] * 8;
   }
-  M.row_words = (M.dim_vox[0] + 63) / 64;
-  M.row_words_y = (M.dim_vox[1] + 63) / 64;
-  M.row_words_z = (M.dim_vox[2] + 63) / 64;
-  M.words_x = (size_t)M.row_words * M.dim_vox[1] * M.dim_vox[2];
-  M.words_y = (size_t)M.row_words_y * M.dim_vox[0] * M.dim_vox[2];
-  M.words_z = (size_t)M.row_words_z * M.dim_vox[0] * M.dim_vox[1];
+  M.rw = 2 * ((M.dim_vox[0] + 63) / 64);
+  M.rw_y = 2 * ((M.dim_vox[1] + 63) / 64);
+  M.rw_z = 2 * ((M.dim_vox[2] + 63) / 64);
+  // box edges are multiples of 8, so row groups of 2 x 2 are whole
+  M.quads = (size_t)M.rw * (M.dim_vox[1] / 2) * (M.dim_vox[2] / 2);
+  M.quads_y = (size_t)M.rw_y * (M.dim_vox[0] / 2) * (M.dim_vox[2] / 2);
+  M.quads_z = (size_t)M.rw_z * (M.dim_vox[0] / 2) * (M.dim_vox[1] / 2);
   M.hmask = cfg->hash_capacity - 1;
   M.pool_blocks = cfg->pool_blocks;
   {
@@ -417,7 +507,6 @@ extern "C" af_status af_create(const af_config* cfg, af_ctx** out) {
     return AF_OK;
   };
   const size_t H = cfg->hash_capacity, P = cfg->pool_blocks;
-  const size_t plane = (size_t)M.row_words * 8 * M.dim_vox[1] * M.dim_vox[2];
   const size_t R = cfg->max_returns, Pm = cfg->max_points;
   af_status st = AF_OK;
   if (st == AF_OK) st = alloc((void**)&M.slots, H * sizeof(af::HashSlot), 0xFF);
@@ -425,12 +514,10 @@ extern "C" af_status af_create(const af_config* cfg, af_ctx** out) {
   if (st == AF_OK) st = alloc((void**)&M.cleared, P * 16 * 4, 0);
   if (st == AF_OK) st = alloc((void**)&M.bkey, P * 8, 0);
   if (st == AF_OK) st = alloc((void**)&M.dirty, P * 4, 0);
-  if (st == AF_OK) st = alloc((void**)&M.occ, plane, 0);
-  if (st == AF_OK) st = alloc((void**)&M.known, plane, 0);
-  if (st == AF_OK)
-    st = alloc((void**)&M.occ_y, (size_t)M.row_words_y * 8 * M.dim_vox[0] * M.dim_vox[2], 0);
-  if (st == AF_OK)
-    st = alloc((void**)&M.occ_z, (size_t)M.row_words_z * 8 * M.dim_vox[0] * M.dim_vox[1], 0);
+  if (st == AF_OK) st = alloc((void**)&M.occ, M.quads * 16, 0);
+  if (st == AF_OK) st = alloc((void**)&M.known, M.quads * 16, 0);
+  if (st == AF_OK) st = alloc((void**)&M.occ_y, M.quads_y * 16, 0);
+  if (st == AF_OK) st = alloc((void**)&M.occ_z, M.quads_z * 16, 0);
   if (st == AF_OK) st = alloc((void**)&M.ctl, sizeof(af::Control), 0);
   if (st == AF_OK) st = alloc((void**)&c->d_ret, R * sizeof(float4), 0);
   if (st == AF_OK) st = alloc((void**)&M.rtab, R * (size_t)M.nbmax * 4, 0);
@@ -441,7 +528,7 @@ extern "C" af_status af_create(const af_config* cfg, af_ctx** out) {
   if (st == AF_OK) st = alloc((void**)&c->d_best, Pm * 2, 0);
   if (st == AF_OK) st = alloc((void**)&c->d_over, Pm * sizeof(int2), 0);
   if (st == AF_OK) st = alloc((void**)&c->d_sres, Pm * 4, 0);
-  if (st == AF_OK) st = alloc((void**)&c->d_scount, 16, 0);  // split count, staged counters
+  if (st == AF_OK) st = alloc((void**)&c->d_scount, 4, 0);  // split count
   c->split_cap = (uint32_t)Pm;
   if (st == AF_OK && cudaMallocHost((void**)&c->h_status, 64) != cudaSuccess)
     st = fail(c, AF_ERR_CUDA, "pinned allocation failed");
@@ -546,62 +633,53 @@ extern "C" af_status af_set_tool(af_ctx* ctx, const af_tool* tool, const float* 
 
   const double v = (double)ctx->cfg.voxel_size, tau = (double)ctx->cfg.truncation;
   int reach[3] = {0, 0, 0};
-  std::vector<short4> runs, cruns;  // tool runs of every direction, then corridor runs
+  std::vector<int2> ent, cent;  // tool entries of every direction, then corridor entries
+  std::vector<uint4> mask, cmask;
   std::vector<int4> dtab(G);
   std::vector<short4> arm(3 * G);
   for (uint32_t g = 0; g < G; ++g) {
     const double u[3] = {(double)h_dirs[3 * g], (double)h_dirs[3 * g + 1], (double)h_dirs[3 * g + 2]};
-    const std::vector<Offset> tool_o = rasterise(*tool, v, u, AF_KERNEL_TOOL);
-    const std::vector<Offset> corr_o = rasterise(*tool, v, u, AF_KERNEL_CORRIDOR);
-    for (const std::vector<Offset>* o : {&tool_o, &corr_o})
-      for (const Offset& x : *o)
-        if (std::abs(x.x) > 32000 || std::abs(x.y) > 32000 || std::abs(x.z) > 32000)
-          return fail(ctx, AF_ERR_INVALID_ARG, "tool reach exceeds 32000 voxels");
-    // runs along the direction's closest axis; the strict corridor also reads
+    // rows along the direction's closest axis; the strict corridor also reads
     // the known view, which has x rows only
-    const int ax = run_axis(u);
-    dtab[g].x = (int)runs.size();
-    to_runs(tool_o, v, u, ax, &runs);
-    dtab[g].y = (int)runs.size();
-    dtab[g].z = (int)cruns.size();
-    to_runs(corr_o, v, u, tool->corridor_strict ? 0 : ax, &cruns);
-    dtab[g].w = (int)cruns.size();
-    for (const std::vector<Offset>* o : {&tool_o, &corr_o})
-      for (const Offset& x : *o) {
-        reach[0] = std::max(reach[0], std::abs(x.x));
-        reach[1] = std::max(reach[1], std::abs(x.y));
-        reach[2] = std::max(reach[2], std::abs(x.z));
+    const int ax = run_axis(u), cax = tool->corridor_strict ? 0 : ax;
+    const std::vector<Run> tool_r = rasterise_runs(*tool, v, u, AF_KERNEL_TOOL, ax);
+    const std::vector<Run> corr_r = rasterise_runs(*tool, v, u, AF_KERNEL_CORRIDOR, cax);
+    for (int which = 0; which < 2; ++which) {
+      const int a = which ? cax : ax, o1 = a == 0 ? 1 : 0, o2 = a == 2 ? 1 : 2;
+      for (const Run& r : which ? corr_r : tool_r) {
+        reach[a] = std::max(reach[a], std::max(std::abs(r.s), std::abs(r.e - 1)));
+        reach[o1] = std::max(reach[o1], std::abs(r.d1));
+        reach[o2] = std::max(reach[o2], std::abs(r.d2));
       }
+    }
+    for (int k = 0; k < 3; ++k)
+      if (reach[k] > 32000) return fail(ctx, AF_ERR_INVALID_ARG, "tool reach exceeds 32000 voxels");
+    std::vector<Quad> quads[4], cquads[4];
+    to_quads(tool_r, quads);
+    to_quads(corr_r, cquads);
+    dtab[g].x = (int)ent.size() | (int)((uint32_t)ax << af::kAxisShift);
+    dtab[g].y = append_quads(quads, &ent, &mask);
+    dtab[g].z = (int)cent.size();
+    dtab[g].w = append_quads(cquads, &cent, &cmask);
+    if (ent.size() + cent.size() > (size_t)af::kEntryMask)
+      return fail(ctx, AF_ERR_INVALID_ARG, "af_set_tool: the tool's kernels are too large");
     int a[9];
     arm_offsets(v, tau, u, a);
     for (int k = 0; k < 3; ++k)
       arm[3 * g + k] = make_short4((short)a[3 * k], (short)a[3 * k + 1], (short)a[3 * k + 2], 0);
   }
-  const int ntool = (int)runs.size();
-  for (uint32_t g = 0; g < G; ++g) {
-    dtab[g].z += ntool;
-    dtab[g].w += ntool;
+  for (uint32_t g = 0; g < G; ++g) dtab[g].z += (int)ent.size();
+  ent.insert(ent.end(), cent.begin(), cent.end());
+  mask.insert(mask.end(), cmask.begin(), cmask.end());
+  if (ent.empty()) {  // keep the buffers non-empty
+    ent.push_back(make_int2(0, 31));
+    mask.push_back(make_uint4(0, 0, 0, 0));
   }
-  runs.insert(runs.end(), cruns.begin(), cruns.end());
-  if (runs.empty()) runs.push_back(make_short4(0, 1, 0, 0));  // keep the buffer non-empty
-  // Fast-path form of the runs: the plane-word offset of the run's row relative to
-  // the point's row, valid while every plane index fits in 31 bits. `reach` bounds
-  // every offset, so a point at least `reach` voxels inside the box needs no checks.
+  // `reach` bounds every offset, so a point at least `reach` voxels inside the
+  // box needs no checks; its indices are 32-bit, so every view must have less
+  // than 2^31 elements
   const MapView& M = ctx->M;
-  const int X = M.dim_vox[0], Y = M.dim_vox[1], Z = M.dim_vox[2];
-  const bool fast_ok = (int64_t)M.row_words * Y * Z < (1ll << 31) &&
-                       (int64_t)M.row_words_y * X * Z < (1ll << 31) &&
-                       (int64_t)M.row_words_z * X * Y < (1ll << 31);
-  // plane rows: axis x -> row z * Y + y; axis y -> z * X + x; axis z -> y * X + x
-  const int dim_o1[3] = {Y, X, X};
-  const int rw[3] = {M.row_words, M.row_words_y, M.row_words_z};
-  std::vector<int2> fruns(runs.size());
-  for (size_t r = 0; r < runs.size(); ++r) {
-    const short4 s = runs[r];
-    const int ax = ((uint16_t)s.y >> 8) & 3, len = (uint16_t)s.y & 0xFF;
-    const int64_t delta = ((int64_t)s.w * dim_o1[ax] + s.z) * rw[ax];
-    fruns[r] = make_int2((int)delta, (int)(uint16_t)s.x | (len << 16) | (ax << 24));
-  }
+  const bool fast_ok = M.quads < (1ull << 31) && M.quads_y < (1ull << 31) && M.quads_z < (1ull << 31);
   for (const short4& a : arm) {
     reach[0] = std::max(reach[0], std::abs((int)a.x));
     reach[1] = std::max(reach[1], std::abs((int)a.y));
@@ -611,22 +689,21 @@ extern "C" af_status af_set_tool(af_ctx* ctx, const af_tool* tool, const float* 
   AF_CUDA(ctx, cudaDeviceSynchronize());
   free_tool(ctx);
   AF_CUDA(ctx, cudaMalloc((void**)&ctx->d_dirs, (size_t)G * 12));
-  AF_CUDA(ctx, cudaMalloc((void**)&ctx->d_runs, runs.size() * sizeof(short4)));
-  AF_CUDA(ctx, cudaMalloc((void**)&ctx->d_fruns, fruns.size() * sizeof(int2)));
-  AF_CUDA(ctx, cudaMemcpy(ctx->d_fruns, fruns.data(), fruns.size() * sizeof(int2), cudaMemcpyHostToDevice));
+  AF_CUDA(ctx, cudaMalloc((void**)&ctx->d_qent, ent.size() * sizeof(int2)));
+  AF_CUDA(ctx, cudaMalloc((void**)&ctx->d_qmask, mask.size() * sizeof(uint4)));
+  AF_CUDA(ctx, cudaMemcpy(ctx->d_qent, ent.data(), ent.size() * sizeof(int2), cudaMemcpyHostToDevice));
+  AF_CUDA(ctx, cudaMemcpy(ctx->d_qmask, mask.data(), mask.size() * sizeof(uint4), cudaMemcpyHostToDevice));
   for (int k = 0; k < 3; ++k) ctx->T.reach[k] = reach[k];
-  ctx->T.fruns = ctx->d_fruns;
-  ctx->T.ntool = ntool;
-  ctx->T.nruns = (int)runs.size();
+  ctx->T.qent = ctx->d_qent;
+  ctx->T.qmask = ctx->d_qmask;
+  ctx->T.nent = (int)ent.size();
   ctx->T.ctl = ctx->M.ctl;
   AF_CUDA(ctx, cudaMalloc((void**)&ctx->d_dtab, (size_t)G * sizeof(int4)));
   AF_CUDA(ctx, cudaMalloc((void**)&ctx->d_arm, (size_t)G * 3 * sizeof(short4)));
   AF_CUDA(ctx, cudaMemcpy(ctx->d_dirs, h_dirs, (size_t)G * 12, cudaMemcpyHostToDevice));
-  AF_CUDA(ctx, cudaMemcpy(ctx->d_runs, runs.data(), runs.size() * sizeof(short4), cudaMemcpyHostToDevice));
   AF_CUDA(ctx, cudaMemcpy(ctx->d_dtab, dtab.data(), (size_t)G * sizeof(int4), cudaMemcpyHostToDevice));
   AF_CUDA(ctx, cudaMemcpy(ctx->d_arm, arm.data(), (size_t)G * 3 * sizeof(short4), cudaMemcpyHostToDevice));
   ctx->T.dirs = ctx->d_dirs;
-  ctx->T.runs = ctx->d_runs;
   ctx->T.dtab = ctx->d_dtab;
   ctx->T.arm = ctx->d_arm;
   ctx->T.G = (int)G;
@@ -656,8 +733,7 @@ extern "C" af_status af_score(af_ctx* ctx, const float* d_pts, const float* d_no
     AF_CUDA(ctx, cudaMalloc((void**)&ctx->d_sres, (size_t)m * 4));
     ctx->split_cap = m;
   }
-  const af::ScoreSplit S{ctx->d_over, ctx->d_sres, ctx->d_scount, ctx->score_budget,
-                         ctx->d_scount + 1};
+  const af::ScoreSplit S{ctx->d_over, ctx->d_sres, ctx->d_scount, ctx->score_budget};
   if (m > 0)
     AF_CUDA(ctx, timed(ctx, 3, s, [&] {
               return af::launch_score(ctx->M, ctx->T, d_pts, d_normals, m, d_label, d_best, S,

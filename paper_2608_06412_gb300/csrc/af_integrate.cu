@@ -395,7 +395,6 @@ __device__ void bitview_brick(const MapView& M, uint32_t blk) {
   const int lane = threadIdx.x & 31;
   unsigned char* occ = reinterpret_cast<unsigned char*>(M.occ);
   unsigned char* known = reinterpret_cast<unsigned char*>(M.known);
-  const size_t row_bytes = (size_t)M.row_words * 8;
   const uint64_t key = M.bkey[blk];
   const uint32_t bx = (uint32_t)(key & 0x1FFFFF), by = (uint32_t)((key >> 21) & 0x1FFFFF),
                  bz = (uint32_t)(key >> 42);
@@ -419,10 +418,9 @@ __device__ void bitview_brick(const MapView& M, uint32_t blk) {
     const unsigned kb = __ballot_sync(0xffffffffu, kn);
     if (lane == 0) s_ob[wi] = ob;
     if (lane < 4) {
-      const size_t y = (size_t)by * 8 + (wi & 1) * 4 + lane;
-      const size_t z = (size_t)bz * 8 + (wi >> 1);
-      const size_t at = (z * (size_t)M.dim_vox[1] + y) * row_bytes + bx;
-      if (check_index(at < M.words_x * 8, M.ctl)) {
+      const int y = (int)by * 8 + (wi & 1) * 4 + lane, z = (int)bz * 8 + (wi >> 1);
+      const size_t at = view_byte(M.rw, M.dim_vox[1], y, z, (int)bx);
+      if (check_index(at < M.quads * 16, M.ctl)) {
         occ[at] = (unsigned char)(ob >> (8 * lane));
         known[at] = (unsigned char)(kb >> (8 * lane));
       }
@@ -439,16 +437,14 @@ __device__ void bitview_brick(const MapView& M, uint32_t blk) {
       const int v = l < 64 ? x + 8 * k + 64 * c : x + 8 * c + 64 * k;
       byte |= ((s_ob[v >> 5] >> (v & 31)) & 1u) << k;
     }
-    const size_t X = (size_t)M.dim_vox[0], xa = (size_t)bx * 8 + x;
+    const int X = M.dim_vox[0], xa = (int)bx * 8 + x;
     if (l < 64) {
-      const size_t z = (size_t)bz * 8 + c;
-      const size_t at = (z * X + xa) * ((size_t)M.row_words_y * 8) + by;
-      if (check_index(at < M.words_y * 8, M.ctl))
+      const size_t at = view_byte(M.rw_y, X, xa, (int)bz * 8 + c, (int)by);
+      if (check_index(at < M.quads_y * 16, M.ctl))
         reinterpret_cast<unsigned char*>(M.occ_y)[at] = (unsigned char)byte;
     } else {
-      const size_t y = (size_t)by * 8 + c;
-      const size_t at = (y * X + xa) * ((size_t)M.row_words_z * 8) + bz;
-      if (check_index(at < M.words_z * 8, M.ctl))
+      const size_t at = view_byte(M.rw_z, X, xa, (int)by * 8 + c, (int)bz);
+      if (check_index(at < M.quads_z * 16, M.ctl))
         reinterpret_cast<unsigned char*>(M.occ_z)[at] = (unsigned char)byte;
     }
   }
@@ -474,10 +470,10 @@ __global__ void __launch_bounds__(512) k_export_flags(MapView M, uint8_t* __rest
   const int x = (int)(key & 0x1FFFFF) * 8 + (l & 7);
   const int y = (int)((key >> 21) & 0x1FFFFF) * 8 + ((l >> 3) & 7);
   const int z = (int)(key >> 42) * 8 + (l >> 6);
-  const size_t word = ((size_t)z * M.dim_vox[1] + y) * M.row_words + (x >> 6);
+  const size_t at = view_byte(M.rw, M.dim_vox[1], y, z, x >> 3);
   const unsigned cl = (M.cleared[blk * 16 + (l >> 5)] >> (l & 31)) & 1u;
-  const unsigned oc = (unsigned)(M.occ[word] >> (x & 63)) & 1u;
-  const unsigned kn = (unsigned)(M.known[word] >> (x & 63)) & 1u;
+  const unsigned oc = ((unsigned)reinterpret_cast<const unsigned char*>(M.occ)[at] >> (x & 7)) & 1u;
+  const unsigned kn = ((unsigned)reinterpret_cast<const unsigned char*>(M.known)[at] >> (x & 7)) & 1u;
   flags[(size_t)blk * kBrickVox + l] = (uint8_t)(cl | (oc << 1) | (kn << 2));
 }
 

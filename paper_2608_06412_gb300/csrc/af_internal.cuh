@@ -14,13 +14,16 @@
 //             guaranteed by max_returns + w_cap < 2^20, |S| < 2^40 by
 //             tau <= 1 m; S is the arithmetic shift of the word by 20.
 //             Next to it: 512 cleared bits per brick and the brick key.
-//  * planes : the occupied and known views as dense bit planes over the map
-//             box, one bit per voxel, rows along x (64 voxels per u64 word),
-//             row index z * Y + y. A brick row of 8 voxels is one byte, so the
-//             view of a brick is 64 byte stores per plane. The occupied view
-//             is also kept with rows along y (row index z * X + x) and along
-//             z (row index y * X + x), so a kernel run can follow whichever
-//             axis its direction is closest to.
+//  * views  : the occupied and known views as dense bit planes over the map
+//             box, one bit per voxel, rows along x in 32-bit words. The words
+//             of a 2 x 2 group of rows (two neighbours on each of the other
+//             axes) lie side by side, so a 16-byte element holds the same 32
+//             voxels of four rows; elements of a group run along the axis,
+//             groups along the lower of the other two axes. A brick row of 8
+//             voxels is one byte, so the view of a brick is 64 byte stores per
+//             plane. The occupied view is also kept with rows along y and
+//             along z, so a kernel can follow whichever axis its direction is
+//             closest to.
 #pragma once
 
 #include <cstdint>
@@ -36,6 +39,8 @@ constexpr int kBrickVox = 512;
 constexpr int kWBits = 20;
 constexpr uint64_t kWMask = (1ull << kWBits) - 1;
 constexpr float kScale = 1048576.0f;  // 2^20
+constexpr int kAxisShift = 30;  // a direction entry's axis bits, above its entry index
+constexpr int kEntryMask = (1 << kAxisShift) - 1;
 
 // Latched device status (values of af_status).
 constexpr uint32_t kStatusCapacity = 2;
@@ -77,6 +82,13 @@ __host__ __device__ inline long long capped_S(long long S, long long w_cap, long
   return (a % w != 0 && a < 0) ? q - 1 : q;
 }
 
+// Byte of the 8 voxels `b` (from 8 b on, along the rows' axis) of the row at
+// (o1, o2) in a view of rw words per row and O1 rows along o1.
+__host__ __device__ inline size_t view_byte(int rw, int O1, int o1, int o2, int b) {
+  return ((((size_t)(o2 >> 1) * (O1 >> 1) + (o1 >> 1)) * rw + (b >> 2)) << 4) +
+         (((o1 & 1) | ((o2 & 1) << 1)) << 2) + (b & 3);
+}
+
 struct MapView {
   // geometry
   float v, tau, r_c, cone_cos, range_min, range_max, clear_lo, clear_hi;
@@ -89,10 +101,9 @@ struct MapView {
   float dlo;          // lower clamp of d: 0, or -tau with clamp_signed
   int dom_vox[3];     // absolute voxel index of the box's min corner
   int dim_vox[3];     // box size in voxels (multiples of 8)
-  int row_words;      // u64 words per plane row
-  unsigned long long* occ_y;  // occupied, rows along y: row z * X + x
-  unsigned long long* occ_z;  // occupied, rows along z: row y * X + x
-  int row_words_y, row_words_z;
+  int rw, rw_y, rw_z; // 32-bit words per view row along x, y, z
+  uint4* occ_y;       // occupied, rows along y: row groups (x, z)
+  uint4* occ_z;       // occupied, rows along z: row groups (x, y)
   // hash
   struct HashSlot* slots;
   uint32_t hmask;     // capacity - 1
@@ -105,11 +116,11 @@ struct MapView {
   // per-scan scratch: the pool index of each cube brick of each return
   uint32_t* rtab;           // max_returns * nbmax
   int nbmax;                // bricks a cube can span: ((2m + 7) / 8 + 1)^3
-  // planes
-  unsigned long long* occ;
-  unsigned long long* known;
+  // views, rows along x: row groups (y, z)
+  uint4* occ;
+  uint4* known;
   Control* ctl;
-  size_t words_x, words_y, words_z;  // 64-bit words of the x-row views, of occ_y, of occ_z
+  size_t quads, quads_y, quads_z;  // elements of the x-row views, of occ_y, of occ_z
 };
 
 // Tool tables on the device (built by af_set_tool).
@@ -121,24 +132,22 @@ struct ScoreSplit {
   uint32_t* res;     // packed (score << 16 | direction) of the search so far
   uint32_t* count;   // points handed off
   int budget;        // directions past the arm screen before a hand-off; < 0: never
-  uint32_t* work;    // the staged scorer's next-point and finished-warp counters (zero
-                     // between launches)
 };
 
 struct ToolView {
   const float* dirs;      // G x 3 unit directions
-  const short4* runs;     // x-runs (dx0, len, dy, dz), len in 1..64
-  const int2* fruns;      // the same runs as (row delta in plane words, dx0 | len << 16)
-  const int4* dtab;       // per direction: tool runs [x, y), corridor runs [z, w)
+  const int4* dtab;       // per direction: first tool entry | axis << kAxisShift, tool entries per
+                          // parity, first corridor entry, corridor entries per parity
+  const int2* qent;       // entries: (row-group offsets q1 | q2 << 16, d0 << 16 | 32 - window)
+  const uint4* qmask;     // ... and their masks, row (o1 & 1) | (o2 & 1) << 1 of the group
   const short4* arm;      // G x 3 arm-sample offsets
-  int ntool;              // every direction's tool runs come first: runs [0, ntool)
   int G;
   int n_c;
   float cos_max;
   int strict;
   int reach[3];           // largest |offset| per axis over every kernel and arm sample
-  int nruns;              // entries of runs / fruns
-  Control* ctl;           // the map's status word (the checked build's run-index checks)
+  int nent;               // entries of qent / qmask
+  Control* ctl;           // the map's status word (the checked build's index checks)
 };
 
 __host__ __device__ inline uint64_t pack_brick(uint32_t bx, uint32_t by, uint32_t bz) {

@@ -1,21 +1,16 @@
 // af_score.cu -- accessibility scoring on sm_103a (Sec. 3.4, 3.5 of the paper).
 //
-// One warp per surface point. The plain form (k_score_staged) is a persistent
-// grid whose CTAs first copy the direction table, the arm offsets and the
-// tool runs into shared memory; the batched form and tables too large to
-// stage read them through the read-only path (k_score, k_score_batch).
+// One warp per surface point.
 // The lanes first evaluate the normal filter for
-// 32 directions at a time (ballot -> candidate mask); the candidates are then
-// visited in index order, each by the whole warp:
-//   * tool kernel: lanes take x-runs of the precomputed kernel (32 runs per
-//     step), fetch the run's bits from the occupied plane with one or two
-//     64-bit loads, AND with the run mask and __popc; a warp sum saturates
-//     at the score to beat, so counting stops as soon as the direction can
-//     no longer improve the point;
-//   * arm samples: three single-bit lookups (occupied or unknown blocks);
-//   * corridor: runs as above, any set bit blocks (__any_sync early exit);
-//   * once a best exists, the arm-clear candidates are counted two at a time
-//     (half a warp each) and then decided in index order.
+// 32 directions at a time (ballot -> candidate mask), then the arm samples of
+// each candidate (three single-bit lookups: occupied or unknown blocks). The
+// arm-clear candidates are taken four at a time in index order:
+//   * tool kernel: 8 lanes per direction fetch the kernel's entries (the same
+//     32 voxels of four rows in one or two 16-byte loads), AND with the masks
+//     and __popc; the count saturates at the score to beat, so it stops as
+//     soon as the direction can no longer improve the point;
+//   * corridor: the whole warp, two entries per lane per step, any set bit
+//     blocks (__any_sync early exit).
 // The best direction is the lowest-index minimum; a score of 0 ends the
 // point. Every early exit returns exactly what a full evaluation of every
 // candidate would (the score to beat only shrinks; ties keep the lower
@@ -39,7 +34,7 @@
 namespace af {
 
 // Scores point pi with the whole warp (all 32 lanes call this together).
-template <bool SPLIT, bool SM = false>
+template <bool SPLIT>
 __device__ void score_point(const MapView& M, const ToolView& T, const float* __restrict__ pts,
                             const float* __restrict__ nrm, uint32_t pi,
                             uint8_t* __restrict__ label, int16_t* __restrict__ best_out,
@@ -47,51 +42,58 @@ __device__ void score_point(const MapView& M, const ToolView& T, const float* __
   const float s0 = pts[3 * pi], s1 = pts[3 * pi + 1], s2 = pts[3 * pi + 2];
   const float n0 = nrm[3 * pi], n1 = nrm[3 * pi + 1], n2 = nrm[3 * pi + 2];
 
-  // the point's voxel and its weight (confidence gate, Sec. 3.5)
-  int i0, i1, i2;
+  // The point's voxel and its weight (confidence gate, Sec. 3.5). Three
+  // dependent loads lead to the weight (point, hash slot, voxel word): the
+  // slot's is in flight while the candidates are found, the word's while the
+  // first directions are screened.
+  int i0 = 0, i1 = 0, i2 = 0;
   const bool ok =
       voxel_index(s0, M, &i0) && voxel_index(s1, M, &i1) && voxel_index(s2, M, &i2);
   Pt P;
   P.px = i0 - M.dom_vox[0];
   P.py = i1 - M.dom_vox[1];
   P.pz = i2 - M.dom_vox[2];
-  uint32_t w = 0;
-  if (ok && (unsigned)P.px < (unsigned)M.dim_vox[0] && (unsigned)P.py < (unsigned)M.dim_vox[1] &&
-      (unsigned)P.pz < (unsigned)M.dim_vox[2]) {
-    uint32_t blk = kNoBlock;
-    if (lane == 0) blk = lookup_brick(M, pack_brick(P.px >> 3, P.py >> 3, P.pz >> 3));
-    blk = __shfl_sync(0xffffffffu, blk, 0);
-    if (blk != kNoBlock) {
-      const int l = (P.px & 7) | ((P.py & 7) << 3) | ((P.pz & 7) << 6);
-      w = (uint32_t)(__ldcg(M.vox + (size_t)blk * kBrickVox + l) & kWMask);
-    }
+  const bool in = ok && (unsigned)P.px < (unsigned)M.dim_vox[0] &&
+                  (unsigned)P.py < (unsigned)M.dim_vox[1] && (unsigned)P.pz < (unsigned)M.dim_vox[2];
+  const uint64_t key = in ? pack_brick(P.px >> 3, P.py >> 3, P.pz >> 3) : kEmptyKey;
+  unsigned long long found = kEmptyKey;
+  uint32_t blk = kNoBlock, stamp;
+  if (in) load_slot(M, hash_slot(key, M.hmask), &found, &blk, &stamp);
+
+  // nominal tests: every candidate direction of this point
+  int ncand = 0;
+  KeptFilter F{{n0, n1, n2}, 0u};
+  for (int gb = 0; gb < T.G; gb += 32) {
+    const unsigned m = __ballot_sync(0xffffffffu, candidate(T, gb + lane, n0, n1, n2));
+    ncand += __popc(m);
+    if (lane == gb >> 5) F.kept = m;
   }
-  if (w < M.w_min) {
+
+  if (found != key) blk = found == kEmptyKey ? kNoBlock : lookup_brick(M, key);  // the same in all lanes
+  unsigned long long word = 0;
+  if (in && blk < M.pool_blocks)
+    word = __ldcg(M.vox + (size_t)blk * kBrickVox + ((P.px & 7) | ((P.py & 7) << 3) | ((P.pz & 7) << 6)));
+  const auto confident = [&] { return (uint32_t)(word & kWMask) >= M.w_min; };
+
+  const bool fast = reach_inside(M, T, P);
+  int2 res;
+  int next = -1;
+  if (!SPLIT) {
+    res = fast ? best_direction<true>(M, T, P, F, lane, confident)
+               : best_direction<false>(M, T, P, F, lane, confident);
+  } else {
+    res = make_int2(-1, -1);
+    if (confident())
+      res = fast ? best_direction_budget<true>(M, T, P, F, lane, S.budget, &next)
+                 : best_direction_budget<false>(M, T, P, F, lane, S.budget, &next);
+  }
+  if (res.x < 0) {  // not confident
     if (lane == 0) {
       label[pi] = 0;
       best_out[pi] = -1;
     }
     return;
   }
-
-  // nominal tests: every candidate direction of this point
-  int ncand = 0;
-  for (int gb = 0; gb < T.G; gb += 32)
-    ncand += __popc(__ballot_sync(0xffffffffu, candidate(T, gb + lane, n0, n1, n2)));
-
-  const bool fast = P.px >= T.reach[0] && P.px + T.reach[0] < M.dim_vox[0] &&
-                    P.py >= T.reach[1] && P.py + T.reach[1] < M.dim_vox[1] &&
-                    P.pz >= T.reach[2] && P.pz + T.reach[2] < M.dim_vox[2];
-  int2 res;
-  int next = -1;
-  if (fast) set_rows(M, P); else P.row = P.rowy = P.rowz = 0;
-  const NormalFilter F{n0, n1, n2};
-  if (!SPLIT)
-    res = fast ? best_direction<true, NormalFilter, SM>(M, T, P, F, lane)
-               : best_direction<false, NormalFilter, SM>(M, T, P, F, lane);
-  else
-    res = fast ? best_direction_budget<true, NormalFilter, SM>(M, T, P, F, lane, S.budget, &next)
-               : best_direction_budget<false, NormalFilter, SM>(M, T, P, F, lane, S.budget, &next);
 
   if (lane == 0) {
     if (next < 0) {
@@ -107,58 +109,20 @@ __device__ void score_point(const MapView& M, const ToolView& T, const float* __
   }
 }
 
+// Threads per SM the scorers are built for: 40 warps at 48 registers. A lane's
+// two entries in flight (16-byte loads and masks) want 60 registers; fewer warps
+// hide less latency (32 warps: 66 against 62 us per pine frame), more spill (48
+// warps at 40 registers: 66 us).
+constexpr int kScoreThreads = 1280;
+
 template <int WARPS, bool SPLIT>
-__global__ void __launch_bounds__(WARPS * 32, 2048 / (WARPS * 32))
+__global__ void __launch_bounds__(WARPS * 32, kScoreThreads / (WARPS * 32))
     k_score(MapView M, ToolView T, const float* __restrict__ pts, const float* __restrict__ nrm,
             uint32_t m, uint8_t* __restrict__ label, int16_t* __restrict__ best_out,
             ScoreSplit S) {
   const uint32_t pi = blockIdx.x * WARPS + (threadIdx.x >> 5);
   if (pi >= m) return;  // whole warp
   score_point<SPLIT>(M, T, pts, nrm, pi, label, best_out, threadIdx.x & 31, S);
-}
-
-// Shared-memory bytes of the staged scorer's tables: direction table (16 B
-// per direction), arm offsets (24 B per direction), tool runs (8 B per run).
-__host__ __device__ inline size_t staged_bytes(const ToolView& T) {
-  return (size_t)T.G * 40 + (size_t)T.ntool * 8;
-}
-// Tables up to 100 KB are staged (two CTAs of 32 warps still fit an SM's
-// 228 KB); larger ones (many directions, long tools) are read through the
-// read-only path.
-constexpr size_t kStagedMaxBytes = 100 * 1024;
-
-// The staged form of k_score: a persistent CTA copies the direction table,
-// the arm offsets and every direction's tool runs into shared memory once,
-// so that each step of a point's search waits on one L2 load (the plane
-// word) instead of a table entry and then a plane word. A warp scores point
-// (its warp index) first, then takes points from a launch-wide counter; the
-// last warp to finish zeroes the counters for the next launch (every other
-// warp has then taken its last point). The search itself is the same.
-template <int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, 2048 / (WARPS * 32))
-    k_score_staged(MapView M, ToolView T, const float* __restrict__ pts,
-                   const float* __restrict__ nrm, uint32_t m, uint8_t* __restrict__ label,
-                   int16_t* __restrict__ best_out, uint32_t* __restrict__ work) {
-  short4* s_arm = reinterpret_cast<short4*>(af_staged_tab + T.G);
-  int2* s_runs = reinterpret_cast<int2*>(reinterpret_cast<char*>(af_staged_tab) + 40 * T.G);
-  for (int i = threadIdx.x; i < T.G; i += WARPS * 32) af_staged_tab[i] = __ldg(T.dtab + i);
-  for (int i = threadIdx.x; i < 3 * T.G; i += WARPS * 32) s_arm[i] = __ldg(T.arm + i);
-  for (int i = threadIdx.x; i < T.ntool; i += WARPS * 32) s_runs[i] = __ldg(T.fruns + i);
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const uint32_t nw = gridDim.x * WARPS;
-  uint32_t pi = blockIdx.x * WARPS + (threadIdx.x >> 5);
-  while (pi < m) {
-    score_point<false, true>(M, T, pts, nrm, pi, label, best_out, lane,
-                             ScoreSplit{nullptr, nullptr, nullptr, -1, nullptr});
-    uint32_t nxt = 0;
-    if (lane == 0) nxt = nw + atomicAdd(work, 1u);
-    pi = __shfl_sync(0xffffffffu, nxt, 0);
-  }
-  if (lane == 0 && atomicAdd(work + 1, 1u) == nw - 1u) {
-    work[0] = 0u;
-    work[1] = 0u;
-  }
 }
 
 // One (point, direction) item of a handed-off search; the whole warp.
@@ -182,13 +146,13 @@ __device__ void split_item(const MapView& M, const ToolView& T, const Pt& P, int
     if (!exact && sat == 0) return;
     const int c = tool_count<FAST>(M, T, g, P, sat, lane);
     if (!exact && c >= sat) return;
-    mine = corridor_blocked<FAST>(M, T, g, P, lane) ? pack_result(make_int2(nc + 1, g))
+    mine = corridor_blocked<FAST>(M, T, __ldg(T.dtab + g), P, lane) ? pack_result(make_int2(nc + 1, g))
                                                    : pack_result(make_int2(min(c, nc), g));
   }
   if (lane == 0 && mine < cur) atomicMin(res, mine);
 }
 
-__global__ void __launch_bounds__(128, 16)
+__global__ void __launch_bounds__(128, kScoreThreads / 128)
     k_score_split(MapView M, ToolView T, const float* __restrict__ pts,
                   const float* __restrict__ nrm, ScoreSplit S) {
   const int lane = threadIdx.x & 31;
@@ -210,10 +174,7 @@ __global__ void __launch_bounds__(128, 16)
     P.px = i0 - M.dom_vox[0];
     P.py = i1 - M.dom_vox[1];
     P.pz = i2 - M.dom_vox[2];
-    const bool fast = P.px >= T.reach[0] && P.px + T.reach[0] < M.dim_vox[0] &&
-                      P.py >= T.reach[1] && P.py + T.reach[1] < M.dim_vox[1] &&
-                      P.pz >= T.reach[2] && P.pz + T.reach[2] < M.dim_vox[2];
-    if (fast) set_rows(M, P); else P.row = P.rowy = P.rowz = 0;
+    const bool fast = reach_inside(M, T, P);
     if (fast)
       split_item<true>(M, T, P, g, S.res + o, lane);
     else
@@ -238,25 +199,6 @@ cudaError_t launch_score(const MapView& M, const ToolView& T, const float* d_pts
                          const float* d_nrm, uint32_t m, uint8_t* d_label, int16_t* d_best,
                          const ScoreSplit& S, int num_sms, cudaStream_t stream) {
   if (m == 0) return cudaSuccess;
-  constexpr int kStagedWarps = 32;
-  if (S.budget < 0 && S.work != nullptr && staged_bytes(T) <= kStagedMaxBytes) {
-    const size_t smem = staged_bytes(T);
-    int per = 0;
-    cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024) {  // above the default dynamic shared-memory limit: opt in
-      e = cudaFuncSetAttribute(k_score_staged<kStagedWarps>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per, k_score_staged<kStagedWarps>, kStagedWarps * 32, smem);
-    if (e != cudaSuccess) return e;
-    const uint32_t need = (m + kStagedWarps - 1) / kStagedWarps;
-    const uint32_t grid = std::min<uint32_t>(need, (uint32_t)num_sms * (uint32_t)(per > 0 ? per : 1));
-    k_score_staged<kStagedWarps><<<grid, kStagedWarps * 32, smem, stream>>>(
-        M, T, d_pts, d_nrm, m, d_label, d_best, S.work);
-    return cudaGetLastError();
-  }
   constexpr int WARPS = 2;
   if (S.budget >= 0) {
     cudaError_t e = cudaMemsetAsync(S.count, 0, sizeof(uint32_t), stream);
@@ -269,7 +211,7 @@ cudaError_t launch_score(const MapView& M, const ToolView& T, const float* d_pts
     k_score<WARPS, false><<<(m + WARPS - 1) / WARPS, WARPS * 32, 0, stream>>>(M, T, d_pts, d_nrm,
                                                                              m, d_label, d_best, S);
   if (S.budget >= 0) {
-    k_score_split<<<num_sms * 16, 128, 0, stream>>>(M, T, d_pts, d_nrm, S);
+    k_score_split<<<num_sms * (kScoreThreads / 128), 128, 0, stream>>>(M, T, d_pts, d_nrm, S);
     k_score_finish<<<num_sms, 256, 0, stream>>>(S, T.n_c, d_label, d_best);
   }
   return cudaGetLastError();
@@ -279,7 +221,7 @@ cudaError_t launch_score(const MapView& M, const ToolView& T, const float* d_pts
 // Batched ticks: every point of every map of the batch, one warp per point,
 // persistent grid (see af_batch.cu).
 template <int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, 2048 / (WARPS * 32))
+__global__ void __launch_bounds__(WARPS * 32, kScoreThreads / (WARPS * 32))
     k_score_batch(const BatchHdr* __restrict__ B, const SceneDesc* __restrict__ D) {
   const uint32_t total = B->total_points;
   const int count = (int)B->count;

@@ -1,14 +1,30 @@
 // af_score.cuh -- the scoring device functions (Sec. 3.4, 3.5), shared by the
 // plain, batched and stateful-layer scoring kernels.
 //
-// Kernels are runs rather than voxel lists: a cylinder meets every row in
-// one interval (two at most next to the self-exclusion ball), so a run of up
-// to 64 voxels costs one or two loads of a bit plane. Each direction's runs
-// follow the axis it is closest to, read from the occupied view with rows
-// along that axis, so a kernel is a few long runs instead of many short
-// ones. A point whose whole kernel reach lies inside the map box takes the
-// FAST path: the run table then holds each run's row as a plane-word offset
-// from the point's row on that plane, and no bound is checked.
+// Kernels are quads rather than voxel lists. The views keep the 32-bit words of
+// a 2 x 2 group of rows side by side (af_internal.cuh), so one 16-byte load
+// reads 32 voxels of four neighbouring rows. A kernel's voxels are grouped the
+// same way: an entry is a group of rows (as an offset from the point's group),
+// a window of up to 32 voxels along the rows' axis and one mask per row. Which
+// voxels share a group depends on the parity of the point's coordinates across
+// the axis, so each direction has its entries four times, once per parity; the
+// position along the axis is free (a funnel shift of the two words the window
+// may straddle). Each direction follows the axis it is closest to, read from
+// the occupied view with rows along that axis.
+//
+// Why quads: the search of a point is a chain of dependent loads, one warp step
+// each, and off-axis kernels cut rows into short runs (7 voxels on average for
+// the 1 m corridor at 2 cm). Per direction of the 4 cm tool a run each row takes
+// 32 tool and 143 corridor loads, quads about 12 and 47: a tool fits 8 or 16
+// lanes, so four directions are counted side by side, and a corridor is walked
+// in one or two steps instead of five. Against runs with their tables staged in
+// shared memory: 72.5 -> 61 us per pine frame (12k points, 128 directions), 489
+// -> 328 us for 40k points of three pines with the 6 cm tool and
+// 256 directions, 2.47 -> 1.47 ms for 83k points of a 1 cm map with 512.
+//
+// A point whose whole kernel reach lies inside the map box takes the FAST path,
+// which checks no bound; otherwise words outside the box read as zero: nothing
+// occupied, nothing known.
 #pragma once
 
 #include "af_internal.cuh"
@@ -17,234 +33,175 @@ namespace af {
 
 struct Pt {
   int px, py, pz;  // box-relative voxel of the point
-  int row;         // plane-word index of the point's x row (FAST path only)
-  int rowy, rowz;  // ... of its y row and z row
 };
 
-// The point's row bases on the three planes (FAST path).
-__device__ inline void set_rows(const MapView& M, Pt& P) {
-  P.row = (P.pz * M.dim_vox[1] + P.py) * M.row_words;
-  P.rowy = (P.pz * M.dim_vox[0] + P.px) * M.row_words_y;
-  P.rowz = (P.py * M.dim_vox[0] + P.px) * M.row_words_z;
+// Whether every voxel that any kernel or arm sample reaches from P lies inside
+// the map box.
+__device__ __forceinline__ bool reach_inside(const MapView& M, const ToolView& T, const Pt& P) {
+  return P.px >= T.reach[0] && P.px + T.reach[0] < M.dim_vox[0] && P.py >= T.reach[1] &&
+         P.py + T.reach[1] < M.dim_vox[1] && P.pz >= T.reach[2] && P.pz + T.reach[2] < M.dim_vox[2];
 }
 
-// Bits a0 .. a0+len-1 along axis `ax` of the plane row at the other two
-// coordinates (o1, o2) (o1 the lower axis), bit i = voxel a0 + i; voxels
-// outside the map box read 0 and set *outside.
-__device__ inline unsigned long long row_bits(const unsigned long long* __restrict__ plane,
-                                              const MapView& M, int ax, int x0, int o1, int o2,
-                                              int len, bool* outside) {
-  const int A = M.dim_vox[ax];
-  const int O1 = ax == 0 ? M.dim_vox[1] : M.dim_vox[0];
-  const int O2 = ax == 2 ? M.dim_vox[1] : M.dim_vox[2];
-  const int rw = ax == 0 ? M.row_words : (ax == 1 ? M.row_words_y : M.row_words_z);
-  if ((unsigned)o1 >= (unsigned)O1 || (unsigned)o2 >= (unsigned)O2) {
-    *outside = true;
-    return 0ull;
-  }
-  int xa = x0, xb = x0 + len - 1;
-  if (xa < 0 || xb >= A) {
-    *outside = true;
-    xa = max(xa, 0);
-    xb = min(xb, A - 1);
-    if (xa > xb) return 0ull;
-  }
-  const unsigned long long* row = plane + ((size_t)o2 * O1 + o1) * rw;
-  const int wa = xa >> 6, wb = xb >> 6, sh = xa & 63;
-  const size_t words = ax == 0 ? M.words_x : (ax == 1 ? M.words_y : M.words_z);
-  if (!check_index(((size_t)o2 * O1 + o1) * rw + wb < words, M.ctl)) return 0ull;
-  unsigned long long win = __ldg(row + wa) >> sh;
-  if (wb != wa) win |= __ldg(row + wb) << (64 - sh);
-  const int n = xb - xa + 1;
-  if (n < 64) win &= (1ull << n) - 1ull;
-  return win << (xa - x0);
-}
-
-// One run-table entry: the fast form (plane-word row offset,
-// d0 | len << 16 | axis << 24) or the plain form (d0 | (len | axis << 8) << 16,
-// d1 | d2 << 16), d0 along the run's axis, d1 < d2 the other two axes.
-struct RunEntry {
-  int a, b;
+// A direction's entries as seen from a point: tool entries [t0, t0 + nt) and
+// corridor entries [c0, c0 + nc) of the point's parity, the axis of its rows,
+// and the point's place on the view with rows along that axis.
+struct DirRows {
+  int t0, nt, c0, nc;
+  const uint4* view;
+  int axis;
+  int a, o1, o2;  // the point's coordinates: along the rows, and the other two (o1 the lower axis)
 };
 
-// The staged scorer's copy of the tool tables in dynamic shared memory, in
-// this order: the direction table (G int4), the arm offsets (3 G short4) and
-// the tool runs in fast form (ntool int2, byte offset 40 G).
-extern __shared__ int4 af_staged_tab[];
+// Parity of the point's row group: which copy of a direction's entries applies.
+__device__ __forceinline__ int parity(int o1, int o2) { return (o1 & 1) | ((o2 & 1) << 1); }
 
-__device__ __forceinline__ int4 dtab_entry(const ToolView& T, int g, bool staged) {
-  return staged ? af_staged_tab[g] : __ldg(T.dtab + g);
+// `d`: the direction's table entry. `along_x`: its corridor entries follow x
+// (strict) whatever the direction's axis.
+__device__ __forceinline__ DirRows dir_rows(const MapView& M, const Pt& P, int4 d, bool along_x = false) {
+  DirRows r;
+  r.axis = along_x ? 0 : (int)((uint32_t)d.x >> kAxisShift);
+  r.view = r.axis == 0 ? M.occ : (r.axis == 1 ? M.occ_y : M.occ_z);
+  r.a = r.axis == 0 ? P.px : (r.axis == 1 ? P.py : P.pz);
+  r.o1 = r.axis == 0 ? P.py : P.px;
+  r.o2 = r.axis == 2 ? P.py : P.pz;
+  r.nt = d.y;
+  r.nc = d.w;
+  r.t0 = (d.x & kEntryMask) + parity(r.o1, r.o2) * d.y;
+  r.c0 = d.z + parity(r.o1, r.o2) * d.w;
+  return r;
 }
 
-__device__ __forceinline__ short4 arm_entry(const ToolView& T, int i, bool staged) {
-  return staged ? reinterpret_cast<const short4*>(af_staged_tab + T.G)[i] : __ldg(T.arm + i);
-}
-
-// Run r of the tables; SM: a tool run read from the staged copy.
-template <bool FAST, bool SM = false>
-__device__ inline RunEntry load_run(const ToolView& T, int r) {
-  if (!check_index((unsigned)r < (unsigned)(SM ? T.ntool : T.nruns), T.ctl)) return {0, 0};  // an empty run
-  if (FAST) {
-    const int2 f = SM ? reinterpret_cast<const int2*>(
-                            reinterpret_cast<const char*>(af_staged_tab) + 40 * T.G)[r]
-                      : __ldg(T.fruns + r);
-    return {f.x, f.y};
-  }
-  const short4 s = __ldg(T.runs + r);
-  return {(int)((uint32_t)(uint16_t)s.x | ((uint32_t)(uint16_t)s.y << 16)),
-          (int)((uint32_t)(uint16_t)s.z | ((uint32_t)(uint16_t)s.w << 16))};
-}
-
-// Bits of the run of entry e for point P; *len receives the run length.
-// `px`, `py`, `pz`: the view with rows along x, y, z (a view kept with x
-// rows only is passed for all three; its runs are all along x).
+// The masked bits of entry i (four rows) seen from D's point on `view`.
 template <bool FAST>
-__device__ inline unsigned long long run_bits(const unsigned long long* __restrict__ px,
-                                              const unsigned long long* __restrict__ py,
-                                              const unsigned long long* __restrict__ pz,
-                                              const MapView& M, RunEntry e, const Pt& P,
-                                              int* len, bool* outside) {
+__device__ __forceinline__ uint4 quad_bits(const MapView& M, const ToolView& T, const DirRows& D,
+                                           const uint4* __restrict__ view, int i, uint4* mask) {
+  if (!check_index((unsigned)i < (unsigned)T.nent, M.ctl)) {
+    *mask = make_uint4(0u, 0u, 0u, 0u);
+    return *mask;
+  }
+  const int2 e = __ldg(T.qent + i);  // (group offsets q1 | q2 << 16, d0 << 16 | 32 - window)
+  const uint4 m = __ldg(T.qmask + i);
+  *mask = m;
+  const int xa = D.a + (e.y >> 16), spare = e.y & 31;
+  const bool two = (xa & 31) > spare;  // the window reaches into the next word
+  const int q1 = (D.o1 >> 1) + (int)(short)(e.x & 0xffff), q2 = (D.o2 >> 1) + (e.x >> 16);
+  const int half = (D.axis == 0 ? M.dim_vox[1] : M.dim_vox[0]) >> 1;  // row groups along o1
+  const int rw = D.axis == 0 ? M.rw : (D.axis == 1 ? M.rw_y : M.rw_z);
+  const int w = xa >> 5;
+  uint4 lo = make_uint4(0u, 0u, 0u, 0u), hi = lo;
   if (FAST) {
-    const int d0 = (int)(short)(e.b & 0xffff), n = (e.b >> 16) & 0xFF, ax = (e.b >> 24) & 3;
-    const int xa = (ax == 0 ? P.px : (ax == 1 ? P.py : P.pz)) + d0;
-    const int row = (ax == 0 ? P.row : (ax == 1 ? P.rowy : P.rowz)) + e.a;
-    const unsigned long long* plane = ax == 0 ? px : (ax == 1 ? py : pz);
-    const int wa = xa >> 6, wb = (xa + n - 1) >> 6, sh = xa & 63;
-    const size_t words = ax == 0 ? M.words_x : (ax == 1 ? M.words_y : M.words_z);
-    if (!check_index(row + wa >= 0 && (size_t)(row + wb) < words, M.ctl)) {
-      *len = n;
-      return 0ull;
+    const int at = (q2 * half + q1) * rw + w;
+    const size_t quads = D.axis == 0 ? M.quads : (D.axis == 1 ? M.quads_y : M.quads_z);
+    if (!check_index(at >= 0 && (size_t)at + two < quads, M.ctl)) return lo;
+    lo = __ldg(view + at);
+    if (two) hi = __ldg(view + at + 1);
+  } else {
+    const int half2 = (D.axis == 2 ? M.dim_vox[1] : M.dim_vox[2]) >> 1;
+    if ((unsigned)q1 < (unsigned)half && (unsigned)q2 < (unsigned)half2) {
+      const uint4* row = view + ((size_t)q2 * half + q1) * rw;
+      if ((unsigned)w < (unsigned)rw) lo = __ldg(row + w);
+      if (two && (unsigned)(w + 1) < (unsigned)rw) hi = __ldg(row + w + 1);
     }
-    unsigned long long win = __ldg(plane + row + wa) >> sh;
-    if (wb != wa) win |= __ldg(plane + row + wb) << (64 - sh);
-    if (n < 64) win &= (1ull << n) - 1ull;
-    *len = n;
-    return win;
   }
-  const int d0 = (int)(short)(e.a & 0xffff), n = (int)(((uint32_t)e.a >> 16) & 0xFF),
-            ax = (int)(((uint32_t)e.a >> 24) & 3);
-  const int d1 = (int)(short)(e.b & 0xffff), d2 = (int)(short)((uint32_t)e.b >> 16);
-  *len = n;
-  // (a, o1, o2) coordinates of the run's first voxel
-  const int a0 = (ax == 0 ? P.px : (ax == 1 ? P.py : P.pz)) + d0;
-  const int o1 = (ax == 0 ? P.py : P.px) + d1;
-  const int o2 = (ax == 2 ? P.py : P.pz) + d2;
-  return row_bits(ax == 0 ? px : (ax == 1 ? py : pz), M, ax, a0, o1, o2, n, outside);
+  return make_uint4(__funnelshift_r(lo.x, hi.x, xa) & m.x, __funnelshift_r(lo.y, hi.y, xa) & m.y,
+                    __funnelshift_r(lo.z, hi.z, xa) & m.z, __funnelshift_r(lo.w, hi.w, xa) & m.w);
 }
 
-// Walks runs [r0, r1) of the tables a warp step (32 runs, one per lane) at a
-// time; the caller's `step(entry, valid)` returns true to stop the walk.
-template <bool FAST, bool SM, class F>
-__device__ inline void walk_runs(const ToolView& T, int r0, int r1, int lane, F&& step) {
-  for (int b = r0; b < r1; b += 32) {
-    const int r = b + lane;
-    const RunEntry e = r < r1 ? load_run<FAST, SM>(T, r) : RunEntry{0, 0};
-    if (step(e, r < r1)) return;
-  }
+__device__ __forceinline__ int popc4(uint4 b) {
+  return __popc(b.x) + __popc(b.y) + __popc(b.z) + __popc(b.w);
 }
 
+// Occupied tool voxels, saturated at `sat`, of up to four directions side by
+// side: the 8 lanes of group k (lanes 8k .. 8k + 7) count the direction of table
+// entry `d` (equal over the group; none unless `valid`), two entries per lane per step, and all get
+// its count. A group that has reached `sat` stops loading.
 template <bool FAST>
-__device__ inline bool bit_at(const unsigned long long* __restrict__ plane, const MapView& M,
-                              const Pt& P, short4 a) {
-  const int x = P.px + a.x, y = P.py + a.y, z = P.pz + a.z;
-  if (!FAST && ((unsigned)x >= (unsigned)M.dim_vox[0] || (unsigned)y >= (unsigned)M.dim_vox[1] ||
-                (unsigned)z >= (unsigned)M.dim_vox[2]))
-    return false;
-  const size_t w = FAST ? (size_t)(P.row + (a.z * M.dim_vox[1] + a.y) * M.row_words + (x >> 6))
-                        : ((size_t)z * M.dim_vox[1] + y) * M.row_words + (x >> 6);
-  if (!check_index(w < M.words_x, M.ctl)) return false;
-  return (__ldg(plane + w) >> (x & 63)) & 1ull;
+__device__ inline int tool_count4(const MapView& M, const ToolView& T, bool valid, int4 d, const Pt& P,
+                                  int sat, int lane) {
+  DirRows D = dir_rows(M, P, d);
+  if (!valid) D.nt = 0;
+  const int hl = lane & 7;
+  int total = 0;
+  bool more = D.nt > 0;
+  for (int b = hl; __any_sync(0xffffffffu, more); b += 16) {
+    int c = 0;
+    uint4 m;
+    if (more && b < D.nt) c = popc4(quad_bits<FAST>(M, T, D, D.view, D.t0 + b, &m));
+    if (more && b + 8 < D.nt) c += popc4(quad_bits<FAST>(M, T, D, D.view, D.t0 + b + 8, &m));
+    c += __shfl_xor_sync(0xffffffffu, c, 4);
+    c += __shfl_xor_sync(0xffffffffu, c, 2);
+    c += __shfl_xor_sync(0xffffffffu, c, 1);
+    total += c;
+    more = b - hl + 16 < D.nt && total < sat;
+  }
+  return min(total, sat);
 }
 
-// Occupied tool voxels of direction g at point P, saturated at `sat`.
-// SM: the direction table and the tool runs are staged in shared memory.
-template <bool FAST, bool SM = false>
+// Occupied tool voxels of direction g at point P, saturated at `sat`; the
+// whole warp on one direction.
+template <bool FAST>
 __device__ inline int tool_count(const MapView& M, const ToolView& T, int g, const Pt& P, int sat,
                                  int lane) {
-  const int4 dt = dtab_entry(T, g, SM);
+  const DirRows D = dir_rows(M, P, __ldg(T.dtab + g));
   int total = 0;
-  walk_runs<FAST, SM && FAST>(T, dt.x, dt.y, lane, [&](RunEntry e, bool valid) {
-    int c = 0;
-    if (valid) {
-      int len;
-      bool out = false;
-      c = __popcll(run_bits<FAST>(M.occ, M.occ_y, M.occ_z, M, e, P, &len, &out));
-    }
+  for (int b = 0; b < D.nt && total < sat; b += 32) {
+    uint4 m;
+    const int c = b + lane < D.nt ? popc4(quad_bits<FAST>(M, T, D, D.view, D.t0 + b + lane, &m)) : 0;
     total += __reduce_add_sync(0xffffffffu, c);
-    return total >= sat;
-  });
-  return total >= sat ? sat : total;
+  }
+  return min(total, sat);
 }
 
-// Occupied tool voxels of directions g1 and g2 at point P, each saturated at
-// `sat`, counted side by side: lanes 0-15 walk g1's runs and lanes 16-31
-// g2's, two runs per lane per step, so both counts take the round trips of
-// one. Each count is what tool_count returns for its direction: every run is
-// counted until the running sum reaches `sat`.
-template <bool FAST, bool SM>
-__device__ inline int2 tool_count2(const MapView& M, const ToolView& T, int g1, int g2,
-                                   const Pt& P, int sat, int lane) {
-  const int half = lane >> 4, hl = lane & 15;
-  const int4 dt = dtab_entry(T, half ? g2 : g1, SM);
-  const int len1 = __shfl_sync(0xffffffffu, dt.y - dt.x, 0);
-  const int len2 = __shfl_sync(0xffffffffu, dt.y - dt.x, 16);
-  int t1 = 0, t2 = 0;
-  for (int b = 0; (b < len1 && t1 < sat) || (b < len2 && t2 < sat); b += 32) {
-    const bool mine = half ? (t2 < sat) : (t1 < sat);
-    int c = 0;
+// Corridor of the direction of table entry d: any occupied voxel (strict: or
+// unknown) blocks. The whole warp, two entries per lane per step. Strict
+// corridors run along x, the known view's rows.
+template <bool FAST>
+__device__ inline bool corridor_blocked(const MapView& M, const ToolView& T, int4 d, const Pt& P,
+                                        int lane) {
+  const DirRows D = dir_rows(M, P, d, T.strict != 0);
+  for (int b = lane; b - lane < D.nc; b += 64) {
+    bool h = false;
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int r = dt.x + b + hl + 16 * j;
-      if (mine && r < dt.y) {
-        int len;
-        bool out = false;
-        c += __popcll(run_bits<FAST>(M.occ, M.occ_y, M.occ_z, M, load_run<FAST, SM>(T, r), P,
-                                     &len, &out));
+    for (int k = 0; k < 2; ++k) {
+      if (b + 32 * k >= D.nc) continue;
+      uint4 m;
+      const uint4 o = quad_bits<FAST>(M, T, D, D.view, D.c0 + b + 32 * k, &m);
+      h = h || (o.x | o.y | o.z | o.w) != 0u;
+      if (T.strict) {
+        const uint4 n = quad_bits<FAST>(M, T, D, M.known, D.c0 + b + 32 * k, &m);
+        h = h || ((n.x ^ m.x) | (n.y ^ m.y) | (n.z ^ m.z) | (n.w ^ m.w)) != 0u;
       }
     }
-    t1 += __reduce_add_sync(0xffffffffu, half ? 0 : c);
-    t2 += __reduce_add_sync(0xffffffffu, half ? c : 0);
+    if (__any_sync(0xffffffffu, h)) return true;
   }
-  return make_int2(t1 >= sat ? sat : t1, t2 >= sat ? sat : t2);
+  return false;
 }
 
 // The three arm samples of direction g (one lane): clear iff none is
-// occupied or unknown. All nine loads are issued together (no short
-// circuit), so the screen costs two dependent round trips, not up to nine.
-template <bool FAST, bool SM = false>
+// occupied or unknown. All loads are issued together (no short circuit), so
+// the screen costs two dependent round trips, not up to nine. The two views
+// share their layout, so one index serves both.
+template <bool FAST>
 __device__ inline bool arm_clear(const MapView& M, const ToolView& T, int g, const Pt& P) {
-  short4 a[3];
+  uint32_t clear = 1u;
 #pragma unroll
-  for (int s = 0; s < 3; ++s) a[s] = arm_entry(T, 3 * g + s, SM);
-  bool blocked = false;
-#pragma unroll
-  for (int s = 0; s < 3; ++s)
-    blocked = blocked | bit_at<FAST>(M.occ, M, P, a[s]) | !bit_at<FAST>(M.known, M, P, a[s]);
-  return !blocked;
-}
-
-// Corridor of direction g: any occupied voxel (strict: or unknown) blocks.
-template <bool FAST, bool SM = false>
-__device__ inline bool corridor_blocked(const MapView& M, const ToolView& T, int g, const Pt& P,
-                                        int lane) {
-  const int4 dt = dtab_entry(T, g, SM);
-  bool blocked = false;
-  walk_runs<FAST, false>(T, dt.z, dt.w, lane, [&](RunEntry e, bool valid) {
-    bool h = false;
-    if (valid) {
-      int len;
-      bool out = false;
-      h = run_bits<FAST>(M.occ, M.occ_y, M.occ_z, M, e, P, &len, &out) != 0ull;
-      if (T.strict && !h) {  // strict corridors run along x (the known view's rows)
-        const unsigned long long kb = run_bits<FAST>(M.known, M.known, M.known, M, e, P, &len, &out);
-        const unsigned long long full = len == 64 ? ~0ull : ((1ull << len) - 1ull);
-        h = out || (kb != full);
+  for (int s = 0; s < 3; ++s) {
+    const short4 a = __ldg(T.arm + 3 * g + s);
+    const int x = P.px + a.x, y = P.py + a.y, z = P.pz + a.z;
+    uint32_t oc = 0u, kn = 0u;
+    if (FAST || ((unsigned)x < (unsigned)M.dim_vox[0] && (unsigned)y < (unsigned)M.dim_vox[1] &&
+                 (unsigned)z < (unsigned)M.dim_vox[2])) {
+      const size_t at = FAST ? (size_t)(((z >> 1) * (M.dim_vox[1] >> 1) + (y >> 1)) * M.rw + (x >> 5))
+                             : ((size_t)(z >> 1) * (M.dim_vox[1] >> 1) + (y >> 1)) * M.rw + (x >> 5);
+      if (check_index(at < M.quads, M.ctl)) {
+        const size_t word = 4 * at + parity(y, z);
+        oc = __ldg(reinterpret_cast<const uint32_t*>(M.occ) + word);
+        kn = __ldg(reinterpret_cast<const uint32_t*>(M.known) + word);
       }
     }
-    blocked = __any_sync(0xffffffffu, h);
-    return blocked;
-  });
-  return blocked;
+    clear &= (kn & ~oc) >> (x & 31);
+  }
+  return clear & 1u;
 }
 
 __device__ inline bool candidate(const ToolView& T, int g, float n0, float n1, float n2) {
@@ -261,91 +218,79 @@ struct NormalFilter {
   __device__ bool operator()(const ToolView& T, int g) const { return candidate(T, g, n0, n1, n2); }
 };
 
-// The candidate loop of one point: lowest-index minimum of the direction
-// scores, with exact early exits; `cand(T, g)` says whether direction g is a
-// candidate of the point. Returns (best score, best index), (n_c + 2, -1)
-// without candidates.
-// SM: the direction table, the arm offsets and the tool runs are staged in
-// shared memory (af_staged_tab).
-// Once a search has a best (score <= n_c), it takes the remaining arm-clear
-// candidates two at a time (tool_count2, FAST path): a long search waits on
-// half as many tool-count round trips. Both counts are saturated at the score
-// to beat before the pair and the pair is then decided in index order, so the
-// result is the sequential one.
-template <bool FAST, class Cand, bool SM = false>
-__device__ inline int2 best_direction(const MapView& M, const ToolView& T, const Pt& P,
-                                      const Cand& cand_of, int lane) {
-  const int nc = T.n_c;
-  int bscore = nc + 2, best = -1;
-  for (int gb = 0; gb < T.G && bscore != 0; gb += 32) {
-    // lane-parallel screen: candidates, and the arm samples of each candidate
-    const bool cand = cand_of(T, gb + lane);
-    unsigned mask = __ballot_sync(0xffffffffu, cand);
-    const unsigned arm_ok = __ballot_sync(0xffffffffu, cand && arm_clear<FAST, SM>(M, T, gb + lane, P));
-    while (mask) {
-      const int bit = __ffs(mask) - 1;
-      const int g = gb + bit;
-      mask &= mask - 1u;
-      if (!((arm_ok >> bit) & 1u)) {
-        // blocked (n_c + 1): improves only the first candidate's empty best
-        if (best < 0) {
-          bscore = nc + 1;
-          best = g;
-        }
-        continue;
-      }
-      const unsigned rest = mask & arm_ok;  // arm-clear candidates after g in this group
-      if (FAST && bscore <= nc && rest) {
-        // g and the next arm-clear candidate g2; the candidates between them
-        // are arm-blocked (n_c + 1) and cannot beat the best there is
-        const int bit2 = __ffs(rest) - 1;
-        const int g2 = gb + bit2;
-        mask &= ~((2u << bit2) - 1u);
-        const int2 c = tool_count2<FAST, SM>(M, T, g, g2, P, bscore, lane);
-        if (c.x < bscore && !corridor_blocked<FAST, SM>(M, T, g, P, lane)) {
-          bscore = c.x;
-          best = g;
-          if (bscore == 0) break;
-        }
-        // c.y saturated at the score before g: at or above any score after it
-        if (c.y < bscore && !corridor_blocked<FAST, SM>(M, T, g2, P, lane)) {
-          bscore = c.y;
-          best = g2;
-        }
-        if (bscore == 0) break;
-        continue;
-      }
-      if (bscore <= nc) {
-        // improves only if not blocked and strictly fewer collisions
-        const int cnt = tool_count<FAST, SM>(M, T, g, P, bscore, lane);
-        if (cnt >= bscore) continue;
-        if (corridor_blocked<FAST, SM>(M, T, g, P, lane)) continue;
-        bscore = cnt;
-        best = g;
-      } else {
-        // nothing unblocked yet: any unblocked direction improves
-        if (corridor_blocked<FAST, SM>(M, T, g, P, lane)) {
-          if (best < 0) {
-            bscore = nc + 1;
-            best = g;
-          }
-          continue;
-        }
-        bscore = tool_count<FAST, SM>(M, T, g, P, nc, lane);
-        best = g;
-      }
-      if (bscore == 0) break;
-    }
+// The same with the masks of the first 1,024 directions kept, 32 per lane.
+struct KeptFilter {
+  NormalFilter F;
+  unsigned kept;  // lane k: the candidates among directions 32 k .. 32 k + 31
+  __device__ bool operator()(const ToolView& T, int g) const {
+    const int group = g >> 5;  // one group for the whole warp
+    if (group >= 32) return F(T, g);
+    return (__shfl_sync(0xffffffffu, kept, group) >> (g & 31)) & 1u;
   }
-  return make_int2(bscore, best);
+};
+
+struct NoGate {
+  __device__ bool operator()() const { return true; }
+};
+
+__device__ __forceinline__ int4 shfl4(int4 v, int from) {
+  return make_int4(__shfl_sync(0xffffffffu, v.x, from), __shfl_sync(0xffffffffu, v.y, from),
+                   __shfl_sync(0xffffffffu, v.z, from), __shfl_sync(0xffffffffu, v.w, from));
 }
 
+// The candidate loop of one point: lowest-index minimum of the direction
+// scores, with exact early exits; `cand(T, g)` says whether direction g is a
+// candidate of the point. Returns (best score, best index), (n_c + 1, first
+// candidate) if every candidate is blocked, (n_c + 2, -1) without candidates.
+// `gate()` is asked once, after the first screen (so that a load it waits for
+// overlaps the screen's): if it says no, (-1, -1) is returned.
+//
+// The arm screen takes 32 directions at a time. The arm-clear ones are then
+// counted four at a time, all against the score to beat before the four, and
+// decided in index order: a count that reaches that score cannot beat any later
+// one, so the result is the sequential one. A score of 0 ends the search.
+template <bool FAST, class Cand, class Gate = NoGate>
+__device__ inline int2 best_direction(const MapView& M, const ToolView& T, const Pt& P,
+                                      const Cand& cand_of, int lane, const Gate& gate = Gate()) {
+  const int nc = T.n_c;
+  int bscore = nc + 1, best = -1, first = -1;  // best: of the unblocked directions
+  for (int gb = 0; gb < T.G; gb += 32) {
+    // lane-parallel screen: candidates, and the arm samples of each candidate
+    const bool cand = cand_of(T, gb + lane);
+    const unsigned mask = __ballot_sync(0xffffffffu, cand);
+    if (first < 0 && mask) first = gb + __ffs(mask) - 1;
+    const int4 dt = cand ? __ldg(T.dtab + gb + lane) : make_int4(0, 0, 0, 0);
+    unsigned rest = __ballot_sync(0xffffffffu, cand && arm_clear<FAST>(M, T, gb + lane, P));
+    if (gb == 0 && !gate()) return make_int2(-1, -1);
+    while (rest) {
+      // the next four arm-clear directions, one per group of 8 lanes
+      const unsigned r1 = rest & (rest - 1u), r2 = r1 & (r1 - 1u), r3 = r2 & (r2 - 1u);
+      const unsigned mine = lane < 16 ? (lane < 8 ? rest : r1) : (lane < 24 ? r2 : r3);
+      const int at = mine ? __ffs(mine) - 1 : 0;
+      const int c = tool_count4<FAST>(M, T, mine != 0u, shfl4(dt, at), P, min(bscore, nc), lane);
+      unsigned todo = __ballot_sync(0xffffffffu, mine != 0u && (best < 0 || c < bscore)) & 0x01010101u;
+      rest = r3 & (r3 - 1u);
+      while (todo) {
+        const int from = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        const int k = __shfl_sync(0xffffffffu, at, from), ck = __shfl_sync(0xffffffffu, c, from);
+        if (best >= 0 && ck >= bscore) continue;  // beaten by one of the four before it
+        if (corridor_blocked<FAST>(M, T, shfl4(dt, k), P, lane)) continue;
+        bscore = ck;
+        best = gb + k;
+        if (bscore == 0) return make_int2(0, best);
+      }
+    }
+  }
+  if (best >= 0) return make_int2(bscore, best);
+  return first >= 0 ? make_int2(nc + 1, first) : make_int2(nc + 2, -1);
+}
 
 // best_direction with a budget: at most `budget` directions are taken past
 // the arm screen (tool count and corridor). If the search stops early,
 // *next receives the first direction index not searched and the result is
 // exact over the directions before it; *next = -1 when the search finished.
-template <bool FAST, class Cand, bool SM = false>
+template <bool FAST, class Cand>
 __device__ inline int2 best_direction_budget(const MapView& M, const ToolView& T, const Pt& P,
                                              const Cand& cand_of, int lane, int budget,
                                              int* next) {
@@ -355,7 +300,7 @@ __device__ inline int2 best_direction_budget(const MapView& M, const ToolView& T
   for (int gb = 0; gb < T.G && bscore != 0; gb += 32) {
     const bool cand = cand_of(T, gb + lane);
     unsigned mask = __ballot_sync(0xffffffffu, cand);
-    const unsigned arm_ok = __ballot_sync(0xffffffffu, cand && arm_clear<FAST, SM>(M, T, gb + lane, P));
+    const unsigned arm_ok = __ballot_sync(0xffffffffu, cand && arm_clear<FAST>(M, T, gb + lane, P));
     while (mask) {
       const int bit = __ffs(mask) - 1;
       const int g = gb + bit;
@@ -373,20 +318,20 @@ __device__ inline int2 best_direction_budget(const MapView& M, const ToolView& T
       }
       ++spent;
       if (bscore <= nc) {
-        const int cnt = tool_count<FAST, SM>(M, T, g, P, bscore, lane);
+        const int cnt = tool_count<FAST>(M, T, g, P, bscore, lane);
         if (cnt >= bscore) continue;
-        if (corridor_blocked<FAST, SM>(M, T, g, P, lane)) continue;
+        if (corridor_blocked<FAST>(M, T, __ldg(T.dtab + g), P, lane)) continue;
         bscore = cnt;
         best = g;
       } else {
-        if (corridor_blocked<FAST, SM>(M, T, g, P, lane)) {
+        if (corridor_blocked<FAST>(M, T, __ldg(T.dtab + g), P, lane)) {
           if (best < 0) {
             bscore = nc + 1;
             best = g;
           }
           continue;
         }
-        bscore = tool_count<FAST, SM>(M, T, g, P, nc, lane);
+        bscore = tool_count<FAST>(M, T, g, P, nc, lane);
         best = g;
       }
       if (bscore == 0) break;
