@@ -987,7 +987,7 @@ def run_soft(args, local):
     total = sum(ms)
     share = sum(v[1] for v in kt.values())
     dom = max(kt, key=lambda k: kt[k][1])
-    roof = {"kernel": dom, "kernel_ms": {k: round(v[1] / v[0], 4) for k, v in kt.items()},
+    roof = {"kernel": dom, "kernel_ms": {k: round(v[1] / 3, 4) for k, v in kt.items()},  # per step
             "kernel_share": {k: round(v[1] / share, 4) for k, v in kt.items()}}
     n_field = m * K
     out = {

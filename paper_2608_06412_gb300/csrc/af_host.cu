@@ -32,7 +32,9 @@ cudaError_t launch_score(const MapView& M, const ToolView& T, const float* d_pts
 cudaError_t launch_export_flags(const MapView& M, uint32_t count, uint8_t* d_flags,
                                 cudaStream_t stream);
 cudaError_t launch_views(const MapView& M, int num_sms, bool fill, bool all, uint32_t since,
-                         float* dense, float4* cells, uint32_t* list, cudaStream_t stream);
+                         float* dense, float4* cells, uint32_t* list, uint32_t* seen,
+                         cudaStream_t stream);
+size_t seen_words(const MapView& M);
 cudaError_t launch_soft_seed(const float* d_nrm, uint32_t m, const float* d_table, uint32_t K,
                              float* d_u0, int num_sms, cudaStream_t stream);
 cudaError_t launch_soft(const SoftView& S, bool grad, const float* pts, uint32_t per_point,
@@ -400,6 +402,7 @@ static void free_all(af_ctx* c) {
   cudaFree(c->d_dense);
   cudaFree(c->d_cells);
   cudaFree(c->d_vlist);
+  cudaFree(c->d_vseen);
   cudaFree(c->d_bgrid);
   cudaFree(c->d_skeys);
   cudaFree(c->d_nslots);
@@ -913,10 +916,12 @@ static af_status ensure_views(af_ctx* ctx, cudaStream_t s) {
         return fail(ctx, AF_ERR_CAPACITY, "soft clearance: the map box has too many cells for the dense SDF view");
       if (cudaMalloc(&ctx->d_dense, nd * sizeof(float)) != cudaSuccess ||
           cudaMalloc(&ctx->d_cells, nc * 2 * sizeof(float4)) != cudaSuccess ||
-          cudaMalloc(&ctx->d_vlist, ((size_t)M.pool_blocks + 1) * sizeof(uint32_t)) != cudaSuccess) {
+          cudaMalloc(&ctx->d_vlist, ((size_t)M.pool_blocks + 1) * sizeof(uint32_t)) != cudaSuccess ||
+          cudaMalloc(&ctx->d_vseen, af::seen_words(M) * sizeof(uint32_t)) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(ctx->d_dense);
         cudaFree(ctx->d_cells);
+        cudaFree(ctx->d_vlist);
         ctx->d_dense = nullptr;
         ctx->d_cells = nullptr;
         ctx->d_vlist = nullptr;
@@ -931,7 +936,7 @@ static af_status ensure_views(af_ctx* ctx, cudaStream_t s) {
       const bool all = fill || !ctx->views_valid || ctx->frame < ctx->views_frame;
       AF_CUDA(ctx, timed(ctx, 4, s, [&] {
         return af::launch_views(M, ctx->num_sms, fill, all, ctx->views_frame, ctx->d_dense,
-                                ctx->d_cells, ctx->d_vlist, s);
+                                ctx->d_cells, ctx->d_vlist, ctx->d_vseen, s);
       }));
       // a captured update has not run yet: the next call updates from where
       // the view is now
@@ -993,6 +998,9 @@ static void view_fields(const af_ctx* ctx, af::SoftView* S) {
   S->sparse = ctx->views_sparse ? 1 : 0;
   S->cells = ctx->views_sparse ? ctx->d_scells : ctx->d_cells;
   S->bgrid = ctx->d_bgrid;
+  S->seen = ctx->d_vseen;
+  S->nblock[0] = M.dim_vox[0] / 8 + 1;
+  S->nblock[1] = M.dim_vox[1] / 8 + 1;
   for (int k = 0; k < 3; ++k) {
     S->glo[k] = M.dom_vox[k] - 8;
     S->gdim[k] = M.dim_vox[k] / 8 + 1;
@@ -1043,6 +1051,8 @@ static af_status soft_view(af_ctx* ctx, float tau_s, af::SoftView* S) {
   S->ref = (float)-mx;
   S->sparse = 0;
   S->bgrid = nullptr;
+  S->seen = nullptr;
+  S->nblock[0] = S->nblock[1] = 0;
   return AF_OK;
 }
 
@@ -1151,7 +1161,7 @@ extern "C" af_status af_soft_refine(af_ctx* ctx, const float* d_pts, uint32_t pe
   AF_CUDA(ctx, timed(ctx, 7, s, [&] {
     return af::launch_soft_refine(S, A, d_pts, per_point, d_u0, d_alpha, d_beta, d_h, n, d_c,
                                   d_cmin, ctx->num_sms, s);
-  }));
+  }, 2));
   ctx->last_stream = s;
   return AF_OK;
 }
@@ -1163,6 +1173,7 @@ extern "C" af_status af_soft_set_view(af_ctx* ctx, int32_t mode) {
   cudaFree(ctx->d_dense);
   cudaFree(ctx->d_cells);
   cudaFree(ctx->d_vlist);
+  cudaFree(ctx->d_vseen);
   cudaFree(ctx->d_bgrid);
   cudaFree(ctx->d_skeys);
   cudaFree(ctx->d_nslots);
@@ -1170,6 +1181,7 @@ extern "C" af_status af_soft_set_view(af_ctx* ctx, int32_t mode) {
   ctx->d_dense = nullptr;
   ctx->d_cells = nullptr;
   ctx->d_vlist = nullptr;
+  ctx->d_vseen = nullptr;
   ctx->d_bgrid = nullptr;
   ctx->d_skeys = nullptr;
   ctx->d_nslots = nullptr;

@@ -255,6 +255,8 @@ struct SoftView {
                         // sparse: 512 cells (2 float4 each) per slot of bgrid
   int lo[3];            // absolute voxel index of the lowest cell's low corner
   int ncell[3];         // cells per axis: box voxels + 1
+  const uint32_t* seen; // dense: a bit per block of 8^3 cells, clear if every corner reads tau
+  int nblock[2];        // blocks along x and y
   int sparse;           // 1: the brick-sparse view
   const uint32_t* bgrid;  // sparse: per grid brick, the slot of its cells (kNoBlock: all tau)
   int glo[3];           // sparse: absolute voxel index of the grid's first brick corner

@@ -93,7 +93,9 @@ __global__ void __launch_bounds__(256) k_dense_view(MapView M, const uint32_t* _
 // from one voxel below the brick to its last voxel, 9^3 cells, from the 10^3
 // voxels around it. One CTA per brick, the voxels staged in shared memory, the
 // records written in runs of nine (288 bytes). Neighbouring bricks of the list
-// write the cells they share twice, with the same values. Bound by the record
+// write the cells they share twice, with the same values. A block of 8^3 cells
+// (cell indices with equal index >> 3) that reads anything but tau is marked in
+// `seen`; marks are never cleared (a voxel does not lose its weight). Bound by the record
 // writes: a scan of the pine stream changes about 900 bricks, 21 MB of records.
 // Rebuilding all 3.7 GB of that box instead took 1.21 ms after each scan; a
 // step of scan, scoring and refinement of its 12k points went from 1.56 ms to
@@ -103,15 +105,19 @@ constexpr int kCellEdge = kBrick + 1, kCornerEdge = kBrick + 2;
 __global__ void __launch_bounds__(256) k_cell_view(MapView M, const uint32_t* __restrict__ list,
                                                    const uint32_t* __restrict__ nlist,
                                                    const float* __restrict__ dense,
-                                                   float4* __restrict__ cells) {
+                                                   float4* __restrict__ cells,
+                                                   uint32_t* __restrict__ seen) {
   __shared__ float s_d[kCornerEdge * kCornerEdge * kCornerEdge];
+  __shared__ uint32_t s_seen;  // of the 8 blocks the brick's cells lie in
   const uint32_t count = __ldcg(nlist);
   const int X = M.dim_vox[0], Y = M.dim_vox[1], Z = M.dim_vox[2];
   for (uint32_t k = blockIdx.x; k < count; k += gridDim.x) {
     const uint64_t key = M.bkey[list[k]];
     const int bx = (int)(key & 0x1FFFFF) * 8, by = (int)((key >> 21) & 0x1FFFFF) * 8,
               bz = (int)(key >> 42) * 8;
-    __syncthreads();  // the previous brick's voxels are no longer read
+    __syncthreads();  // the previous brick's voxels and marks are no longer read
+    if (threadIdx.x == 0) s_seen = 0;
+    uint32_t mine = 0;
     for (int i = threadIdx.x; i < kCornerEdge * kCornerEdge * kCornerEdge; i += blockDim.x) {
       const int x = bx - 1 + i % kCornerEdge, y = by - 1 + (i / kCornerEdge) % kCornerEdge,
                 z = bz - 1 + i / (kCornerEdge * kCornerEdge);
@@ -128,6 +134,19 @@ __global__ void __launch_bounds__(256) k_cell_view(MapView M, const uint32_t* __
       constexpr int sy = kCornerEdge, sz = kCornerEdge * kCornerEdge;
       rec[0] = make_float4(c[0], c[1], c[sy], c[sy + 1]);
       rec[1] = make_float4(c[sz], c[sz + 1], c[sz + sy], c[sz + sy + 1]);
+      const float t = M.tau;
+      if (c[0] != t || c[1] != t || c[sy] != t || c[sy + 1] != t || c[sz] != t || c[sz + 1] != t ||
+          c[sz + sy] != t || c[sz + sy + 1] != t)
+        mine |= 1u << ((cx >> 3) | ((cy >> 3) << 1) | ((cz >> 3) << 2));
+    }
+    mine = __reduce_or_sync(0xffffffffu, mine);
+    if ((threadIdx.x & 31) == 0 && mine) atomicOr(&s_seen, mine);
+    __syncthreads();
+    if (threadIdx.x < 8 && ((s_seen >> threadIdx.x) & 1u)) {
+      const size_t b = ((size_t)((bz >> 3) + (threadIdx.x >> 2)) * (Y / 8 + 1) +
+                        (size_t)((by >> 3) + ((threadIdx.x >> 1) & 1))) * (X / 8 + 1) +
+                       (size_t)((bx >> 3) + (threadIdx.x & 1));
+      atomicOr(seen + (b >> 5), 1u << (b & 31));
     }
   }
 }
@@ -198,27 +217,16 @@ __device__ inline Dir make_dir(const SoftView& S, const float u0[3], const float
   return d;
 }
 
-// Cell of sample j: false when the cell lies outside the view (all corners
-// read tau). f receives the fractional position in the cell; *idx the record
-// index (dense view) or the cell's brick in the brick grid, *loc then its cell
-// within the brick (sparse view).
+// Position of the sample at t (standoff plus index, in voxels) in the point's
+// cell frame on axis i, in the order of operations the method states.
+__device__ inline float sample_pos(const PointCell& pc, const Dir& d, float t, int i) {
+  return __fadd_rn(pc.r[i], __fmul_rn(t, d.u[i]));
+}
+
+// Where a record is: its index (dense view), or its cell's brick in the brick
+// grid and its cell within the brick (sparse view).
 template <bool SPARSE>
-__device__ inline bool sample_cell(const SoftView& S, const PointCell& pc, const Dir& d, int j,
-                                   float f[3], uint32_t* idx, uint32_t* loc) {
-  const float t = __fadd_rn(d.e, (float)j);
-  int c[3];
-  bool in = pc.ok;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const float l = __fadd_rn(pc.r[i], __fmul_rn(t, d.u[i]));
-    const float fl = floorf(l);
-    f[i] = l - fl;  // exact
-    const bool ok = fabsf(l) < 1.0e7f;
-    const int base = SPARSE ? S.glo[i] : S.lo[i];
-    const int lim = SPARSE ? 8 * S.gdim[i] : S.ncell[i];
-    c[i] = ok ? (int)pc.I[i] + (int)fl - base : -1;
-    in = in && ok && (unsigned)c[i] < (unsigned)lim;
-  }
+__device__ inline void record_of(const SoftView& S, const int c[3], uint32_t* idx, uint32_t* loc) {
   if (SPARSE) {
     *idx = ((uint32_t)(c[2] >> 3) * (uint32_t)S.gdim[1] + (uint32_t)(c[1] >> 3)) *
                (uint32_t)S.gdim[0] + (uint32_t)(c[0] >> 3);
@@ -228,6 +236,65 @@ __device__ inline bool sample_cell(const SoftView& S, const PointCell& pc, const
            (uint32_t)c[0];
     *loc = 0;
   }
+}
+
+// Cell of the sample at t: false when the cell lies outside the view (all
+// corners read tau). f receives the fractional position in the cell.
+template <bool SPARSE>
+__device__ inline bool sample_cell(const SoftView& S, const PointCell& pc, const Dir& d, float t,
+                                   float f[3], int c[3]) {
+  bool in = pc.ok;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const float l = sample_pos(pc, d, t, i);
+    const float fl = floorf(l);
+    f[i] = l - fl;  // exact
+    const bool ok = fabsf(l) < 1.0e7f;
+    const int base = SPARSE ? S.glo[i] : S.lo[i];
+    const int lim = SPARSE ? 8 * S.gdim[i] : S.ncell[i];
+    c[i] = ok ? (int)pc.I[i] + (int)fl - base : -1;
+    in = in && ok && (unsigned)c[i] < (unsigned)lim;
+  }
+  return in;
+}
+
+// The same for a pair whose samples all lie inside the view and within 2^22
+// voxels of its point (samples_inside): no check is left, and the floor comes
+// from adding 1.5 2^23, which rounds to an integer kept in the low bits -- four
+// single-precision operations at full rate in the place of a rounding and a
+// conversion at a quarter of it. `cb` is the point's cell less the view's base
+// and that constant's bits. Same cell and same f.
+constexpr float kRound = 12582912.0f;        // 1.5 2^23
+constexpr int kRoundBits = 0x4B400000;
+__device__ inline void sample_cell_inside(const PointCell& pc, const Dir& d, const int cb[3], float t,
+                                          float f[3], int c[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const float l = sample_pos(pc, d, t, i);
+    const float y0 = __fadd_rn(l, kRound), y = __fsub_rn(y0, kRound);
+    const bool up = y > l;  // rounded up: the floor is one below
+    f[i] = l - (up ? y - 1.0f : y);
+    c[i] = __float_as_int(y0) + cb[i] - (up ? 1 : 0);
+  }
+}
+
+// Whether every sample j0..J lies inside the view, and the constants of
+// sample_cell_inside. Rounding is monotone, so on each axis the samples' cells
+// lie between those of the first and the last sample.
+template <bool SPARSE>
+__device__ inline bool samples_inside(const SoftView& S, const PointCell& pc, const Dir& d, int cb[3]) {
+  bool in = true;
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const float t = __fadd_rn(d.e, (float)(e ? S.J : S.j0));
+    float f[3];
+    int c[3];
+    in = in && sample_cell<SPARSE>(S, pc, d, t, f, c);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) in = in && fabsf(sample_pos(pc, d, t, i)) < 4.0e6f;
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) cb[i] = (int)pc.I[i] - (SPARSE ? S.glo[i] : S.lo[i]) - kRoundBits;
   return in;
 }
 
@@ -373,54 +440,101 @@ __device__ inline float trilinear(const float4& lo, const float4& hi, const floa
 
 // Records in flight per lane (NF): the lane computes NF sample cells, issues
 // their loads, then folds them into the softmin in sample order, so the
-// result does not depend on NF. The field takes 3, the refinement 4
-// (measured best; more in flight trade registers for memory parallelism).
-constexpr int kInFlightField = 3;
-constexpr int kInFlightRefine = 4;
+// result does not depend on NF. More in flight trade registers for memory
+// parallelism: the field of 1.9M pairs takes 487 us with 2, 495 with 3, 545 with
+// 4; the refinement of 30k pairs 236 us with 3, 271 with 4 (spills), 263 with 2.
+constexpr int kInFlightField = 2;
+constexpr int kInFlightRefine = 3;
+
+// Folds lane g's samples j0 + g, j0 + g + kLanes, ... into sm. INSIDE: every
+// sample lies inside the view (samples_inside).
+//
+// Most samples of a 1.25 m axis read nothing but tau (78% of those of a finished
+// pine map), so the dense view's records are only read in blocks of cells that
+// hold anything else: one bit per 8^3 cells, 29 KB for the pine box, which stays
+// in L1. The records then read are a 27 MB part of the 3.7 GB view and stay in L2.
+// With the checks of the cells gone as well, the field of a finished map's 30k
+// points (1.9M pairs) went from 862 to 487 us, forward plus adjoint of 113k pairs
+// from 149 to 72 us, the refinement of 30k pairs from 315 to 236 us.
+template <bool INSIDE, bool GRAD, bool FIXED, bool SPARSE, int NF>
+__device__ inline void fold_samples(Softmin<GRAD, FIXED>& sm, const SoftView& S, const PointCell& pc,
+                                    const Dir& d, const int cb[3], int g) {
+#pragma unroll 1
+  for (int j = S.j0 + g; j <= S.J; j += NF * kLanes) {
+    float f[NF][3];
+    uint32_t id[NF], loc[NF];
+    size_t rec[NF];
+    bool has[NF], in[NF];
+    uint32_t mark[NF], bit[NF];
+#pragma unroll
+    for (int q = 0; q < NF; ++q) {
+      has[q] = j + q * kLanes <= S.J;
+      const float t = __fadd_rn(d.e, (float)(j + q * kLanes));
+      int c[3];
+      if (INSIDE) {
+        sample_cell_inside(pc, d, cb, t, f[q], c);
+        in[q] = has[q];
+      } else {
+        in[q] = has[q] && sample_cell<SPARSE>(S, pc, d, t, f[q], c);
+      }
+      record_of<SPARSE>(S, c, &id[q], &loc[q]);
+      rec[q] = id[q];
+      if (!SPARSE) {
+        const uint32_t b = ((uint32_t)(c[2] >> 3) * (uint32_t)S.nblock[1] + (uint32_t)(c[1] >> 3)) *
+                               (uint32_t)S.nblock[0] + (uint32_t)(c[0] >> 3);
+        mark[q] = in[q] ? __ldg(S.seen + (b >> 5)) : 0u;
+        bit[q] = b;
+      }
+    }
+    if (SPARSE) {  // the slots of the cells' bricks first, then the records
+      uint32_t slot[NF];
+#pragma unroll
+      for (int q = 0; q < NF; ++q) slot[q] = in[q] ? __ldg(S.bgrid + id[q]) : kNoBlock;
+#pragma unroll
+      for (int q = 0; q < NF; ++q) {
+        in[q] = in[q] && slot[q] != kNoBlock;
+        rec[q] = (size_t)slot[q] * kBrickVox + loc[q];
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < NF; ++q) in[q] = (mark[q] >> (bit[q] & 31u)) & 1u;
+    }
+    float4 lo[NF], hi[NF];
+#pragma unroll
+    for (int q = 0; q < NF; ++q)
+      if (in[q]) load_cell(S, rec[q], lo[q], hi[q]);
+#pragma unroll
+    for (int q = 0; q < NF; ++q) {
+      if (!has[q]) break;
+      const int jq = j + q * kLanes;
+      float G[3] = {0.f, 0.f, 0.f};
+      const float D = in[q] ? trilinear<GRAD>(lo[q], hi[q], f[q], G) : S.tau;
+      sm.add(D - (jq <= S.jt ? S.r : S.r_corr), d.e + (float)jq, G, S);
+    }
+  }
+}
+
+// How a kernel takes its samples: every pair whose samples lie inside the view
+// without checks and the others with them (kBoth), the others not at all
+// (kInside: *outside is set instead), every pair with checks (kChecked).
+enum Road { kBoth, kInside, kChecked };
 
 // C of one pair and, with GRAD, dC / d(alpha, beta, h); *cmin = min_j phi_j.
 // Called by all kLanes lanes of the pair's group (lane g of it); with
 // `live` false the lane samples nothing.
-template <bool GRAD, bool FIXED, bool SPARSE, int NF>
+template <bool GRAD, bool FIXED, bool SPARSE, int NF, Road ROAD>
 __device__ inline float soft_eval(const SoftView& S, const PointCell& pc, const Dir& d,
                                   const float t1[3], const float t2[3], bool live, int g,
-                                  float* ga, float* gb, float* gh, float* cmin) {
+                                  float* ga, float* gb, float* gh, float* cmin, bool* outside) {
   Softmin<GRAD, FIXED> sm;
   if (live) {
-    for (int j = S.j0 + g; j <= S.J; j += NF * kLanes) {
-      float f[NF][3];
-      uint32_t id[NF], loc[NF];
-      size_t rec[NF];
-      bool has[NF], in[NF];
-#pragma unroll
-      for (int q = 0; q < NF; ++q) {
-        has[q] = j + q * kLanes <= S.J;
-        in[q] = has[q] && sample_cell<SPARSE>(S, pc, d, j + q * kLanes, f[q], &id[q], &loc[q]);
-        rec[q] = id[q];
-      }
-      if (SPARSE) {  // the slots of the cells' bricks first, then the records
-        uint32_t slot[NF];
-#pragma unroll
-        for (int q = 0; q < NF; ++q) slot[q] = in[q] ? __ldg(S.bgrid + id[q]) : kNoBlock;
-#pragma unroll
-        for (int q = 0; q < NF; ++q) {
-          in[q] = in[q] && slot[q] != kNoBlock;
-          rec[q] = (size_t)slot[q] * kBrickVox + loc[q];
-        }
-      }
-      float4 lo[NF], hi[NF];
-#pragma unroll
-      for (int q = 0; q < NF; ++q)
-        if (in[q]) load_cell(S, rec[q], lo[q], hi[q]);
-#pragma unroll
-      for (int q = 0; q < NF; ++q) {
-        if (!has[q]) break;
-        const int jq = j + q * kLanes;
-        float G[3] = {0.f, 0.f, 0.f};
-        const float D = in[q] ? trilinear<GRAD>(lo[q], hi[q], f[q], G) : S.tau;
-        sm.add(D - (jq <= S.jt ? S.r : S.r_corr), d.e + (float)jq, G, S);
-      }
-    }
+    int cb[3] = {0, 0, 0};
+    if (ROAD != kChecked && samples_inside<SPARSE>(S, pc, d, cb))
+      fold_samples<true, GRAD, FIXED, SPARSE, NF>(sm, S, pc, d, cb, g);
+    else if (ROAD == kInside)
+      *outside = true;
+    else
+      fold_samples<false, GRAD, FIXED, SPARSE, ROAD == kChecked ? NF : 1>(sm, S, pc, d, cb, g);
   }
   sm.reduce(S.k2);
   const float C = (FIXED ? S.ref : sm.m) - S.ln2_tau_s * lg2(sm.Z);
@@ -505,8 +619,8 @@ __global__ void __launch_bounds__(128) k_soft(SoftView S, const float* __restric
     const Dir d = make_dir(S, u, t1, t2, __ldg(alpha + i), __ldg(beta + i), __ldg(hh + i));
     const bool fin = pc.finite && d.finite;
     float da, db, dh, mn;
-    float C = soft_eval<GRAD, FIXED, SPARSE, kInFlightField>(S, pc, d, t1, t2, fin && act, w.g,
-                                                             &da, &db, &dh, &mn);
+    float C = soft_eval<GRAD, FIXED, SPARSE, kInFlightField, kBoth>(S, pc, d, t1, t2, fin && act, w.g,
+                                                                    &da, &db, &dh, &mn, nullptr);
     if (!act || w.g != 0) continue;
     if (!fin) C = mn = da = db = dh = NAN;
     if (c) c[i] = C;
@@ -520,10 +634,60 @@ __global__ void __launch_bounds__(128) k_soft(SoftView S, const float* __restric
   }
 }
 
-// `steps` ascent steps on C per pair in registers, then C at the final state.
-// The group's lanes update identical copies of (alpha, beta, h).
-template <bool FIXED, bool SPARSE>
-__global__ void __launch_bounds__(128) k_soft_refine(SoftView S, RefineArgs R,
+// `steps` ascent steps on C of pair i in registers, then C at the final state;
+// the group's lanes (`act`: the pair is taken) update identical copies of
+// (alpha, beta, h). False, with nothing written, if a step takes a sample out of
+// the view (ROAD == kInside).
+template <bool FIXED, bool SPARSE, int NF, Road ROAD>
+__device__ inline bool refine_pair(const SoftView& S, const RefineArgs& R, const float* __restrict__ pts,
+                                   uint32_t per_point, const float* __restrict__ u0,
+                                   float* __restrict__ alpha, float* __restrict__ beta,
+                                   float* __restrict__ hh, float* __restrict__ c,
+                                   float* __restrict__ cmin, size_t i, bool act, int g) {
+  float s[3], u[3], t1[3], t2[3];
+  load3(pts, i / per_point, s);
+  load3(u0, i, u);
+  onb(u, t1, t2);
+  const PointCell pc = point_cell(S, s);
+  float al = alpha[i], be = beta[i], h = hh[i];
+  // a pair that is not finite (e.g. a point with no start) samples nothing
+  const bool fin = pc.finite && make_dir(S, u, t1, t2, al, be, h).finite;
+  bool outside = false;
+#pragma unroll 1
+  for (int k = 0; k < R.steps; ++k) {
+    const Dir d = make_dir(S, u, t1, t2, al, be, h);
+    const bool live = fin && act && d.finite && !outside;
+    float da, db, dh, mn;
+    soft_eval<true, FIXED, SPARSE, NF, ROAD>(S, pc, d, t1, t2, live, g, &da, &db, &dh, &mn, &outside);
+    if (live) {
+      al = __fmaf_rn(R.lr_dir, da, al);
+      be = __fmaf_rn(R.lr_dir, db, be);
+      h = fminf(fmaxf(__fmaf_rn(R.lr_h, dh, h), 0.0f), R.h_max);
+    }
+  }
+  const Dir d = make_dir(S, u, t1, t2, al, be, h);
+  const bool ok = fin && d.finite;
+  float mn;
+  float C = soft_eval<false, FIXED, SPARSE, NF, ROAD>(S, pc, d, t1, t2, ok && act && !outside, g, nullptr,
+                                                      nullptr, nullptr, &mn, &outside);
+  if (!act || outside || g != 0) return !outside;
+  if (!ok) C = mn = al = be = h = NAN;
+  alpha[i] = al;
+  beta[i] = be;
+  hh[i] = h;
+  c[i] = C;
+  if (cmin) cmin[i] = mn;
+  return true;
+}
+
+// Two launches: the checks of the samples' cells would cost every pair 70
+// registers, so the first (ROAD kInside) leaves a pair that a step takes out of
+// the view as it was and marks its C with a NaN of its own, and the second takes
+// the marked pairs from their start again, with the checks.
+constexpr unsigned kRedo = 0x7FC05EDDu;
+
+template <bool FIXED, bool SPARSE, Road ROAD>
+__global__ void __launch_bounds__(128, 4) k_soft_refine(SoftView S, RefineArgs R,
                                                      const float* __restrict__ pts,
                                                      uint32_t per_point,
                                                      const float* __restrict__ u0,
@@ -535,40 +699,15 @@ __global__ void __launch_bounds__(128) k_soft_refine(SoftView S, RefineArgs R,
   const GroupWalk w;
   for (size_t base = w.first; base < n; base += w.stride) {
     const size_t i0 = base + w.slot;
-    const bool act = i0 < n;
+    bool act = i0 < n;
     const size_t i = act ? i0 : n - 1;
-    float s[3], u[3], t1[3], t2[3];
-    load3(pts, i / per_point, s);
-    load3(u0, i, u);
-    onb(u, t1, t2);
-    const PointCell pc = point_cell(S, s);
-    float al = alpha[i], be = beta[i], h = hh[i];
-    // a pair that is not finite (e.g. a point with no start) samples nothing
-    const bool fin = pc.finite && make_dir(S, u, t1, t2, al, be, h).finite;
-    for (int k = 0; k < R.steps; ++k) {
-      const Dir d = make_dir(S, u, t1, t2, al, be, h);
-      const bool live = fin && act && d.finite;
-      float da, db, dh, mn;
-      soft_eval<true, FIXED, SPARSE, kInFlightRefine>(S, pc, d, t1, t2, live, w.g, &da, &db, &dh,
-                                                      &mn);
-      if (live) {
-        al = __fmaf_rn(R.lr_dir, da, al);
-        be = __fmaf_rn(R.lr_dir, db, be);
-        h = fminf(fmaxf(__fmaf_rn(R.lr_h, dh, h), 0.0f), R.h_max);
-      }
+    if (ROAD == kChecked) {
+      act = act && __float_as_uint(c[i]) == kRedo;
+      if (!__any_sync(kFull, act)) continue;
     }
-    const Dir d = make_dir(S, u, t1, t2, al, be, h);
-    const bool ok = fin && d.finite;
-    float mn;
-    float C = soft_eval<false, FIXED, SPARSE, kInFlightRefine>(S, pc, d, t1, t2, ok && act, w.g,
-                                                                nullptr, nullptr, nullptr, &mn);
-    if (!act || w.g != 0) continue;
-    if (!ok) C = mn = al = be = h = NAN;
-    alpha[i] = al;
-    beta[i] = be;
-    hh[i] = h;
-    c[i] = C;
-    if (cmin) cmin[i] = mn;
+    if (!refine_pair<FIXED, SPARSE, ROAD == kChecked ? 1 : kInFlightRefine, ROAD>(
+            S, R, pts, per_point, u0, alpha, beta, hh, c, cmin, i, act, w.g) && act && w.g == 0)
+      c[i] = __uint_as_float(kRedo);
   }
 }
 
@@ -718,24 +857,33 @@ cudaError_t launch_sview_fill(const MapView& M, int num_sms, const uint32_t* key
   return cudaGetLastError();
 }
 
+// Words of the dense view's block marks.
+size_t seen_words(const MapView& M) {
+  const size_t n = ((size_t)M.dim_vox[0] / 8 + 1) * (M.dim_vox[1] / 8 + 1) * (M.dim_vox[2] / 8 + 1);
+  return (n + 31) / 32;
+}
+
 // Brings the dense view up to date with the map: the bricks changed after scan
 // `since`, or every brick (`all`); with `fill` the buffers are new and every
 // value starts as tau.
 cudaError_t launch_views(const MapView& M, int num_sms, bool fill, bool all, uint32_t since,
-                         float* dense, float4* cells, uint32_t* list, cudaStream_t stream) {
+                         float* dense, float4* cells, uint32_t* list, uint32_t* seen,
+                         cudaStream_t stream) {
   const size_t nd = (size_t)M.dim_vox[0] * M.dim_vox[1] * M.dim_vox[2];  // a multiple of 512
   const size_t nc = ((size_t)M.dim_vox[0] + 1) * (M.dim_vox[1] + 1) * (M.dim_vox[2] + 1);
   if (fill) {
     k_fill<<<grid_for(nd / 4, 256, num_sms, 8), 256, 0, stream>>>(reinterpret_cast<float4*>(dense),
                                                                    nd / 4, M.tau);
     k_fill<<<grid_for(nc * 2, 256, num_sms, 8), 256, 0, stream>>>(cells, nc * 2, M.tau);
+    const cudaError_t z = cudaMemsetAsync(seen, 0, seen_words(M) * sizeof(uint32_t), stream);
+    if (z != cudaSuccess) return z;
   }
   uint32_t* nlist = list + M.pool_blocks;
   cudaError_t e = cudaMemsetAsync(nlist, 0, sizeof(uint32_t), stream);
   if (e != cudaSuccess) return e;
   k_view_list<<<grid_for(M.pool_blocks, 256, num_sms, 8), 256, 0, stream>>>(M, since, all ? 1 : 0, list, nlist);
   k_dense_view<<<(unsigned)num_sms * 8, 256, 0, stream>>>(M, list, nlist, dense);
-  k_cell_view<<<(unsigned)num_sms * 8, 256, 0, stream>>>(M, list, nlist, dense, cells);
+  k_cell_view<<<(unsigned)num_sms * 8, 256, 0, stream>>>(M, list, nlist, dense, cells, seen);
   return cudaGetLastError();
 }
 
@@ -776,8 +924,9 @@ cudaError_t launch_soft_refine(const SoftView& S, const RefineArgs& R, const flo
                                cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
   const unsigned g = grid_for(n * kLanes, 128, num_sms, 16);
-#define AF_REFINE_LAUNCH(FX, SP) \
-  k_soft_refine<FX, SP><<<g, 128, 0, stream>>>(S, R, pts, per_point, u0, al, be, h, n, c, cmin)
+#define AF_REFINE_LAUNCH(FX, SP)                                                                            \
+  (k_soft_refine<FX, SP, kInside><<<g, 128, 0, stream>>>(S, R, pts, per_point, u0, al, be, h, n, c, cmin), \
+   k_soft_refine<FX, SP, kChecked><<<g, 128, 0, stream>>>(S, R, pts, per_point, u0, al, be, h, n, c, cmin))
   if (S.fixed && S.sparse)
     AF_REFINE_LAUNCH(true, true);
   else if (S.fixed)

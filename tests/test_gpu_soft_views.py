@@ -71,6 +71,15 @@ def test_updated_view_equals_whole(tight, how):
         got = kept.soft_clearance_raw(*pairs[:2], *pairs[2:], 1)
         want = whole.soft_clearance_raw(*pairs[:2], *pairs[2:], 1)
         assert torch.equal(got, want)
+        # refinement of pairs in and out of the view: C and the hard clearance at
+        # the state it reports, whether a step takes the pair out or not
+        for steps in (0, 3):
+            a, b, h = (t.clone() for t in pairs[2:])
+            c, cmin = kept.soft_refine(*pairs[:2], a, b, h, 1, steps=steps)
+            hard = torch.empty_like(c)
+            assert torch.equal(c, whole.soft_clearance_raw(*pairs[:2], a, b, h, 1, cmin=hard))
+            assert torch.equal(cmin, hard)
+            assert steps == 0 or not torch.equal(a, pairs[2])
         whole_batch.close()
         whole.close()
     far = got.max().item()
