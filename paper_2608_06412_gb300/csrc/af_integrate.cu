@@ -27,6 +27,7 @@
 // cheaper approximate value is used, it only takes decisions that the exact
 // value is certain to agree with (margins of 2^-16).
 
+#include "af_cube.cuh"
 #include "af_internal.cuh"
 
 namespace af {
@@ -180,31 +181,6 @@ __global__ void __launch_bounds__(256) k_alloc(MapView M, const float* __restric
   alloc_slot<false>(M, xyz, n, P, ret, frame, blockIdx.x * blockDim.x + threadIdx.x, 0u);
 }
 
-// Approximate square root (MUFU reciprocal square root), relative error well
-// below 2^-20 for the normal arguments it is used on. Only ever used to take
-// a decision that the exact result is certain to agree with (margins of
-// 2^-16 relative); near any threshold the exact IEEE operation decides.
-__device__ inline float sqrt_approx(float x) { return x * rsqrtf(x); }
-
-constexpr float kMargin = 1.52587890625e-05f;  // 2^-16
-
-// The exact cone decision, RN(dot / RN(RN(sqrt(aa)) range)) > cone, out of
-// line: it runs only within 2^-16 of the threshold, so divergent lanes call it
-// instead of every lane carrying its instructions.
-__device__ __noinline__ bool cone_excludes_exact(float dot, float aa, float range, float cone) {
-  return __fdiv_rn(dot, __fmul_rn(__fsqrt_rn(aa), range)) > cone;
-}
-
-template <int W>
-struct CubeShape {
-  static constexpr int C = W * W * W;                                 // offsets
-  static constexpr int NT = ((C + 31) / 32) * 32 <= 1024 ? ((C + 31) / 32) * 32 : 1024;
-  static constexpr int OPT = (C + NT - 1) / NT;                       // offsets per thread
-  static constexpr int BA = (W + 6) / 8 + 1;                          // bricks per edge
-  static constexpr int NB = BA * BA * BA;
-  static constexpr int MR = W / 2;
-};
-
 // A tile of one scan: returns [r0, r1), r1 - r0 <= T; called by the whole
 // CTA of CubeShape<W>::NT threads. W = 2m + 1 voxels per cube edge.
 template <int W, int T>
@@ -236,19 +212,11 @@ __device__ void integrate_tile(const MapView& M, const float4* __restrict__ ret,
   if (tid < T) {
     const uint32_t k = r0 + tid;
     float4 p = k < r1 ? ret[k] : make_float4(0.f, 0.f, 0.f, 0.f);
-    float bb = 0.f, range = 0.f, ir = 0.f;
-    if (p.w != 0.f) {
-      const float b[3] = {__fsub_rn(p.x, q0), __fsub_rn(p.y, q1), __fsub_rn(p.z, q2)};
-      bb = __fadd_rn(__fadd_rn(__fmul_rn(b[0], b[0]), __fmul_rn(b[1], b[1])), __fmul_rn(b[2], b[2]));
-      range = __fsqrt_rn(bb);
-      ir = __frcp_rn(range);
-    }
     s_p[tid] = p;
-    s_pr[tid] = make_float4(range, bb, ir, p.w);
+    s_pr[tid] = return_record(p, q0, q1, q2);
   }
   // Per-axis terms of every (return, axis, offset), each thread from the
   // return itself (no barrier between the per-return and per-axis steps).
-  const float v = M.v, tau = M.tau, cone = M.cone_cos;
   for (int e = tid; e < T * 3 * W; e += NT) {
     const int t = e / (3 * W), ax = (e / W) % 3, k = e % W;
     if (r0 + t >= r1) continue;
@@ -259,14 +227,13 @@ __device__ void integrate_tile(const MapView& M, const float4* __restrict__ ret,
     voxel_index(pa, M, &i);
     const int rel = i - M.dom_vox[ax];                 // box-relative voxel of p on this axis
     const int j = rel + k - MR;                        // ... of the cube voxel
-    const float x = voxel_centre(j + M.dom_vox[ax], v);
-    const float a = __fsub_rn(x, pa), b = __fsub_rn(pa, q[ax]), c = __fsub_rn(x, q[ax]);
+    float4 term = axis_terms(M, pa, q[ax], j + M.dom_vox[ax]);
     // brick offset within the tile's brick table (weight 1, BA, BA^2) in the
     // high half, the voxel's slot bits within its brick in the low half
     const int bk = (j >> 3) - ((rel - MR) >> 3);
     const int code = ((bk * (ax == 0 ? 1 : (ax == 1 ? BA : BA * BA))) << 16) | ((j & 7) << (3 * ax));
-    s_term[t][ax][k] = make_float4(__fmul_rn(a, a), __fmul_rn(a, b), __fmul_rn(c, c),
-                                   __int_as_float(code));
+    term.w = __int_as_float(code);
+    s_term[t][ax][k] = term;
   }
   // The tile's brick tables; bricks created by this scan are looked up now.
   for (int e = tid; e < T * NB; e += NT) {
@@ -309,43 +276,12 @@ __device__ void integrate_tile(const MapView& M, const float4* __restrict__ ret,
   for (int t = 0; t < T; ++t) {
     const float4 pr = s_pr[t];
     if (pr.w == 0.f) continue;  // uniform across the block
-    const float range = pr.x, bb = pr.y, ir = pr.z;
 #pragma unroll
     for (int s = 0; s < OPT; ++s) {
       if (tid + s * NT >= C) break;
       const float4 tx = s_term[t][0][kx[s]], ty = s_term[t][1][ky[s]], tz = s_term[t][2][kz[s]];
-      const float aa = __fadd_rn(__fadd_rn(tx.x, ty.x), tz.x);
-      // behind-surface cone: theta between x - p and p - q; excluded iff
-      // RN(dot / RN(RN(sqrt(aa)) * range)) > cone
-      if (aa > 0.f) {
-        const float dot = __fadd_rn(__fadd_rn(tx.y, ty.y), tz.y);
-        // dot <= 0 makes the rounded cosine <= 0, so with cone >= 0 it is kept
-        if (dot > 0.f || cone < 0.f) {
-          bool decided = false;
-          if (aa > 1e-20f) {
-            // a few ulp from the exact cosine (rsqrtf, two products, RN(1 / range))
-            const float ca = dot * rsqrtf(aa) * ir;
-            if (ca > cone + kMargin) continue;  // certainly excluded
-            decided = ca < cone - kMargin;      // certainly kept
-          }
-          if (!decided && cone_excludes_exact(dot, aa, range, cone)) continue;
-        }
-      }
-      // d = |p - q| - |x - q|, clamped to [0, tau] ([-tau, tau] in the ablation)
-      const float cc = __fadd_rn(__fadd_rn(tx.z, ty.z), tz.z);
-      float d;
-      if (cc >= bb && !M.clamp_signed) {
-        d = 0.f;  // |x - q| >= |p - q|: the rounded difference is <= 0
-      } else if (cc > 1e-20f && range - sqrt_approx(cc) > tau + range * kMargin) {
-        d = tau;  // the exact difference exceeds tau
-      } else {
-        d = __fsub_rn(range, __fsqrt_rn(cc));
-        d = d < M.dlo ? M.dlo : d;
-        d = d > tau ? tau : d;
-      }
-      // |d| <= tau <= 1 m, so |d 2^20| < 2^31: the 32-bit conversion rounds
-      // exactly as a 64-bit one would, and stays off the FP64 pipe
-      const long long dq = (long long)__float2int_rn(__fmul_rn(d, kScale));
+      long long dq;
+      if (!pair_contribution(M, tx, ty, tz, pr, &dq)) continue;
       const int code = __float_as_int(tx.w) + __float_as_int(ty.w) + __float_as_int(tz.w);
       const uint32_t blk = s_blk[t][code >> 16];
       if (blk >= M.pool_blocks) continue;

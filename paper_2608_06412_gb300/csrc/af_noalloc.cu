@@ -26,6 +26,7 @@
 #include <cstdio>
 #include <mutex>
 
+#include "af_cube.cuh"
 #include "af_internal.cuh"
 
 namespace af {
@@ -85,82 +86,101 @@ __device__ inline bool box_index(const Box& B, int x, int y, int z, size_t* at) 
   return true;
 }
 
-__global__ void __launch_bounds__(256) k_na_prepare(MapView M, const float* __restrict__ xyz,
-                                                     uint32_t n, Pose P,
-                                                     float4* __restrict__ scratch) {
-  const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  float p[3], range;
-  int rel[3];
-  const bool valid = prepare_return(M, P, xyz[3 * k], xyz[3 * k + 1], xyz[3 * k + 2], p, &range, rel);
-  scratch[k] = make_float4(p[0], p[1], p[2], valid ? 1.f : 0.f);
+// Returns per CTA of the two kernels below: the per-axis work of a return is
+// done once for its (2m+1)^3 cube voxels.
+constexpr int kBoxTile = 8;
+
+// Box offset of the coordinate with domain-relative index j on axis ax (the
+// three axes' offsets add up to the voxel's element), or -1 outside the box.
+__device__ inline long long box_offset(const Box& B, int ax, int j) {
+  j -= B.lo[ax];
+  if ((unsigned)j >= (unsigned)B.dim[ax]) return -1;
+  return ax == 0 ? (long long)j
+                 : (ax == 1 ? (long long)j * B.dim[0] : (long long)j * ((long long)B.dim[0] * B.dim[1]));
 }
 
-// One thread per (return, cube offset), the same arithmetic as the hashed
-// path, accumulating into the caller's dense box; cleared-band marks too.
-__global__ void __launch_bounds__(256) k_na_integrate(MapView M, const float4* __restrict__ scratch,
-                                                       uint32_t n, float q0, float q1, float q2,
-                                                       Box B) {
-  const int W = 2 * M.m + 1;
-  const uint64_t C = (uint64_t)W * W * W;
-  const uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint64_t pairs = C * n;
-  const uint64_t band = (uint64_t)M.ns * n;
-  if (e < pairs) {
-    const uint32_t k = (uint32_t)(e / C);
-    const int o = (int)(e % C);
-    const float4 p = scratch[k];
-    if (p.w == 0.f) return;
-    const float b0 = __fsub_rn(p.x, q0), b1 = __fsub_rn(p.y, q1), b2 = __fsub_rn(p.z, q2);
-    const float range =
-        __fsqrt_rn(__fadd_rn(__fadd_rn(__fmul_rn(b0, b0), __fmul_rn(b1, b1)), __fmul_rn(b2, b2)));
-    int i[3];
-    // k_na_prepare accepted the return, so its voxel index exists; checked
-    // again here so that no index is used unchecked
-    if (!(voxel_index(p.x, M, &i[0]) && voxel_index(p.y, M, &i[1]) &&
-          voxel_index(p.z, M, &i[2])))
-      return;
-    const int jx = i[0] - M.dom_vox[0] + o % W - M.m;
-    const int jy = i[1] - M.dom_vox[1] + (o / W) % W - M.m;
-    const int jz = i[2] - M.dom_vox[2] + o / (W * W) - M.m;
-    size_t at;
-    if (!box_index(B, jx, jy, jz, &at)) return;
-    const float x0 = voxel_centre(jx + M.dom_vox[0], M.v);
-    const float x1 = voxel_centre(jy + M.dom_vox[1], M.v);
-    const float x2 = voxel_centre(jz + M.dom_vox[2], M.v);
-    const float a0 = __fsub_rn(x0, p.x), a1 = __fsub_rn(x1, p.y), a2 = __fsub_rn(x2, p.z);
-    const float aa = __fadd_rn(__fadd_rn(__fmul_rn(a0, a0), __fmul_rn(a1, a1)), __fmul_rn(a2, a2));
-    if (aa > 0.f) {
-      const float dot = __fadd_rn(__fadd_rn(__fmul_rn(a0, b0), __fmul_rn(a1, b1)), __fmul_rn(a2, b2));
-      if (__fdiv_rn(dot, __fmul_rn(__fsqrt_rn(aa), range)) > M.cone_cos) return;
+// One CTA per kBoxTile returns, one thread per cube offset: the returns are
+// transformed and their per-axis terms and box offsets computed once into
+// shared memory, then each thread walks the returns for its offset, the same
+// arithmetic as the hashed path (af_cube.cuh), one 64-bit atomic add per pair;
+// the cleared-band marks follow. The world positions go to `scratch` for
+// k_box_finalize. Issue-bound like k_integrate: 32.5 us per pine frame; with one
+// thread per (return, offset) that did all of a pair's work, 64-bit divisions
+// included, for itself, 73 us and a launch for the transform.
+template <int W>
+__global__ void __launch_bounds__(CubeShape<W>::NT) k_box_integrate(MapView M,
+                                                                    const float* __restrict__ xyz,
+                                                                    uint32_t n, Pose P,
+                                                                    float4* __restrict__ scratch,
+                                                                    Box B) {
+  using S = CubeShape<W>;
+  __shared__ float4 s_p[kBoxTile], s_pr[kBoxTile];
+  __shared__ float4 s_term[kBoxTile][3][W];
+  __shared__ long long s_off[kBoxTile][3][W];
+  const int tid = threadIdx.x;
+  const uint32_t r0 = blockIdx.x * kBoxTile;
+  const float q[3] = {P.r[0][3], P.r[1][3], P.r[2][3]};
+  if (tid < kBoxTile) {
+    const uint32_t k = r0 + tid;
+    float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (k < n) {
+      float w[3], range;
+      int rel[3];
+      const bool valid = prepare_return(M, P, xyz[3 * k], xyz[3 * k + 1], xyz[3 * k + 2], w, &range, rel);
+      p = valid ? make_float4(w[0], w[1], w[2], 1.f) : p;
+      scratch[k] = p;
     }
-    const float c0 = __fsub_rn(x0, q0), c1 = __fsub_rn(x1, q1), c2 = __fsub_rn(x2, q2);
-    const float cc = __fadd_rn(__fadd_rn(__fmul_rn(c0, c0), __fmul_rn(c1, c1)), __fmul_rn(c2, c2));
-    float d = __fsub_rn(range, __fsqrt_rn(cc));
-    d = d < M.dlo ? M.dlo : d;
-    d = d > M.tau ? M.tau : d;
-    const long long dq = __float2ll_rn(__fmul_rn(d, kScale));
-    atomicAdd(B.vox + at, make_word(dq, 1ull));
-  } else if (e < pairs + band) {
-    const uint64_t f = e - pairs;
-    const uint32_t k = (uint32_t)(f / M.ns);
-    const int s = (int)(f % M.ns) + 1;
-    const float4 p4 = scratch[k];
-    if (p4.w == 0.f) return;
-    const float p[3] = {p4.x, p4.y, p4.z}, q[3] = {q0, q1, q2};
-    const float b0 = __fsub_rn(p[0], q0), b1 = __fsub_rn(p[1], q1), b2 = __fsub_rn(p[2], q2);
-    const float range =
-        __fsqrt_rn(__fadd_rn(__fadd_rn(__fmul_rn(b0, b0), __fmul_rn(b1, b1)), __fmul_rn(b2, b2)));
+    s_p[tid] = p;
+    s_pr[tid] = return_record(p, q[0], q[1], q[2]);
+  }
+  __syncthreads();
+  for (int e = tid; e < kBoxTile * 3 * W; e += S::NT) {
+    const int t = e / (3 * W), ax = (e / W) % 3, k = e % W;
+    const float4 p = s_p[t];
+    if (p.w == 0.f) continue;
+    const float pa = ax == 0 ? p.x : (ax == 1 ? p.y : p.z);
+    int i;
+    voxel_index(pa, M, &i);  // accepted by prepare_return
+    s_term[t][ax][k] = axis_terms(M, pa, q[ax], i + k - S::MR);
+    s_off[t][ax][k] = box_offset(B, ax, i - M.dom_vox[ax] + k - S::MR);
+  }
+  __syncthreads();
+  int kx[S::OPT], ky[S::OPT], kz[S::OPT];  // ox fastest: neighbouring threads, neighbouring words
+#pragma unroll
+  for (int s = 0; s < S::OPT; ++s) {
+    const int o = tid + s * S::NT;
+    kx[s] = o % W;
+    ky[s] = (o / W) % W;
+    kz[s] = o / (W * W);
+  }
+  for (int t = 0; t < kBoxTile; ++t) {
+    const float4 pr = s_pr[t];
+    if (pr.w == 0.f) continue;  // uniform across the block
+#pragma unroll
+    for (int s = 0; s < S::OPT; ++s) {
+      if (tid + s * S::NT >= S::C) break;
+      long long dq;
+      if (!pair_contribution(M, s_term[t][0][kx[s]], s_term[t][1][ky[s]], s_term[t][2][kz[s]], pr, &dq))
+        continue;
+      const long long ox = s_off[t][0][kx[s]], oy = s_off[t][1][ky[s]], oz = s_off[t][2][kz[s]];
+      if ((ox | oy | oz) >= 0) atomicAdd(B.vox + (ox + oy + oz), make_word(dq, 1ull));
+    }
+  }
+  for (int e = tid; e < kBoxTile * M.ns; e += S::NT) {
+    const int t = e / M.ns, s = e % M.ns + 1;
+    if (s_p[t].w == 0.f) continue;
+    const float p[3] = {s_p[t].x, s_p[t].y, s_p[t].z};
     int sv[3];
-    if (!band_sample(M, p, q, range, s, sv)) return;
     size_t at;
-    if (box_index(B, sv[0], sv[1], sv[2], &at)) B.flags[at] |= 1u;  // every writer sets bit 0
+    if (band_sample(M, p, q, s_pr[t].x, s, sv) && box_index(B, sv[0], sv[1], sv[2], &at))
+      B.flags[at] |= 1u;  // every writer sets bit 0
   }
 }
 
 // Weight cap and occupied / known flags of box voxel `at`. Idempotent (a
 // capped weight is not capped again), so threads that reach the same voxel
-// through different returns write the same word and flags.
+// through different returns write the same word and flags; a voxel that another
+// thread has done is read but not written.
 __device__ inline void finalize_voxel(const MapView& M, const Box& B, size_t at) {
   unsigned long long word = B.vox[at];
   unsigned long long w = word & kWMask;
@@ -170,51 +190,60 @@ __device__ inline void finalize_voxel(const MapView& M, const Box& B, size_t at)
     w = M.w_cap;
     B.vox[at] = make_word(S, w);
   }
-  const unsigned cl = B.flags[at] & 1u;
+  const unsigned was = B.flags[at], cl = was & 1u;
   const unsigned occ = (w >= 1 && S < (long long)M.rcq * (long long)w) ? 1u : 0u;
   const unsigned kn = (w >= 1 || cl) ? 1u : 0u;
-  B.flags[at] = (uint8_t)(cl | (occ << 1) | (kn << 2));
+  const unsigned now = cl | (occ << 1) | (kn << 2);
+  if (now != was) B.flags[at] = (uint8_t)now;
 }
 
 // Weight cap and flags of every voxel this scan touched -- the cube voxels
 // and cleared-band samples of its accepted returns, enumerated as in
-// k_na_integrate -- after all of the scan's additions (a launch of its own).
-// Voxels the scan does not touch keep their words and flags.
-__global__ void __launch_bounds__(256) k_na_finalize(MapView M, const float4* __restrict__ scratch,
-                                                      uint32_t n, float q0, float q1, float q2,
-                                                      Box B) {
-  const int W = 2 * M.m + 1;
-  const uint64_t C = (uint64_t)W * W * W;
-  const uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint64_t pairs = C * n;
-  const uint64_t band = (uint64_t)M.ns * n;
-  size_t at;
-  if (e < pairs) {
-    const uint32_t k = (uint32_t)(e / C);
-    const int o = (int)(e % C);
-    const float4 p = scratch[k];
-    if (p.w == 0.f) return;
-    int i[3];
-    if (!(voxel_index(p.x, M, &i[0]) && voxel_index(p.y, M, &i[1]) &&
-          voxel_index(p.z, M, &i[2])))
-      return;
-    const int jx = i[0] - M.dom_vox[0] + o % W - M.m;
-    const int jy = i[1] - M.dom_vox[1] + (o / W) % W - M.m;
-    const int jz = i[2] - M.dom_vox[2] + o / (W * W) - M.m;
-    if (box_index(B, jx, jy, jz, &at)) finalize_voxel(M, B, at);
-  } else if (e < pairs + band) {
-    const uint64_t f = e - pairs;
-    const uint32_t k = (uint32_t)(f / M.ns);
-    const int s = (int)(f % M.ns) + 1;
-    const float4 p4 = scratch[k];
-    if (p4.w == 0.f) return;
-    const float p[3] = {p4.x, p4.y, p4.z}, q[3] = {q0, q1, q2};
-    const float b0 = __fsub_rn(p[0], q0), b1 = __fsub_rn(p[1], q1), b2 = __fsub_rn(p[2], q2);
-    const float range =
-        __fsqrt_rn(__fadd_rn(__fadd_rn(__fmul_rn(b0, b0), __fmul_rn(b1, b1)), __fmul_rn(b2, b2)));
+// k_box_integrate -- after all of the scan's additions (a launch of its own).
+// Voxels the scan does not touch keep their words and flags. A voxel is reached
+// through many returns: bound by the L2 reads of its word and flags (32 us per
+// pine frame; one thread per (return, offset) that found its voxel by itself and
+// always wrote the flags took 117 us).
+template <int W>
+__global__ void __launch_bounds__(CubeShape<W>::NT) k_box_finalize(MapView M,
+                                                                   const float4* __restrict__ scratch,
+                                                                   uint32_t n, float q0, float q1,
+                                                                   float q2, Box B) {
+  using S = CubeShape<W>;
+  __shared__ float4 s_p[kBoxTile];
+  __shared__ long long s_off[kBoxTile][3][W];
+  const int tid = threadIdx.x;
+  const uint32_t r0 = blockIdx.x * kBoxTile;
+  for (int e = tid; e < kBoxTile * 3 * W; e += S::NT) {
+    const int t = e / (3 * W), ax = (e / W) % 3, k = e % W;
+    const float4 p = r0 + t < n ? scratch[r0 + t] : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (ax == 0 && k == 0) s_p[t] = p;
+    if (p.w == 0.f) continue;
+    int i;
+    voxel_index(ax == 0 ? p.x : (ax == 1 ? p.y : p.z), M, &i);
+    s_off[t][ax][k] = box_offset(B, ax, i - M.dom_vox[ax] + k - S::MR);
+  }
+  __syncthreads();
+  for (int t = 0; t < kBoxTile; ++t) {
+    if (s_p[t].w == 0.f) continue;
+#pragma unroll
+    for (int s = 0; s < S::OPT; ++s) {
+      const int o = tid + s * S::NT;
+      if (o >= S::C) break;
+      const long long ox = s_off[t][0][o % W], oy = s_off[t][1][(o / W) % W], oz = s_off[t][2][o / (W * W)];
+      if ((ox | oy | oz) >= 0) finalize_voxel(M, B, (size_t)(ox + oy + oz));
+    }
+  }
+  const float q[3] = {q0, q1, q2};
+  for (int e = tid; e < kBoxTile * M.ns; e += S::NT) {
+    const int t = e / M.ns, s = e % M.ns + 1;
+    if (s_p[t].w == 0.f) continue;
+    const float p[3] = {s_p[t].x, s_p[t].y, s_p[t].z};
     int sv[3];
-    if (!band_sample(M, p, q, range, s, sv)) return;
-    if (box_index(B, sv[0], sv[1], sv[2], &at)) finalize_voxel(M, B, at);
+    size_t at;
+    if (band_sample(M, p, q, return_record(s_p[t], q0, q1, q2).x, s, sv) &&
+        box_index(B, sv[0], sv[1], sv[2], &at))
+      finalize_voxel(M, B, at);
   }
 }
 
@@ -300,12 +329,16 @@ extern "C" af_status af_integrate_scan_noalloc(const af_config* cfg, const float
 
   cudaStream_t s = (cudaStream_t)stream;
   if (n > 0) {
-    k_na_prepare<<<(n + 255) / 256, 256, 0, s>>>(M, d_xyz, n, P, scratch);
-    const int W = 2 * M.m + 1;
-    const uint64_t work = (uint64_t)n * W * W * W + (uint64_t)n * M.ns;
-    const unsigned grid = (unsigned)((work + 255) / 256);
-    k_na_integrate<<<grid, 256, 0, s>>>(M, scratch, n, pose[3], pose[7], pose[11], B);
-    k_na_finalize<<<grid, 256, 0, s>>>(M, scratch, n, pose[3], pose[7], pose[11], B);
+    const unsigned grid = (n + kBoxTile - 1) / kBoxTile;
+    switch (2 * M.m + 1) {
+#define AF_CASE(W)                                                                                    \
+  case W:                                                                                             \
+    k_box_integrate<W><<<grid, CubeShape<W>::NT, 0, s>>>(M, d_xyz, n, P, scratch, B);                \
+    k_box_finalize<W><<<grid, CubeShape<W>::NT, 0, s>>>(M, scratch, n, pose[3], pose[7], pose[11], B); \
+    break;
+      AF_CASE(3) AF_CASE(5) AF_CASE(7) AF_CASE(9) AF_CASE(11) AF_CASE(13) AF_CASE(15) AF_CASE(17)
+#undef AF_CASE
+    }
   }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return nfail(AF_ERR_CUDA, "af_integrate_scan_noalloc: launch failed: %s",
