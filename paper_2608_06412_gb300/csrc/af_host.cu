@@ -411,7 +411,7 @@ static void free_all(af_ctx* c) {
   cudaFree(c->d_img);
   for (void* p : {(void*)c->d_pid, (void*)c->d_pst, (void*)c->d_pviews, (void*)c->d_pnew,
                   (void*)c->d_pnear, (void*)c->d_psnapw, (void*)c->d_psnapc, (void*)c->d_pchgmask,
-                  (void*)c->d_phist, (void*)c->d_psamp, (void*)c->d_psel, (void*)c->d_pblock,
+                  (void*)c->d_phist, (void*)c->d_psamp, (void*)c->d_pdrawn, (void*)c->d_psel, (void*)c->d_pblock,
                   (void*)c->d_pcount, (void*)c->d_pnnoff, (void*)c->d_pc2f, (void*)c->d_psnap})
     cudaFree(p);
   cudaFreeHost(c->h_status);

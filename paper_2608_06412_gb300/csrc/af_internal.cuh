@@ -299,7 +299,16 @@ struct PtCounters {
   uint32_t nsnap;     // bricks whose state was copied before the frame's scan
   uint32_t nsel;      // points selected for evaluation
   uint32_t evals;     // evaluations of the last call
-  uint32_t pad[2];
+  uint32_t ended;     // CTAs that have ended (count_ended; zero between kernels)
+  uint32_t ndrawn;    // listed candidates of the draw
+};
+
+// A candidate of the draw: a changed voxel whose hash lies at or below the bin
+// that holds the draw's bound.
+struct PtDrawn {
+  unsigned long long h;
+  uint32_t at;  // index in the dirty list * 512 + voxel
+  uint32_t pad;
 };
 
 // The draw of changed voxels for the neighbourhood trigger: a radix
@@ -309,6 +318,8 @@ struct PtSample {
   unsigned long long t;       // the largest hash drawn (all ones: every changed voxel)
   uint32_t below;             // changed voxels known to lie below the prefix's range
   uint32_t done;              // 1 once t is final
+  uint32_t listed;            // 1: every drawn voxel is in the list of candidates
+  uint32_t pad;
 };
 
 // Parameters of the layer as the kernels read them.
@@ -323,6 +334,7 @@ struct PtView {
   uint32_t* chgmask;          // per dirty brick: 512 bits, voxels whose state changed
   uint32_t* hist;             // 2048 bins of the draw's radix selection
   PtSample* samp;
+  PtDrawn* drawn;             // kDrawList candidates
   int trig_exact;             // 1: changed voxels within trig_radius; 0: touched bricks
   int trig_radius;
   uint32_t trig_sample;       // changed voxels drawn per frame (0: all)

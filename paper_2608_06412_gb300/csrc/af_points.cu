@@ -12,17 +12,22 @@
 //                 per-brick point-id table)
 //  k_pts_near     (brick rule) bricks next to the scan's touched bricks
 //  k_pts_create   new points numbered by key order within the frame, so ids
-//                 never depend on thread timing
+//                 never depend on thread timing; the last CTA commits them
 //  k_pts_views    once per (point, scan): sensor sum and stored viewpoints
-//  k_pts_diff     per touched brick: the voxels whose stored state changed
-//  k_pts_hist / k_pts_pick
-//                 the draw: radix selection, 11 bits per pass, of the
-//                 trig_sample smallest hashes of the changed voxels
-//  k_pts_scatter  every drawn changed voxel queues the points within r_u
+//  k_pts_diff     per touched brick: the voxels whose stored state changed, and
+//                 the histogram of the top 11 bits of their hashes; the last
+//                 CTA finds the bin that holds the draw's bound
+//  k_pts_collect  the changed voxels up to that bin, as a list; the last CTA
+//                 ranks those of the bin: t, the largest hash drawn
+//  k_pts_scatter_list
+//                 every drawn voxel of the list queues the points within r_u
+//  k_pts_hist / k_pts_pick / k_pts_scatter
+//                 the same for draws too large to list (or of every changed
+//                 voxel): radix selection, 11 bits per pass
 //  k_pts_trigger  one thread per point: TSDF change, brick rule, sensor
-//                 motion for blocked points
-//  k_pts_count / k_pts_scan / k_pts_select
-//                 the first `budget` queued ids in id order
+//                 motion for blocked points; queued points per 1024 ids, summed
+//                 up by the last CTA
+//  k_pts_select   the first `budget` queued ids in id order
 //  k_pts_snap     (coarse-to-fine search only) the stored best directions
 //                 as they are before the batch
 //  k_pts_eval     one warp per selected point: confidence gate, nearest
@@ -89,6 +94,21 @@ __device__ inline bool return_voxel(const MapView& M, const float4* ret, uint32_
   return true;
 }
 
+// Whether the calling CTA is the launch's last to get here, its threads' writes
+// before it and every other CTA's visible to it. The counter is left at zero.
+__device__ inline bool last_cta(uint32_t* ended) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(ended, 1u) == gridDim.x - 1u;
+    if (last) *ended = 0u;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
 // One thread per return: the voxel of an accepted return becomes a new
 // point if it has none (claimed with -2 until k_pts_create numbers it).
 __global__ void __launch_bounds__(256) k_pts_mark(MapView M, const float4* __restrict__ ret,
@@ -152,28 +172,6 @@ __device__ inline void brick_voxel(const MapView& M, uint32_t blk, int l, int* x
   *z = (int)(key >> 42) * 8 + (l >> 6);
 }
 
-// Per touched brick (after the weight cap): voxels whose word or cleared mark
-// differs from the snapshot, as a 512-bit mask, and their count.
-__global__ void __launch_bounds__(512) k_pts_diff(MapView M, PtView V) {
-  const uint32_t count = __ldcg(&M.ctl->dirty_count), nsnap = V.C->nsnap;
-  if (count > nsnap && blockIdx.x == 0 && threadIdx.x == 0)
-    latch_status(M.ctl, kStatusCapacity);  // a brick missed by the snapshot: never expected
-  const int l = threadIdx.x, lane = l & 31, wi = l >> 5;
-  const uint32_t nd = min(count, nsnap);
-  for (uint32_t d = blockIdx.x; d < nd; d += gridDim.x) {
-    const uint32_t blk = M.dirty[d];
-    const bool cl_now = (__ldcg(M.cleared + (size_t)blk * 16 + wi) >> lane) & 1u;
-    const bool cl_then = (V.snapc[(size_t)d * 16 + wi] >> lane) & 1u;
-    const bool ch = __ldcg(M.vox + (size_t)blk * kBrickVox + l) != V.snapw[(size_t)d * kBrickVox + l] ||
-                    cl_now != cl_then;
-    const unsigned b = __ballot_sync(0xffffffffu, ch);
-    if (lane == 0) {
-      V.chgmask[(size_t)d * 16 + wi] = b;
-      if (b) atomicAdd(&V.C->nchanged, (unsigned)__popc(b));
-    }
-  }
-}
-
 // The draw's radix selection: digits of kDrawBits bits from the top of the
 // hash down (the last one narrower), at most kDrawPasses passes; it stops as
 // soon as a digit's bin holds exactly the draws still missing.
@@ -183,6 +181,174 @@ constexpr int kDrawPasses = (64 + kDrawBits - 1) / kDrawBits;
 
 __device__ inline int draw_hi(int pass) { return 64 - kDrawBits * pass; }  // bits above the digit
 __device__ inline int draw_lo(int pass) { return max(0, 64 - kDrawBits * (pass + 1)); }
+
+// Draws of up to kDrawSample voxels go through a list of candidates: the voxels
+// of the bins up to the one that holds the bound. The last of those bins holds
+// nchanged / 2048 voxels on average, so the list overflows only when one scan
+// changes tens of millions of voxels (then one CTA finds t by itself).
+constexpr uint32_t kDrawSample = 4096;
+#ifdef AF_CHECKED
+constexpr uint32_t kDrawList = 64;  // the checked build's draws of 256 overflow it
+#else
+constexpr uint32_t kDrawList = 32768;
+#endif
+
+// The digit of the bin that holds the `need`-th smallest of the histogrammed
+// hashes, and the count before it and in it (1024 threads, 2 bins each; the CTA
+// calls together); clears the histogram.
+__device__ inline void pick_bin(uint32_t* hist, uint32_t need, uint32_t* digit, uint32_t* before,
+                                uint32_t* count) {
+  __shared__ uint32_t part[32];
+  __shared__ uint32_t res[3];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const uint32_t h0 = __ldcg(hist + 2 * tid), h1 = __ldcg(hist + 2 * tid + 1), sum = h0 + h1;
+  hist[2 * tid] = 0u;
+  hist[2 * tid + 1] = 0u;
+  uint32_t v = sum;
+  for (int off = 1; off < 32; off <<= 1) {
+    const uint32_t u = __shfl_up_sync(0xffffffffu, v, off);
+    if (lane >= off) v += u;
+  }
+  if (lane == 31) part[w] = v;
+  __syncthreads();
+  if (w == 0) {
+    uint32_t p = part[lane];
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t u = __shfl_up_sync(0xffffffffu, p, off);
+      if (lane >= off) p += u;
+    }
+    part[lane] = p;
+  }
+  __syncthreads();
+  const uint32_t incl = v + (w ? part[w - 1] : 0u), excl = incl - sum;
+  if (excl < need && need <= incl) {
+    const bool first = excl + h0 >= need;
+    res[0] = 2 * tid + (first ? 0 : 1);
+    res[1] = excl + (first ? 0u : h0);
+    res[2] = first ? h0 : h1;
+  }
+  __syncthreads();
+  *digit = res[0];
+  *before = res[1];
+  *count = res[2];
+  __syncthreads();
+}
+
+// Per touched brick (after the weight cap): voxels whose word or cleared mark
+// differs from the snapshot, as a 512-bit mask, and their count. With `draw`
+// also the histogram of the top digit of their hashes (1024 threads: two bricks
+// at a time); the last CTA picks the bound's bin, or takes every voxel when no
+// more changed than are drawn.
+__global__ void __launch_bounds__(1024) k_pts_diff(MapView M, PtView V, int draw) {
+  __shared__ uint32_t s_hist[kDrawBins];
+  const uint32_t count = __ldcg(&M.ctl->dirty_count), nsnap = V.C->nsnap;
+  if (count > nsnap && blockIdx.x == 0 && threadIdx.x == 0)
+    latch_status(M.ctl, kStatusCapacity);  // a brick missed by the snapshot: never expected
+  const int l = threadIdx.x & 511, lane = l & 31, wi = l >> 5;
+  const uint32_t nd = min(count, nsnap);
+  if (draw) {
+    s_hist[2 * threadIdx.x] = 0u;
+    s_hist[2 * threadIdx.x + 1] = 0u;
+    __syncthreads();
+  }
+  uint32_t changed = 0;  // of this warp's voxels
+  for (uint32_t d = 2 * blockIdx.x + (threadIdx.x >> 9); d < nd; d += 2 * gridDim.x) {
+    const uint32_t blk = M.dirty[d];
+    const bool cl_now = (__ldcg(M.cleared + (size_t)blk * 16 + wi) >> lane) & 1u;
+    const bool cl_then = (V.snapc[(size_t)d * 16 + wi] >> lane) & 1u;
+    const bool ch = __ldcg(M.vox + (size_t)blk * kBrickVox + l) != V.snapw[(size_t)d * kBrickVox + l] ||
+                    cl_now != cl_then;
+    const unsigned b = __ballot_sync(0xffffffffu, ch);
+    changed += __popc(b);
+    if (lane == 0) V.chgmask[(size_t)d * 16 + wi] = b;
+    if (draw && ch) {
+      int x, y, z;
+      brick_voxel(M, blk, l, &x, &y, &z);
+      atomicAdd(s_hist + (mix64(draw_key(M, x, y, z) ^ V.salt) >> draw_lo(0)), 1u);
+    }
+  }
+  if (lane == 0 && changed) atomicAdd(&V.C->nchanged, changed);
+  if (!draw) return;
+  __syncthreads();
+  for (int b = threadIdx.x; b < kDrawBins; b += 1024)
+    if (s_hist[b]) atomicAdd(V.hist + b, s_hist[b]);
+  if (!last_cta(&V.C->ended)) return;
+  const uint32_t k = V.trig_sample, n = __ldcg(&V.C->nchanged);
+  uint32_t digit = 0, before = 0, cnt = 0;
+  const bool all = n <= k;
+  pick_bin(V.hist, all ? n : k, &digit, &before, &cnt);
+  if (threadIdx.x == 0) {
+    PtSample* S = V.samp;
+    S->done = all;
+    S->t = ~0ull;
+    S->prefix = all ? kDrawBins - 1 : digit;
+    S->below = before;
+    S->listed = (all ? n : before + cnt) <= kDrawList;
+    V.C->ndrawn = 0;
+  }
+}
+
+// The list of the draw's candidates; the last CTA finds t among those of the
+// bound's bin: the need-th smallest (mix64 is a bijection, so hashes never tie).
+// Candidates that overflow the list: the last CTA takes the remaining digits over
+// all changed voxels.
+__global__ void __launch_bounds__(1024) k_pts_collect(MapView M, PtView V) {
+  __shared__ uint32_t s_hist[kDrawBins];
+  PtSample* S = V.samp;
+  const unsigned long long prefix = S->prefix;
+  const bool listed = S->listed, done = S->done;
+  const int l = threadIdx.x & 511, lane = l & 31, wi = l >> 5;
+  const uint32_t nd = min(__ldcg(&M.ctl->dirty_count), V.C->nsnap);
+  if (listed)
+    for (uint32_t d = 2 * blockIdx.x + (threadIdx.x >> 9); d < nd; d += 2 * gridDim.x) {
+      if (!((V.chgmask[(size_t)d * 16 + wi] >> lane) & 1u)) continue;
+      int x, y, z;
+      brick_voxel(M, M.dirty[d], l, &x, &y, &z);
+      const unsigned long long h = mix64(draw_key(M, x, y, z) ^ V.salt);
+      if ((h >> draw_lo(0)) > prefix) continue;
+      const uint32_t at = atomicAdd(&V.C->ndrawn, 1u);
+      if (at < kDrawList) V.drawn[at] = PtDrawn{h, d * (uint32_t)kBrickVox + (uint32_t)l, 0u};
+    }
+  if (!last_cta(&V.C->ended) || done) return;
+  const uint32_t need = V.trig_sample - S->below;
+  if (listed) {
+    const uint32_t n = min(__ldcg(&V.C->ndrawn), kDrawList);
+    for (uint32_t i = threadIdx.x; i < n; i += 1024) {
+      const unsigned long long h = __ldcg(&V.drawn[i].h);
+      if ((h >> draw_lo(0)) != prefix) continue;
+      uint32_t rank = 0;
+      for (uint32_t j = 0; j < n; ++j) {
+        const unsigned long long o = __ldcg(&V.drawn[j].h);
+        rank += (o >> draw_lo(0)) == prefix && o < h;
+      }
+      if (rank + 1 == need) S->t = h;
+    }
+    return;
+  }
+  unsigned long long pre = prefix;
+  uint32_t left = need;
+  for (int pass = 1; pass < kDrawPasses; ++pass) {
+    const int hi = draw_hi(pass), lo = draw_lo(pass);
+    s_hist[2 * threadIdx.x] = 0u;
+    s_hist[2 * threadIdx.x + 1] = 0u;
+    __syncthreads();
+    for (uint32_t d = threadIdx.x >> 9; d < nd; d += 2) {
+      if (!((V.chgmask[(size_t)d * 16 + wi] >> lane) & 1u)) continue;
+      int x, y, z;
+      brick_voxel(M, M.dirty[d], l, &x, &y, &z);
+      const unsigned long long h = mix64(draw_key(M, x, y, z) ^ V.salt);
+      if ((h >> hi) == pre) atomicAdd(s_hist + ((h >> lo) & ((1ull << (hi - lo)) - 1ull)), 1u);
+    }
+    __syncthreads();
+    V.hist[2 * threadIdx.x] = s_hist[2 * threadIdx.x];  // pick_bin reads and clears it
+    V.hist[2 * threadIdx.x + 1] = s_hist[2 * threadIdx.x + 1];
+    uint32_t digit, before, cnt;
+    pick_bin(V.hist, left, &digit, &before, &cnt);
+    pre = (pre << (hi - lo)) | digit;
+    left -= before;
+  }
+  if (threadIdx.x == 0) S->t = pre;
+}
 
 // One pass of the draw: histogram (per CTA in shared memory, then merged) of
 // this pass's digit of the hashes of the changed voxels whose higher bits
@@ -297,6 +463,69 @@ __global__ void __launch_bounds__(512) k_pts_scatter(MapView M, PtView V) {
   }
 }
 
+// k_pts_scatter for a listed draw: one warp per candidate, the ball's offsets over
+// its lanes, the candidate's neighbour bricks looked up by lanes 0-26. (One thread
+// per changed voxel that walked the ball alone: 65 us per pine frame.)
+__global__ void __launch_bounds__(256) k_pts_scatter_list(MapView M, PtView V) {
+  const PtSample* S = V.samp;
+  const int lane = threadIdx.x & 31;
+  const int R = V.trig_radius, R2 = R * R, E = 2 * R + 1;
+  const int BX = M.dim_vox[0] >> 3, BY = M.dim_vox[1] >> 3, BZ = M.dim_vox[2] >> 3;
+  const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+  uint32_t w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (S->listed) {
+    const unsigned long long t = S->t;
+    const uint32_t n = min(V.C->ndrawn, kDrawList);
+    for (; w < n; w += warps) {
+      const PtDrawn c = V.drawn[w];
+      if (c.h > t) continue;
+      int x, y, z;
+      brick_voxel(M, M.dirty[c.at / kBrickVox], (int)(c.at % kBrickVox), &x, &y, &z);
+      const int bx = x >> 3, by = y >> 3, bz = z >> 3;
+      uint32_t nb = kNoBlock;
+      if (lane < 27) {
+        const int nx = bx + lane % 3 - 1, ny = by + (lane / 3) % 3 - 1, nz = bz + lane / 9 - 1;
+        // bricks that the ball reaches
+        const bool reach = ((x + R) >> 3) >= nx && ((x - R) >> 3) <= nx && ((y + R) >> 3) >= ny &&
+                           ((y - R) >> 3) <= ny && ((z + R) >> 3) >= nz && ((z - R) >> 3) <= nz;
+        if (reach && (unsigned)nx < (unsigned)BX && (unsigned)ny < (unsigned)BY && (unsigned)nz < (unsigned)BZ)
+          nb = lookup_brick(M, pack_brick(nx, ny, nz));
+      }
+      for (int o0 = 0; o0 < E * E * E; o0 += 32) {
+        const int o = o0 + lane;
+        const int dx = o % E - R, dy = (o / E) % E - R, dz = o / (E * E) - R;
+        const int nx = x + dx, ny = y + dy, nz = z + dz;
+        const bool in = o < E * E * E && dx * dx + dy * dy + dz * dz <= R2 && box_rel(M, nx, ny, nz);
+        const int i = ((nx >> 3) - bx + 1) + 3 * (((ny >> 3) - by + 1) + 3 * ((nz >> 3) - bz + 1));
+        const uint32_t b = __shfl_sync(0xffffffffu, nb, in ? i : 0);
+        if (!in || b == kNoBlock) continue;
+        const int32_t id = V.pid[(size_t)b * kBrickVox + vox_slot(nx, ny, nz)];
+        if (id >= 0 && check_index((uint32_t)id < V.capacity, M.ctl)) V.st[id].queued = 1;
+      }
+    }
+    return;
+  }
+  // an overflowed list: every changed voxel up to t, one lane each
+  const unsigned long long t = S->t;
+  const uint32_t nd = min(__ldcg(&M.ctl->dirty_count), V.C->nsnap);
+  for (uint32_t u = w; u < nd * 16u; u += warps) {
+    const uint32_t d = u >> 4;
+    const int l = (int)(u & 15u) * 32 + lane;
+    if (!((V.chgmask[u] >> lane) & 1u)) continue;
+    int x, y, z;
+    brick_voxel(M, M.dirty[d], l, &x, &y, &z);
+    if (mix64(draw_key(M, x, y, z) ^ V.salt) > t) continue;
+    for (int o = 0; o < E * E * E; ++o) {
+      const int dx = o % E - R, dy = (o / E) % E - R, dz = o / (E * E) - R;
+      if (dx * dx + dy * dy + dz * dz > R2 || !box_rel(M, x + dx, y + dy, z + dz)) continue;
+      const uint32_t b = lookup_brick(M, pack_brick((x + dx) >> 3, (y + dy) >> 3, (z + dz) >> 3));
+      if (b == kNoBlock) continue;
+      const int32_t id = V.pid[(size_t)b * kBrickVox + vox_slot(x + dx, y + dy, z + dz)];
+      if (id >= 0 && check_index((uint32_t)id < V.capacity, M.ctl)) V.st[id].queued = 1;
+    }
+  }
+}
+
 // New points: id = count + rank of the key among the frame's new keys.
 __global__ void __launch_bounds__(256) k_pts_create(MapView M, PtView V) {
   __shared__ unsigned long long tile[256];
@@ -343,10 +572,7 @@ __global__ void __launch_bounds__(256) k_pts_create(MapView M, PtView V) {
     s.pad = 0;
     V.st[id] = s;
   }
-}
-
-__global__ void k_pts_commit(PtView V) {
-  V.C->count = min(V.C->count + V.C->nnew, V.capacity);
+  if (last_cta(&V.C->ended) && threadIdx.x == 0) V.C->count = min(base + nnew, V.capacity);
 }
 
 __global__ void __launch_bounds__(256) k_pts_views(MapView M, const float4* __restrict__ ret,
@@ -383,54 +609,68 @@ __global__ void __launch_bounds__(256) k_pts_views(MapView M, const float4* __re
   }
 }
 
-__global__ void __launch_bounds__(256) k_pts_trigger(MapView M, PtView V, uint32_t frame, int moved) {
-  const uint32_t count = V.C->count;
-  for (uint32_t id = blockIdx.x * blockDim.x + threadIdx.x; id < count; id += gridDim.x * blockDim.x) {
-    PtState* s = V.st + id;
-    const float cur = tsdf_word(__ldcg(M.vox + (size_t)s->blk * kBrickVox + vox_slot(s->x, s->y, s->z)), M.tau);
-    bool q = s->queued != 0;
-    if (fabsf(__fsub_rn(cur, s->last_tsdf)) > V.trig_tsdf) q = true;
-    s->last_tsdf = cur;
-    if (!V.trig_exact && V.near[s->blk] == frame) q = true;  // (ii) by the brick rule
-    if (moved && s->label == 2) q = true;
-    s->queued = q ? 1 : 0;
-  }
+// Blocks of kSelBlock ids in use.
+__device__ inline uint32_t sel_blocks(const PtView& V) {
+  return (V.C->count + kSelBlock - 1) / kSelBlock;
 }
 
-// Selection of the first `budget` queued ids: per-block counts, one scan, scatter.
-__global__ void __launch_bounds__(kSelBlock) k_pts_count(PtView V) {
+// Per block of ids: the triggers of a frame (trigger != 0), then the number of
+// queued points; the last CTA turns the counts into exclusive sums and takes
+// min(their total, budget) for the selection.
+__global__ void __launch_bounds__(kSelBlock) k_pts_trigger(MapView M, PtView V, uint32_t frame, int moved,
+                                                           int trigger, uint32_t budget) {
   __shared__ uint32_t part[kSelBlock / 32];
-  const uint32_t id = blockIdx.x * kSelBlock + threadIdx.x;
-  const bool q = id < V.C->count && V.st[id].queued;
-  const unsigned b = __ballot_sync(0xffffffffu, q);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = __popc(b);
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    uint32_t v = part[threadIdx.x];
-    v = __reduce_add_sync(0xffffffffu, v);
-    if (threadIdx.x == 0) V.blocksum[blockIdx.x] = v;
-  }
-}
-
-__global__ void __launch_bounds__(1024) k_pts_scan(PtView V, uint32_t nblocks, uint32_t budget) {
-  // exclusive scan of the block counts, 1024 at a time
-  __shared__ uint32_t buf[1024];
-  uint32_t carry = 0;
-  for (uint32_t b0 = 0; b0 < nblocks; b0 += 1024) {
-    const uint32_t b = b0 + threadIdx.x;
-    const uint32_t v = b < nblocks ? V.blocksum[b] : 0u;
-    buf[threadIdx.x] = v;
-    __syncthreads();
-    for (uint32_t off = 1; off < 1024; off <<= 1) {
-      const uint32_t t = threadIdx.x >= off ? buf[threadIdx.x - off] : 0u;
-      __syncthreads();
-      buf[threadIdx.x] += t;
-      __syncthreads();
+  const uint32_t count = V.C->count, nblocks = sel_blocks(V);
+  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+  for (uint32_t b = blockIdx.x; b < nblocks; b += gridDim.x) {
+    const uint32_t id = b * kSelBlock + threadIdx.x;
+    bool q = false;
+    if (id < count) {
+      PtState* s = V.st + id;
+      q = s->queued != 0;
+      if (trigger) {
+        const float cur =
+            tsdf_word(__ldcg(M.vox + (size_t)s->blk * kBrickVox + vox_slot(s->x, s->y, s->z)), M.tau);
+        if (fabsf(__fsub_rn(cur, s->last_tsdf)) > V.trig_tsdf) q = true;
+        s->last_tsdf = cur;
+        if (!V.trig_exact && V.near[s->blk] == frame) q = true;  // (ii) by the brick rule
+        if (moved && s->label == 2) q = true;
+        s->queued = q ? 1 : 0;
+      }
     }
-    if (b < nblocks) V.blocksum[b] = carry + buf[threadIdx.x] - v;
-    const uint32_t total = buf[1023];
+    const unsigned m = __ballot_sync(0xffffffffu, q);
+    if (lane == 0) part[wi] = __popc(m);
     __syncthreads();
-    carry += total;
+    if (wi == 0) {
+      const uint32_t v = __reduce_add_sync(0xffffffffu, part[lane]);
+      if (lane == 0) V.blocksum[b] = v;
+    }
+    __syncthreads();
+  }
+  if (!last_cta(&V.C->ended)) return;
+  uint32_t carry = 0;
+  for (uint32_t b0 = 0; b0 < nblocks; b0 += kSelBlock) {  // 1024 counts at a time
+    const uint32_t b = b0 + threadIdx.x;
+    const uint32_t own = b < nblocks ? __ldcg(V.blocksum + b) : 0u;
+    uint32_t v = own;
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t u = __shfl_up_sync(0xffffffffu, v, off);
+      if (lane >= off) v += u;
+    }
+    if (lane == 31) part[wi] = v;
+    __syncthreads();
+    if (wi == 0) {
+      uint32_t p = part[lane];
+      for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, p, off);
+        if (lane >= off) p += u;
+      }
+      part[lane] = p;
+    }
+    __syncthreads();
+    if (b < nblocks) V.blocksum[b] = carry + v - own + (wi ? part[wi - 1] : 0u);
+    carry += part[kSelBlock / 32 - 1];
+    __syncthreads();
   }
   if (threadIdx.x == 0) {
     V.C->nsel = min(carry, budget);
@@ -440,16 +680,21 @@ __global__ void __launch_bounds__(1024) k_pts_scan(PtView V, uint32_t nblocks, u
 
 __global__ void __launch_bounds__(kSelBlock) k_pts_select(PtView V, uint32_t budget) {
   __shared__ uint32_t part[kSelBlock / 32];
-  const uint32_t id = blockIdx.x * kSelBlock + threadIdx.x;
-  const bool q = id < V.C->count && V.st[id].queued;
+  const uint32_t count = V.C->count, nblocks = sel_blocks(V);
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-  const unsigned b = __ballot_sync(0xffffffffu, q);
-  if (lane == 0) part[wi] = __popc(b);
-  __syncthreads();
-  uint32_t before = 0;
-  for (int j = 0; j < wi; ++j) before += part[j];
-  const uint32_t rank = V.blocksum[blockIdx.x] + before + __popc(b & ((1u << lane) - 1u));
-  if (q && rank < budget) V.sel[rank] = id;
+  for (uint32_t blk = blockIdx.x; blk < nblocks; blk += gridDim.x) {
+    if (V.blocksum[blk] >= budget) return;  // uniform: the later blocks' sums are no smaller
+    const uint32_t id = blk * kSelBlock + threadIdx.x;
+    const bool q = id < count && V.st[id].queued;
+    const unsigned b = __ballot_sync(0xffffffffu, q);
+    if (lane == 0) part[wi] = __popc(b);
+    __syncthreads();
+    uint32_t before = 0;
+    for (int j = 0; j < wi; ++j) before += part[j];
+    const uint32_t rank = V.blocksum[blk] + before + __popc(b & ((1u << lane) - 1u));
+    if (q && rank < budget) V.sel[rank] = id;
+    __syncthreads();
+  }
 }
 
 // Candidate test of the layer: the normal filter and the observation-side
@@ -815,6 +1060,7 @@ PtView pt_view(af_ctx* ctx) {
   V.chgmask = ctx->d_pchgmask;
   V.hist = ctx->d_phist;
   V.samp = ctx->d_psamp;
+  V.drawn = ctx->d_pdrawn;
   V.trig_exact = c.trig_exact;
   V.trig_radius = c.trig_radius;
   V.trig_sample = c.trig_sample;
@@ -845,12 +1091,14 @@ PtView pt_view(af_ctx* ctx) {
   return V;
 }
 
-af_status select_and_eval(af_ctx* ctx, uint32_t budget, cudaStream_t s) {
+// Evaluates the first `budget` queued points; with `trigger` after a frame's
+// triggers (sensor moved: `moved`).
+af_status select_and_eval(af_ctx* ctx, uint32_t budget, int trigger, int moved, cudaStream_t s) {
   const PtView V = pt_view(ctx);
   const uint32_t nblocks = (ctx->pcfg.capacity + kSelBlock - 1) / kSelBlock;
-  k_pts_count<<<nblocks, kSelBlock, 0, s>>>(V);
-  k_pts_scan<<<1, 1024, 0, s>>>(V, nblocks, budget);
-  k_pts_select<<<nblocks, kSelBlock, 0, s>>>(V, budget);
+  const unsigned grid = std::min<uint32_t>(nblocks, (uint32_t)ctx->num_sms * 2);
+  k_pts_trigger<<<grid, kSelBlock, 0, s>>>(ctx->M, V, ctx->frame, moved, trigger, budget);
+  k_pts_select<<<grid, kSelBlock, 0, s>>>(V, budget);
   if (V.c2f_stride > 0) k_pts_snap<<<grid_cap(ctx->pcfg.capacity, 256, ctx->num_sms, 8), 256, 0, s>>>(V);
   k_pts_eval<<<(unsigned)ctx->num_sms * 8, 128, 0, s>>>(ctx->M, ctx->T, V);
   PT_CUDA(ctx, cudaGetLastError());
@@ -926,6 +1174,7 @@ extern "C" af_status af_points_enable(af_ctx* ctx, const af_points_config* cfg) 
     if (e == cudaSuccess) e = alloc((void**)&ctx->d_pchgmask, B * 16 * 4, 0);
     if (e == cudaSuccess) e = alloc((void**)&ctx->d_phist, af::kDrawBins * 4, 0);
     if (e == cudaSuccess) e = alloc((void**)&ctx->d_psamp, sizeof(af::PtSample), 0);
+    if (e == cudaSuccess) e = alloc((void**)&ctx->d_pdrawn, af::kDrawList * sizeof(af::PtDrawn), 0);
   }
   if (e == cudaSuccess) e = alloc((void**)&ctx->d_psel, P * 4, 0);
   if (e == cudaSuccess) e = alloc((void**)&ctx->d_pblock, nblocks * 4, 0);
@@ -981,18 +1230,24 @@ extern "C" af_status af_points_frame(af_ctx* ctx, const float* d_xyz, uint32_t n
   if (!exact)
     af::k_pts_near<<<af::grid_cap((size_t)M.pool_blocks * 27, 256, ctx->num_sms, 8), 256, 0, s>>>(M, V, frame);
   af::k_pts_create<<<af::grid_cap(ctx->cfg.max_returns, 256, ctx->num_sms, 8), 256, 0, s>>>(M, V);
-  af::k_pts_commit<<<1, 1, 0, s>>>(V);
   const float q[3] = {pose[3], pose[7], pose[11]};
   if (n > 0) af::k_pts_views<<<(n + 255) / 256, 256, 0, s>>>(M, ctx->d_ret, n, V, q[0], q[1], q[2], frame);
   if (exact) {  // trigger (ii): the changed voxels, their draw, the points near the drawn ones
-    const unsigned grid = (unsigned)ctx->num_sms * 4;
-    PT_CUDA(ctx, cudaMemsetAsync(ctx->d_psamp, 0, sizeof(af::PtSample), s));
-    af::k_pts_diff<<<grid, 512, 0, s>>>(M, V);
-    for (int pass = 0; pass < af::kDrawPasses; ++pass) {
-      af::k_pts_hist<<<grid, 512, 0, s>>>(M, V, pass);
-      af::k_pts_pick<<<1, 1024, 0, s>>>(V, pass);
+    const unsigned grid = (unsigned)ctx->num_sms * 2;
+    const bool list = ctx->pcfg.trig_sample > 0 && ctx->pcfg.trig_sample <= af::kDrawSample;
+    if (!list) PT_CUDA(ctx, cudaMemsetAsync(ctx->d_psamp, 0, sizeof(af::PtSample), s));
+    af::k_pts_diff<<<grid, 1024, 0, s>>>(M, V, list ? 1 : 0);
+    if (list) {
+      af::k_pts_collect<<<grid, 1024, 0, s>>>(M, V);
+      af::k_pts_scatter_list<<<(unsigned)ctx->num_sms, 256, 0, s>>>(M, V);
+    } else {
+      // every changed voxel (trig_sample 0): t without a pass over them
+      for (int pass = 0; pass < (ctx->pcfg.trig_sample ? af::kDrawPasses : 1); ++pass) {
+        if (ctx->pcfg.trig_sample) af::k_pts_hist<<<2 * grid, 512, 0, s>>>(M, V, pass);
+        af::k_pts_pick<<<1, 1024, 0, s>>>(V, pass);
+      }
+      af::k_pts_scatter<<<2 * grid, 512, 0, s>>>(M, V);
     }
-    af::k_pts_scatter<<<grid, 512, 0, s>>>(M, V);
   }
   // sensor motion since the motion trigger last fired
   int moved = 0;
@@ -1007,16 +1262,15 @@ extern "C" af_status af_points_frame(af_ctx* ctx, const float* d_xyz, uint32_t n
     std::memcpy(ctx->q_last, q, sizeof q);
     ctx->have_q_last = true;
   }
-  af::k_pts_trigger<<<af::grid_cap(ctx->pcfg.capacity, 256, ctx->num_sms, 8), 256, 0, s>>>(M, V, frame, moved);
   PT_CUDA(ctx, cudaGetLastError());
-  return af::select_and_eval(ctx, ctx->pcfg.budget, s);
+  return af::select_and_eval(ctx, ctx->pcfg.budget, 1, moved, s);
 }
 
 extern "C" af_status af_points_drain(af_ctx* ctx, uint32_t max_evals, void* stream) {
   if (!ctx) return af::pfail(ctx, AF_ERR_INVALID_ARG, "af_points_drain: NULL context");
   if (!ctx->pts_on) return af::pfail(ctx, AF_ERR_STATE, "af_points_drain: call af_points_enable first");
   if (!ctx->has_tool) return af::pfail(ctx, AF_ERR_STATE, "af_points_drain: call af_set_tool first");
-  return af::select_and_eval(ctx, max_evals, (cudaStream_t)stream);
+  return af::select_and_eval(ctx, max_evals, 0, 0, (cudaStream_t)stream);
 }
 
 extern "C" af_status af_points_stats(af_ctx* ctx, uint32_t* count, uint32_t* last_evals) {
