@@ -172,25 +172,46 @@ def _check(st: int, ctx=None):
         raise AfError(st, load().af_last_error(ctx).decode())
 
 
-def _np_ptr(a: np.ndarray):
-    return a.ctypes.data_as(C.c_void_p)
+def _np_ptr(a: np.ndarray) -> int:
+    """Address of an array's data; the caller keeps the array alive."""
+    return a.__array_interface__["data"][0]
 
 
-def _dev_ptr(t, dtype, shape_tail=None):
-    import torch
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
+def _pose(pose) -> np.ndarray:
+    return np.ascontiguousarray(pose, np.float32).reshape(16)
+
+
+_torch = None
+
+
+def _import_torch():
+    """torch, imported on the first call that needs it."""
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    return _torch
+
+
+# Marshalling is on the path of the smallest calls (a 500-return packet is
+# integrated and scored in 34 us of GPU time), so it makes no objects it can do
+# without: addresses are plain integers, the stream is read as its raw handle.
+
+def _dev_ptr(t, dtype, shape_tail=None) -> int:
+    if not isinstance(t, _import_torch().Tensor) or not t.is_cuda:
         raise TypeError("expected a CUDA tensor")
     if t.dtype != dtype or not t.is_contiguous():
         raise TypeError(f"expected a contiguous {dtype} tensor")
-    if shape_tail is not None and tuple(t.shape[1:]) != shape_tail:
+    if shape_tail is not None and t.shape[1:] != shape_tail:
         raise TypeError(f"expected shape (n, {shape_tail})")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream_ptr(stream):
-    import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+def _stream_ptr(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    torch = _import_torch()
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 @dataclass
@@ -311,20 +332,20 @@ class Map:
     def integrate_scan(self, xyz, pose, stream=None):
         """af_integrate_scan: xyz is an (n, 3) float32 CUDA tensor (sensor frame),
         pose a 4x4 world_from_sensor matrix."""
-        import torch
+        torch = _import_torch()
         n = int(xyz.shape[0])
-        p = _dev_ptr(xyz, torch.float32, (3,)) if n else C.c_void_p(0)
-        pose = np.ascontiguousarray(pose, np.float32).reshape(16)
+        p = _dev_ptr(xyz, torch.float32, (3,)) if n else None
+        pose = _pose(pose)
         _check(self._lib.af_integrate_scan(self._h, p, n, _np_ptr(pose), _stream_ptr(stream)),
                self._h)
 
     def integrate_scan_projective(self, xyz, pose, bins: int = 812, stream=None):
         """af_integrate_scan_projective: the projective ablation of Tab. 3 over
         a bins x bins octahedral range image."""
-        import torch
+        torch = _import_torch()
         n = int(xyz.shape[0])
-        p = _dev_ptr(xyz, torch.float32, (3,)) if n else C.c_void_p(0)
-        pose = np.ascontiguousarray(pose, np.float32).reshape(16)
+        p = _dev_ptr(xyz, torch.float32, (3,)) if n else None
+        pose = _pose(pose)
         _check(self._lib.af_integrate_scan_projective(self._h, p, n, _np_ptr(pose), int(bins),
                                                       _stream_ptr(stream)), self._h)
 
@@ -343,7 +364,7 @@ class Map:
 
     def score(self, pts, normals, label=None, best=None, stream=None):
         """af_score: returns (label uint8, best int16) CUDA tensors."""
-        import torch
+        torch = _import_torch()
         m = int(pts.shape[0])
         if label is None:
             label = torch.empty(m, dtype=torch.uint8, device=pts.device)
@@ -359,7 +380,7 @@ class Map:
     def frame_host(self, xyz: np.ndarray, pose, pts: np.ndarray, normals: np.ndarray,
                    label: np.ndarray, best: np.ndarray, stream=None):
         """af_frame_host: one frame from (ideally page-locked) host arrays."""
-        pose = np.ascontiguousarray(pose, np.float32).reshape(16)
+        pose = _pose(pose)
         _check(self._lib.af_frame_host(self._h, _np_ptr(xyz), len(xyz), _np_ptr(pose),
                                        _np_ptr(pts), _np_ptr(normals), len(pts),
                                        _np_ptr(label), _np_ptr(best), _stream_ptr(stream)),
@@ -411,10 +432,10 @@ class Map:
 
     def points_frame(self, xyz, pose, stream=None):
         """af_points_frame: integrate a scan and update the point layer."""
-        import torch
+        torch = _import_torch()
         n = int(xyz.shape[0])
-        p = _dev_ptr(xyz, torch.float32, (3,)) if n else C.c_void_p(0)
-        pose = np.ascontiguousarray(pose, np.float32).reshape(16)
+        p = _dev_ptr(xyz, torch.float32, (3,)) if n else None
+        pose = _pose(pose)
         _check(self._lib.af_points_frame(self._h, p, n, _np_ptr(pose), _stream_ptr(stream)),
                self._h)
 
@@ -431,10 +452,10 @@ class Map:
     def points_export(self) -> dict:
         """Every point in id order: ijk, normal, label, score, best, a, queued, nviews."""
         n, _ = self.points_stats()
-        out = dict(ijk=np.zeros((n, 3), np.int32), normal=np.zeros((n, 3), np.float32),
-                   label=np.zeros(n, np.uint8), score=np.zeros(n, np.int16),
-                   best=np.zeros(n, np.int16), a=np.zeros(n, np.float32),
-                   queued=np.zeros(n, np.uint8), nviews=np.zeros(n, np.int32))
+        out = dict(ijk=np.empty((n, 3), np.int32), normal=np.empty((n, 3), np.float32),
+                   label=np.empty(n, np.uint8), score=np.empty(n, np.int16),
+                   best=np.empty(n, np.int16), a=np.empty(n, np.float32),
+                   queued=np.empty(n, np.uint8), nviews=np.empty(n, np.int32))
         cnt = C.c_uint32()
         _check(self._lib.af_points_export(self._h, n, *(_np_ptr(out[k]) for k in
                                                         ("ijk", "normal", "label", "score", "best",
@@ -447,14 +468,14 @@ class Map:
     def soft_seed(self, normals, table, out=None, stream=None):
         """af_soft_seed: (m*K, 3) base directions, the K rows of `table`
         (K x 3, around +z) rotated into each normal's tangent frame."""
-        import torch
+        torch = _import_torch()
         m = int(normals.shape[0])
         table = np.ascontiguousarray(table, np.float32).reshape(-1, 3)
         u0 = out if out is not None else \
             torch.empty((m * len(table), 3), dtype=torch.float32, device=normals.device)
         _check(self._lib.af_soft_seed(self._h, _dev_ptr(normals, torch.float32, (3,)) if m
-                                      else C.c_void_p(0), m, _np_ptr(table), len(table),
-                                      _dev_ptr(u0, torch.float32, (3,)) if m else C.c_void_p(0),
+                                      else None, m, _np_ptr(table), len(table),
+                                      _dev_ptr(u0, torch.float32, (3,)) if m else None,
                                       _stream_ptr(stream)), self._h)
         return u0
 
@@ -466,11 +487,11 @@ class Map:
         """af_soft_start: (m, 3) start directions of refinement -- the best
         direction of each ACCESSIBLE point of af_score's output, NaN for the
         others."""
-        import torch
+        torch = _import_torch()
         m = int(label.shape[0])
         u0 = out if out is not None else \
             torch.empty((m, 3), dtype=torch.float32, device=label.device)
-        z = C.c_void_p(0)
+        z = None
         _check(self._lib.af_soft_start(self._h, _dev_ptr(label, torch.uint8) if m else z,
                                        _dev_ptr(best, torch.int16) if m else z, m,
                                        _dev_ptr(u0, torch.float32, (3,)) if m else z,
@@ -478,7 +499,7 @@ class Map:
         return u0
 
     def _pair_ptrs(self, pts, u0, alpha, beta, h, per_point):
-        import torch
+        torch = _import_torch()
         n = int(u0.shape[0])
         if per_point < 1 or int(pts.shape[0]) * per_point < n:
             raise ValueError("need per_point >= 1 and a point for every pair")
@@ -486,7 +507,7 @@ class Map:
             if t.shape != (n,):
                 raise ValueError("alpha, beta and h need one value per pair")
         if n == 0:
-            return n, [C.c_void_p(0)] * 5
+            return n, [None] * 5
         return n, [_dev_ptr(pts, torch.float32, (3,)), _dev_ptr(u0, torch.float32, (3,)),
                    _dev_ptr(alpha, torch.float32), _dev_ptr(beta, torch.float32),
                    _dev_ptr(h, torch.float32)]
@@ -495,24 +516,29 @@ class Map:
                            cmin=None, stream=None):
         """af_soft_clearance: C of every pair (no autograd); `cmin`, if
         given, receives the hard clearance."""
-        import torch
+        torch = _import_torch()
         n, ptr = self._pair_ptrs(pts, u0, alpha, beta, h, per_point)
         c = torch.empty(n, dtype=torch.float32, device=u0.device) if out is None else out
         _check(self._lib.af_soft_clearance(self._h, ptr[0], per_point, *ptr[1:], n, tau_s,
-                                           _dev_ptr(c, torch.float32) if n else C.c_void_p(0),
+                                           _dev_ptr(c, torch.float32) if n else None,
                                            _dev_ptr(cmin, torch.float32) if (cmin is not None
                                                                             and n)
-                                           else C.c_void_p(0), _stream_ptr(stream)), self._h)
+                                           else None, _stream_ptr(stream)), self._h)
         return c
 
     def soft_clearance_adjoint(self, pts, u0, alpha, beta, h, per_point, tau_s=TAU_S,
                                grad_c=None, stream=None):
         """af_soft_clearance_adjoint: (C, g dC/dalpha, g dC/dbeta, g dC/dh)."""
-        import torch
+        c = _import_torch().empty(int(u0.shape[0]), dtype=_torch.float32, device=u0.device)
+        return (c, *self._adjoint(pts, u0, alpha, beta, h, per_point, tau_s, grad_c, c, stream))
+
+    def _adjoint(self, pts, u0, alpha, beta, h, per_point, tau_s, grad_c, c, stream=None):
+        """The three gradients; C goes to `c` unless it is None."""
+        torch = _import_torch()
         n, ptr = self._pair_ptrs(pts, u0, alpha, beta, h, per_point)
-        out = [torch.empty(n, dtype=torch.float32, device=u0.device) for _ in range(4)]
-        op = [_dev_ptr(t, torch.float32) if n else C.c_void_p(0) for t in out]
-        gp = _dev_ptr(grad_c, torch.float32) if (grad_c is not None and n) else C.c_void_p(0)
+        out = [torch.empty(n, dtype=torch.float32, device=u0.device) for _ in range(3)]
+        op = [_dev_ptr(t, torch.float32) if (t is not None and n) else None for t in (c, *out)]
+        gp = _dev_ptr(grad_c, torch.float32) if (grad_c is not None and n) else None
         _check(self._lib.af_soft_clearance_adjoint(self._h, ptr[0], per_point, *ptr[1:], n,
                                                    tau_s, gp, *op, _stream_ptr(stream)),
                self._h)
@@ -526,13 +552,13 @@ class Map:
                     lr_h=0.005, h_max=0.05, tau_s=TAU_S, out=None, stream=None):
         """af_soft_refine: `steps` ascent steps on every pair in one launch;
         alpha, beta, h are updated in place. Returns (C, hard clearance)."""
-        import torch
+        torch = _import_torch()
         n, ptr = self._pair_ptrs(pts, u0, alpha, beta, h, per_point)
         R = _Refine(steps, lr_dir, lr_h, h_max)
         c, cmin = out if out is not None else \
             (torch.empty(n, dtype=torch.float32, device=u0.device),
              torch.empty(n, dtype=torch.float32, device=u0.device))
-        op = [_dev_ptr(t, torch.float32) if n else C.c_void_p(0) for t in (c, cmin)]
+        op = [_dev_ptr(t, torch.float32) if n else None for t in (c, cmin)]
         _check(self._lib.af_soft_refine(self._h, ptr[0], per_point, *ptr[1:], n, tau_s,
                                         C.byref(R), *op, _stream_ptr(stream)), self._h)
         return c, cmin
@@ -540,7 +566,7 @@ class Map:
     def soft_best(self, c, per_point, u0=None, out=None, stream=None):
         """af_soft_best: per point (index of its largest C, that C, and --
         with u0 -- that pair's base direction)."""
-        import torch
+        torch = _import_torch()
         n = int(c.shape[0])
         npts = (n + per_point - 1) // per_point
         if out is not None:
@@ -550,7 +576,7 @@ class Map:
             bc = torch.empty(npts, dtype=torch.float32, device=c.device)
             bu = torch.empty((npts, 3), dtype=torch.float32, device=c.device) \
                 if u0 is not None else None
-        z = C.c_void_p(0)
+        z = None
         _check(self._lib.af_soft_best(self._h, _dev_ptr(c, torch.float32) if n else z, n,
                                       per_point, _dev_ptr(u0, torch.float32, (3,))
                                       if (u0 is not None and n) else z,
@@ -563,7 +589,7 @@ class Map:
 
 
 def _soft_function():
-    import torch
+    torch = _import_torch()
 
     class SoftClearance(torch.autograd.Function):
         """C = soft clearance of (point, direction) pairs; backward runs the
@@ -574,15 +600,13 @@ def _soft_function():
         def forward(ctx, m, pts, u0, alpha, beta, h, per_point, tau_s):
             ctx.save_for_backward(pts, u0, alpha, beta, h)
             ctx.m, ctx.per_point, ctx.tau_s = m, per_point, tau_s
-            return m.soft_clearance_raw(pts, u0, alpha.detach(), beta.detach(), h.detach(),
-                                        per_point, tau_s)
+            return m.soft_clearance_raw(pts, u0, alpha, beta, h, per_point, tau_s)
 
         @staticmethod
         def backward(ctx, grad_c):
             pts, u0, alpha, beta, h = ctx.saved_tensors
-            _, ga, gb, gh = ctx.m.soft_clearance_adjoint(
-                pts, u0, alpha.detach(), beta.detach(), h.detach(), ctx.per_point, ctx.tau_s,
-                grad_c.contiguous())
+            ga, gb, gh = ctx.m._adjoint(pts, u0, alpha, beta, h, ctx.per_point, ctx.tau_s,
+                                        grad_c.contiguous(), None)
             return (None, None, None, ga if ctx.needs_input_grad[3] else None,
                     gb if ctx.needs_input_grad[4] else None,
                     gh if ctx.needs_input_grad[5] else None, None, None)
@@ -658,12 +682,12 @@ def integrate_scan_noalloc(cfg: MapConfig, xyz, pose, box_min, box_dim, vox, fla
     (vox: int64 CUDA tensor of (S << 20) | w words, flags: uint8 CUDA tensor;
     both box_dim[0] * box_dim[1] * box_dim[2] long). The library allocates
     nothing for this call, for callers that cannot allocate device memory."""
-    import torch
+    torch = _import_torch()
     lib = load()
     cc = cfg._c()
     n = int(xyz.shape[0])
-    p = _dev_ptr(xyz, torch.float32, (3,)) if n else C.c_void_p(0)
-    pose = np.ascontiguousarray(pose, np.float32).reshape(16)
+    p = _dev_ptr(xyz, torch.float32, (3,)) if n else None
+    pose = _pose(pose)
     bmin = np.ascontiguousarray(box_min, np.int32).reshape(3)
     bdim = np.ascontiguousarray(box_dim, np.uint32).reshape(3)
     count = int(np.prod(bdim.astype(np.int64)))
@@ -701,19 +725,19 @@ class Batch:
         """items[s] = (xyz, pose, pts, normals, label, best) for scene s: CUDA
         tensors as for Map.integrate_scan / Map.score (pts may hold 0 rows).
         The tensors must stay alive until the tick has run."""
-        import torch
+        torch = _import_torch()
         arr = (_BatchItem * len(self.maps))()
         for s, (xyz, pose, pts, nrm, lab, best) in enumerate(items):
             it = arr[s]
             it.n = int(xyz.shape[0])
-            it.d_xyz = _dev_ptr(xyz, torch.float32, (3,)).value if it.n else None
+            it.d_xyz = _dev_ptr(xyz, torch.float32, (3,)) if it.n else None
             it.pose[:] = [float(x) for x in np.asarray(pose, np.float32).reshape(16)]
             it.m = int(pts.shape[0])
             if it.m:
-                it.d_pts = _dev_ptr(pts, torch.float32, (3,)).value
-                it.d_normals = _dev_ptr(nrm, torch.float32, (3,)).value
-                it.d_label = _dev_ptr(lab, torch.uint8).value
-                it.d_best = _dev_ptr(best, torch.int16).value
+                it.d_pts = _dev_ptr(pts, torch.float32, (3,))
+                it.d_normals = _dev_ptr(nrm, torch.float32, (3,))
+                it.d_label = _dev_ptr(lab, torch.uint8)
+                it.d_best = _dev_ptr(best, torch.int16)
         _check(self._lib.af_batch_tick(self._h, arr, _stream_ptr(stream)))
 
     def set_tuning(self, returns_per_tile: int, warps_per_cta: int):
