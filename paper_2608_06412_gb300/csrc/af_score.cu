@@ -4,12 +4,12 @@
 // The lanes first evaluate the normal filter for
 // 32 directions at a time (ballot -> candidate mask), then the arm samples of
 // each candidate (three single-bit lookups: occupied or unknown blocks). The
-// arm-clear candidates are taken four at a time in index order:
+// arm-clear candidates are taken four at a time (kSide) in index order:
 //   * tool kernel: 8 lanes per direction fetch the kernel's entries (the same
 //     32 voxels of four rows in one or two 16-byte loads), AND with the masks
 //     and __popc; the count saturates at the score to beat, so it stops as
 //     soon as the direction can no longer improve the point;
-//   * corridor: the whole warp, two entries per lane per step, any set bit
+//   * corridor: the whole warp, one entry per lane per step, any set bit
 //     blocks (__any_sync early exit).
 // The best direction is the lowest-index minimum; a score of 0 ends the
 // point. Every early exit returns exactly what a full evaluation of every
@@ -109,10 +109,9 @@ __device__ void score_point(const MapView& M, const ToolView& T, const float* __
   }
 }
 
-// Threads per SM the scorers are built for: 40 warps at 48 registers. A lane's
-// two entries in flight (16-byte loads and masks) want 60 registers; fewer warps
-// hide less latency (32 warps: 66 against 62 us per pine frame), more spill (48
-// warps at 40 registers: 66 us).
+// Threads per SM the scorers are built for: 40 warps at 48 registers. Fewer warps
+// hide less latency, more spill: 32 / 40 / 48 / 64 warps take 55.9 / 52.9 / 54.7 /
+// 61.8 us per pine frame, 1.50 / 1.34 / 1.38 / 1.48 ms on the 1 cm map.
 constexpr int kScoreThreads = 1280;
 
 template <int WARPS, bool SPLIT>

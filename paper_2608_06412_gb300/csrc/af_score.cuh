@@ -17,10 +17,12 @@
 // the 1 m corridor at 2 cm). Per direction of the 4 cm tool a run each row takes
 // 32 tool and 143 corridor loads, quads about 12 and 47: a tool fits 8 or 16
 // lanes, so four directions are counted side by side, and a corridor is walked
-// in one or two steps instead of five. Against runs with their tables staged in
-// shared memory: 72.5 -> 61 us per pine frame (12k points, 128 directions), 489
-// -> 328 us for 40k points of three pines with the 6 cm tool and
-// 256 directions, 2.47 -> 1.47 ms for 83k points of a 1 cm map with 512.
+// in two steps instead of five. Against runs with their tables staged in
+// shared memory: 72.5 -> 53 us per pine frame (12k points, 128 directions), 489
+// -> 282 us for 40k points of three pines with the 6 cm tool and 256 directions,
+// 2.5 -> 1.34 ms for 83k points of a 1 cm map with 512. The latter two are bound
+// by L1 wavefronts (80% of their peak on the 1 cm map: a gather of 16-byte words
+// takes a wavefront per lane), the pine frame by the chain and its tail.
 //
 // A point whose whole kernel reach lies inside the map box takes the FAST path,
 // which checks no bound; otherwise words outside the box read as zero: nothing
@@ -111,28 +113,36 @@ __device__ __forceinline__ int popc4(uint4 b) {
   return __popc(b.x) + __popc(b.y) + __popc(b.z) + __popc(b.w);
 }
 
-// Occupied tool voxels, saturated at `sat`, of up to four directions side by
-// side: the 8 lanes of group k (lanes 8k .. 8k + 7) count the direction of table
-// entry `d` (equal over the group; none unless `valid`), two entries per lane per step, and all get
-// its count. A group that has reached `sat` stops loading.
+// Lanes that count one direction: kSide directions are counted side by side. With
+// 4 / 8 / 16 lanes 53.2 / 52.9 / 56.9 us per pine frame, 1.39 / 1.34 / 1.48 ms on
+// the 1 cm map.
+constexpr int kDirLanes = 8;
+constexpr int kSide = 32 / kDirLanes;
+
+// Occupied tool voxels, saturated at `sat`, of up to kSide directions side by
+// side: the lanes of group k (lanes kDirLanes k on) count the direction of table
+// entry `d` (equal over the group; none unless `valid`), one entry per lane per
+// step, and all get its count. A group that has reached `sat` stops loading.
+// One entry per lane, not two: entries come nearest first and most directions
+// are decided by the first few, so wider steps load words that nobody needs
+// (61 -> 52 us per pine frame together with the corridor's).
 template <bool FAST>
-__device__ inline int tool_count4(const MapView& M, const ToolView& T, bool valid, int4 d, const Pt& P,
+__device__ inline int tool_counts(const MapView& M, const ToolView& T, bool valid, int4 d, const Pt& P,
                                   int sat, int lane) {
   DirRows D = dir_rows(M, P, d);
   if (!valid) D.nt = 0;
-  const int hl = lane & 7;
-  int total = 0;
-  bool more = D.nt > 0;
-  for (int b = hl; __any_sync(0xffffffffu, more); b += 16) {
+  int total = 0, b = lane & (kDirLanes - 1), left = D.nt;
+  while (__any_sync(0xffffffffu, left > 0)) {
     int c = 0;
-    uint4 m;
-    if (more && b < D.nt) c = popc4(quad_bits<FAST>(M, T, D, D.view, D.t0 + b, &m));
-    if (more && b + 8 < D.nt) c += popc4(quad_bits<FAST>(M, T, D, D.view, D.t0 + b + 8, &m));
-    c += __shfl_xor_sync(0xffffffffu, c, 4);
-    c += __shfl_xor_sync(0xffffffffu, c, 2);
-    c += __shfl_xor_sync(0xffffffffu, c, 1);
+    if (left > 0 && b < D.nt) {
+      uint4 m;
+      c = popc4(quad_bits<FAST>(M, T, D, D.view, D.t0 + b, &m));
+    }
+#pragma unroll
+    for (int off = kDirLanes / 2; off; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
     total += c;
-    more = b - hl + 16 < D.nt && total < sat;
+    b += kDirLanes;
+    left = total < sat ? left - kDirLanes : 0;
   }
   return min(total, sat);
 }
@@ -153,22 +163,21 @@ __device__ inline int tool_count(const MapView& M, const ToolView& T, int g, con
 }
 
 // Corridor of the direction of table entry d: any occupied voxel (strict: or
-// unknown) blocks. The whole warp, two entries per lane per step. Strict
-// corridors run along x, the known view's rows.
+// unknown) blocks. The whole warp, one entry per lane per step (most blocked
+// corridors are so by their nearest entries). Strict corridors run along x, the
+// known view's rows.
 template <bool FAST>
 __device__ inline bool corridor_blocked(const MapView& M, const ToolView& T, int4 d, const Pt& P,
                                         int lane) {
   const DirRows D = dir_rows(M, P, d, T.strict != 0);
-  for (int b = lane; b - lane < D.nc; b += 64) {
+  for (int b = lane; b - lane < D.nc; b += 32) {
     bool h = false;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      if (b + 32 * k >= D.nc) continue;
+    if (b < D.nc) {
       uint4 m;
-      const uint4 o = quad_bits<FAST>(M, T, D, D.view, D.c0 + b + 32 * k, &m);
-      h = h || (o.x | o.y | o.z | o.w) != 0u;
+      const uint4 o = quad_bits<FAST>(M, T, D, D.view, D.c0 + b, &m);
+      h = (o.x | o.y | o.z | o.w) != 0u;
       if (T.strict) {
-        const uint4 n = quad_bits<FAST>(M, T, D, M.known, D.c0 + b + 32 * k, &m);
+        const uint4 n = quad_bits<FAST>(M, T, D, M.known, D.c0 + b, &m);
         h = h || ((n.x ^ m.x) | (n.y ^ m.y) | (n.z ^ m.z) | (n.w ^ m.w)) != 0u;
       }
     }
@@ -246,7 +255,7 @@ __device__ __forceinline__ int4 shfl4(int4 v, int from) {
 // overlaps the screen's): if it says no, (-1, -1) is returned.
 //
 // The arm screen takes 32 directions at a time. The arm-clear ones are then
-// counted four at a time, all against the score to beat before the four, and
+// counted kSide at a time, all against the score to beat before them, and
 // decided in index order: a count that reaches that score cannot beat any later
 // one, so the result is the sequential one. A score of 0 ends the search.
 template <bool FAST, class Cand, class Gate = NoGate>
@@ -263,18 +272,23 @@ __device__ inline int2 best_direction(const MapView& M, const ToolView& T, const
     unsigned rest = __ballot_sync(0xffffffffu, cand && arm_clear<FAST>(M, T, gb + lane, P));
     if (gb == 0 && !gate()) return make_int2(-1, -1);
     while (rest) {
-      // the next four arm-clear directions, one per group of 8 lanes
-      const unsigned r1 = rest & (rest - 1u), r2 = r1 & (r1 - 1u), r3 = r2 & (r2 - 1u);
-      const unsigned mine = lane < 16 ? (lane < 8 ? rest : r1) : (lane < 24 ? r2 : r3);
+      // the next kSide arm-clear directions, one per group of lanes
+      unsigned mine = rest;
+#pragma unroll
+      for (int k = 1; k < kSide; ++k) {
+        if (lane >= k * kDirLanes) mine &= mine - 1u;
+        rest &= rest - 1u;
+      }
+      rest &= rest - 1u;
       const int at = mine ? __ffs(mine) - 1 : 0;
-      const int c = tool_count4<FAST>(M, T, mine != 0u, shfl4(dt, at), P, min(bscore, nc), lane);
-      unsigned todo = __ballot_sync(0xffffffffu, mine != 0u && (best < 0 || c < bscore)) & 0x01010101u;
-      rest = r3 & (r3 - 1u);
+      const int c = tool_counts<FAST>(M, T, mine != 0u, shfl4(dt, at), P, min(bscore, nc), lane);
+      unsigned todo = __ballot_sync(0xffffffffu, mine != 0u && (best < 0 || c < bscore) &&
+                                                     (lane & (kDirLanes - 1)) == 0);
       while (todo) {
         const int from = __ffs(todo) - 1;
         todo &= todo - 1u;
         const int k = __shfl_sync(0xffffffffu, at, from), ck = __shfl_sync(0xffffffffu, c, from);
-        if (best >= 0 && ck >= bscore) continue;  // beaten by one of the four before it
+        if (best >= 0 && ck >= bscore) continue;  // beaten by one before it
         if (corridor_blocked<FAST>(M, T, shfl4(dt, k), P, lane)) continue;
         bscore = ck;
         best = gb + k;
