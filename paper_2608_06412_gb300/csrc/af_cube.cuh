@@ -12,12 +12,9 @@
 
 namespace af {
 
-// Approximate square root (MUFU reciprocal square root), relative error well
-// below 2^-20 for the normal arguments it is used on. Only ever used to take
-// a decision that the exact result is certain to agree with (margins of
-// 2^-16 relative); near any threshold the exact IEEE operation decides.
-__device__ inline float sqrt_approx(float x) { return x * rsqrtf(x); }
-
+// Relative margin of decisions taken from approximate values: the reciprocal
+// square root and two products are within 2^-20 for the normal arguments they
+// are used on.
 constexpr float kMargin = 1.52587890625e-05f;  // 2^-16
 
 // The exact cone decision, RN(dot / RN(RN(sqrt(aa)) range)) > cone, out of
@@ -37,17 +34,26 @@ struct CubeShape {
   static constexpr int MR = W / 2;
 };
 
-// What a pair reads of its return: range |p - q|, RN(|p - q|^2), RN(1 / range)
-// (for the approximate cone test), valid flag.
+// Returns per CTA ("tile") of one scan's integration, by the scan's size. A tile's
+// setup (brick table or box offsets, per-axis terms) is spread over its pairs, so
+// larger tiles cost less a return as long as enough CTAs are left to overlap: with
+// tiles of 8 / 12 / 16 the map's kernel takes 26.9 / 25.5 / 26.7 us for 20,000
+// returns and 68.5 / 63.9 / 60.8 us for 60,000, the box's 27.6 / 27.0 / 26.3 us for
+// 20,000. Small scans take small tiles, so that every SM has one.
+constexpr int kTileSmall = 4, kTile = 12, kTileLarge = 16;
+constexpr uint32_t kTileSmallBelow = 4000, kTileLargeFrom = 40000;
+
+// What a pair reads of its return: x = range |p - q|, y = RN(1 / range) (for the
+// approximate cone test), w = valid flag.
 __device__ inline float4 return_record(float4 p, float q0, float q1, float q2) {
-  float bb = 0.f, range = 0.f, ir = 0.f;
+  float range = 0.f, ir = 0.f;
   if (p.w != 0.f) {
     const float b[3] = {__fsub_rn(p.x, q0), __fsub_rn(p.y, q1), __fsub_rn(p.z, q2)};
-    bb = __fadd_rn(__fadd_rn(__fmul_rn(b[0], b[0]), __fmul_rn(b[1], b[1])), __fmul_rn(b[2], b[2]));
-    range = __fsqrt_rn(bb);
+    range = __fsqrt_rn(
+        __fadd_rn(__fadd_rn(__fmul_rn(b[0], b[0]), __fmul_rn(b[1], b[1])), __fmul_rn(b[2], b[2])));
     ir = __frcp_rn(range);
   }
-  return make_float4(range, bb, ir, p.w);
+  return make_float4(range, ir, 0.f, p.w);
 }
 
 // The rounded terms of one axis of the three sums a pair needs, (x - p)^2,
@@ -65,7 +71,7 @@ __device__ inline float4 axis_terms(const MapView& M, float pa, float qa, int i)
 __device__ __forceinline__ bool pair_contribution(const MapView& M, const float4& tx, const float4& ty,
                                                   const float4& tz, const float4& pr, long long* dq) {
   const float tau = M.tau, cone = M.cone_cos;
-  const float range = pr.x, bb = pr.y, ir = pr.z;
+  const float range = pr.x, ir = pr.y;
   const float aa = __fadd_rn(__fadd_rn(tx.x, ty.x), tz.x);
   // behind-surface cone: theta between x - p and p - q; excluded iff
   // RN(dot / RN(RN(sqrt(aa)) * range)) > cone
@@ -83,18 +89,13 @@ __device__ __forceinline__ bool pair_contribution(const MapView& M, const float4
       if (!decided && cone_excludes_exact(dot, aa, range, cone)) return false;
     }
   }
-  // d = |p - q| - |x - q|, clamped to [0, tau] ([-tau, tau] in the ablation)
+  // d = |p - q| - |x - q|, clamped to [0, tau] ([-tau, tau] in the ablation). The
+  // exact root for every pair: a warp's voxels lie on both sides of the surface
+  // and beyond tau, so screens that spared some lanes the root (|x - q| >= |p - q|,
+  // or an approximate root beyond tau) cost every warp their branches as well
+  // (31.9 against 26.7 us per pine frame, 84.8 against 68.0 us for 60,000 returns).
   const float cc = __fadd_rn(__fadd_rn(tx.z, ty.z), tz.z);
-  float d;
-  if (cc >= bb && !M.clamp_signed) {
-    d = 0.f;  // |x - q| >= |p - q|: the rounded difference is <= 0
-  } else if (cc > 1e-20f && range - sqrt_approx(cc) > tau + range * kMargin) {
-    d = tau;  // the exact difference exceeds tau
-  } else {
-    d = __fsub_rn(range, __fsqrt_rn(cc));
-    d = d < M.dlo ? M.dlo : d;
-    d = d > tau ? tau : d;
-  }
+  const float d = fminf(fmaxf(__fsub_rn(range, __fsqrt_rn(cc)), M.dlo), tau);
   // |d| <= tau <= 1 m, so |d 2^20| < 2^31: the 32-bit conversion rounds
   // exactly as a 64-bit one would, and stays off the FP64 pipe
   *dq = (long long)__float2int_rn(__fmul_rn(d, kScale));

@@ -8,7 +8,7 @@
 //              so one probe per distinct key per warp reaches L2. The pool
 //              index of each cube brick goes into a per-return brick table,
 //              and the brick is marked dirty.
-//  k_integrate one CTA per tile of 8 returns, one thread per cube offset: the
+//  k_integrate one CTA per tile of returns, one thread per cube offset: the
 //              tile's brick tables are loaded once (bricks created by this
 //              scan are looked up here), and the per-axis terms of every
 //              return's sums (squares, products, brick / slot codes) are
@@ -189,8 +189,7 @@ __device__ void integrate_tile(const MapView& M, const float4* __restrict__ ret,
   using S = CubeShape<W>;
   constexpr int C = S::C, NT = S::NT, OPT = S::OPT, BA = S::BA, NB = S::NB, MR = S::MR;
   __shared__ float4 s_p[T];        // p, valid flag
-  // what the pair loop reads of a return, in one record: range |p - q|,
-  // RN(|p - q|^2), RN(1 / range) (for the approximate cone test), valid flag
+  // what the pair loop reads of a return, in one record (return_record)
   __shared__ float4 s_pr[T];
   __shared__ uint32_t s_blk[T][NB];
   // Per return, axis and cube offset k (voxel rel + k - MR on that axis),
@@ -305,18 +304,15 @@ __device__ void integrate_tile(const MapView& M, const float4* __restrict__ ret,
   }
 }
 
-// Tiles of 8 returns for the single-map path, one CTA each (measured against
-// 12, 16, 20, 26 and 32 on the pine stream, and against persistent CTAs that
-// each take an equal share of the returns: slower, 40.9 against 35.4 us).
-constexpr int kTile = 8;
-
-template <int W>
+// The single-map path: one CTA per tile (against persistent CTAs that each take
+// an equal share of the returns: slower, 40.9 against 35.4 us).
+template <int W, int T>
 __global__ void __launch_bounds__(CubeShape<W>::NT) k_integrate(MapView M,
                                                                 const float4* __restrict__ ret,
                                                                 uint32_t n, float q0, float q1,
                                                                 float q2, uint32_t frame) {
-  const uint32_t r0 = blockIdx.x * kTile;
-  integrate_tile<W, kTile>(M, ret, r0, min(r0 + kTile, n), q0, q1, q2, frame);
+  const uint32_t r0 = blockIdx.x * T;
+  integrate_tile<W, T>(M, ret, r0, min(r0 + T, n), q0, q1, q2, frame);
 }
 
 // Weight cap and bit view of one dirty brick; called by a CTA of NT threads
@@ -437,15 +433,20 @@ cudaError_t launch_alloc(const MapView& M, const float* d_xyz, uint32_t n, const
 cudaError_t launch_cube(const MapView& M, uint32_t n, const float pose[16], const float4* d_ret,
                         uint32_t frame, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
-  const unsigned grid = (n + kTile - 1) / kTile;
+  const int T = n < kTileSmallBelow ? kTileSmall : (n < kTileLargeFrom ? kTile : kTileLarge);
+  const unsigned grid = (n + T - 1) / T;
+#define AF_TILE(W, TT) \
+  k_integrate<W, TT><<<grid, CubeShape<W>::NT, 0, stream>>>(M, d_ret, n, pose[3], pose[7], pose[11], frame)
   switch (2 * M.m + 1) {
-#define AF_CASE(W)                                                                          \
-  case W:                                                                                   \
-    k_integrate<W><<<grid, CubeShape<W>::NT, 0, stream>>>(M, d_ret, n, pose[3], pose[7],   \
-                                                          pose[11], frame);                 \
+#define AF_CASE(W)                                   \
+  case W:                                            \
+    if (T == kTileSmall) AF_TILE(W, kTileSmall);     \
+    else if (T == kTile) AF_TILE(W, kTile);          \
+    else AF_TILE(W, kTileLarge);                     \
     break;
     AF_CASE(3) AF_CASE(5) AF_CASE(7) AF_CASE(9) AF_CASE(11) AF_CASE(13) AF_CASE(15) AF_CASE(17)
 #undef AF_CASE
+#undef AF_TILE
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -86,10 +86,6 @@ __device__ inline bool box_index(const Box& B, int x, int y, int z, size_t* at) 
   return true;
 }
 
-// Returns per CTA of the two kernels below: the per-axis work of a return is
-// done once for its (2m+1)^3 cube voxels.
-constexpr int kBoxTile = 8;
-
 // Box offset of the coordinate with domain-relative index j on axis ax (the
 // three axes' offsets add up to the voxel's element), or -1 outside the box.
 __device__ inline long long box_offset(const Box& B, int ax, int j) {
@@ -99,28 +95,28 @@ __device__ inline long long box_offset(const Box& B, int ax, int j) {
                  : (ax == 1 ? (long long)j * B.dim[0] : (long long)j * ((long long)B.dim[0] * B.dim[1]));
 }
 
-// One CTA per kBoxTile returns, one thread per cube offset: the returns are
+// One CTA per T returns, one thread per cube offset: the returns are
 // transformed and their per-axis terms and box offsets computed once into
 // shared memory, then each thread walks the returns for its offset, the same
 // arithmetic as the hashed path (af_cube.cuh), one 64-bit atomic add per pair;
 // the cleared-band marks follow. The world positions go to `scratch` for
-// k_box_finalize. Issue-bound like k_integrate: 32.5 us per pine frame; with one
+// k_box_finalize. Issue-bound like k_integrate: 26.3 us per pine frame; with one
 // thread per (return, offset) that did all of a pair's work, 64-bit divisions
 // included, for itself, 73 us and a launch for the transform.
-template <int W>
+template <int W, int T>
 __global__ void __launch_bounds__(CubeShape<W>::NT) k_box_integrate(MapView M,
                                                                     const float* __restrict__ xyz,
                                                                     uint32_t n, Pose P,
                                                                     float4* __restrict__ scratch,
                                                                     Box B) {
   using S = CubeShape<W>;
-  __shared__ float4 s_p[kBoxTile], s_pr[kBoxTile];
-  __shared__ float4 s_term[kBoxTile][3][W];
-  __shared__ long long s_off[kBoxTile][3][W];
+  __shared__ float4 s_p[T], s_pr[T];
+  __shared__ float4 s_term[T][3][W];
+  __shared__ long long s_off[T][3][W];
   const int tid = threadIdx.x;
-  const uint32_t r0 = blockIdx.x * kBoxTile;
+  const uint32_t r0 = blockIdx.x * T;
   const float q[3] = {P.r[0][3], P.r[1][3], P.r[2][3]};
-  if (tid < kBoxTile) {
+  if (tid < T) {
     const uint32_t k = r0 + tid;
     float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
     if (k < n) {
@@ -134,7 +130,7 @@ __global__ void __launch_bounds__(CubeShape<W>::NT) k_box_integrate(MapView M,
     s_pr[tid] = return_record(p, q[0], q[1], q[2]);
   }
   __syncthreads();
-  for (int e = tid; e < kBoxTile * 3 * W; e += S::NT) {
+  for (int e = tid; e < T * 3 * W; e += S::NT) {
     const int t = e / (3 * W), ax = (e / W) % 3, k = e % W;
     const float4 p = s_p[t];
     if (p.w == 0.f) continue;
@@ -153,7 +149,7 @@ __global__ void __launch_bounds__(CubeShape<W>::NT) k_box_integrate(MapView M,
     ky[s] = (o / W) % W;
     kz[s] = o / (W * W);
   }
-  for (int t = 0; t < kBoxTile; ++t) {
+  for (int t = 0; t < T; ++t) {
     const float4 pr = s_pr[t];
     if (pr.w == 0.f) continue;  // uniform across the block
 #pragma unroll
@@ -166,7 +162,7 @@ __global__ void __launch_bounds__(CubeShape<W>::NT) k_box_integrate(MapView M,
       if ((ox | oy | oz) >= 0) atomicAdd(B.vox + (ox + oy + oz), make_word(dq, 1ull));
     }
   }
-  for (int e = tid; e < kBoxTile * M.ns; e += S::NT) {
+  for (int e = tid; e < T * M.ns; e += S::NT) {
     const int t = e / M.ns, s = e % M.ns + 1;
     if (s_p[t].w == 0.f) continue;
     const float p[3] = {s_p[t].x, s_p[t].y, s_p[t].z};
@@ -201,20 +197,20 @@ __device__ inline void finalize_voxel(const MapView& M, const Box& B, size_t at)
 // and cleared-band samples of its accepted returns, enumerated as in
 // k_box_integrate -- after all of the scan's additions (a launch of its own).
 // Voxels the scan does not touch keep their words and flags. A voxel is reached
-// through many returns: bound by the L2 reads of its word and flags (32 us per
+// through many returns: bound by the L2 reads of its word and flags (29 us per
 // pine frame; one thread per (return, offset) that found its voxel by itself and
 // always wrote the flags took 117 us).
-template <int W>
+template <int W, int T>
 __global__ void __launch_bounds__(CubeShape<W>::NT) k_box_finalize(MapView M,
                                                                    const float4* __restrict__ scratch,
                                                                    uint32_t n, float q0, float q1,
                                                                    float q2, Box B) {
   using S = CubeShape<W>;
-  __shared__ float4 s_p[kBoxTile];
-  __shared__ long long s_off[kBoxTile][3][W];
+  __shared__ float4 s_p[T];
+  __shared__ long long s_off[T][3][W];
   const int tid = threadIdx.x;
-  const uint32_t r0 = blockIdx.x * kBoxTile;
-  for (int e = tid; e < kBoxTile * 3 * W; e += S::NT) {
+  const uint32_t r0 = blockIdx.x * T;
+  for (int e = tid; e < T * 3 * W; e += S::NT) {
     const int t = e / (3 * W), ax = (e / W) % 3, k = e % W;
     const float4 p = r0 + t < n ? scratch[r0 + t] : make_float4(0.f, 0.f, 0.f, 0.f);
     if (ax == 0 && k == 0) s_p[t] = p;
@@ -224,7 +220,7 @@ __global__ void __launch_bounds__(CubeShape<W>::NT) k_box_finalize(MapView M,
     s_off[t][ax][k] = box_offset(B, ax, i - M.dom_vox[ax] + k - S::MR);
   }
   __syncthreads();
-  for (int t = 0; t < kBoxTile; ++t) {
+  for (int t = 0; t < T; ++t) {
     if (s_p[t].w == 0.f) continue;
 #pragma unroll
     for (int s = 0; s < S::OPT; ++s) {
@@ -235,7 +231,7 @@ __global__ void __launch_bounds__(CubeShape<W>::NT) k_box_finalize(MapView M,
     }
   }
   const float q[3] = {q0, q1, q2};
-  for (int e = tid; e < kBoxTile * M.ns; e += S::NT) {
+  for (int e = tid; e < T * M.ns; e += S::NT) {
     const int t = e / M.ns, s = e % M.ns + 1;
     if (s_p[t].w == 0.f) continue;
     const float p[3] = {s_p[t].x, s_p[t].y, s_p[t].z};
@@ -329,15 +325,23 @@ extern "C" af_status af_integrate_scan_noalloc(const af_config* cfg, const float
 
   cudaStream_t s = (cudaStream_t)stream;
   if (n > 0) {
-    const unsigned grid = (n + kBoxTile - 1) / kBoxTile;
+    // the box's kernels take the large tile from the middle range on
+    const int T = n < kTileSmallBelow ? kTileSmall : kTileLarge;
+    const unsigned grid = (n + T - 1) / T;
+#define AF_TILE(W, TT)                                                                                    \
+  {                                                                                                       \
+    k_box_integrate<W, TT><<<grid, CubeShape<W>::NT, 0, s>>>(M, d_xyz, n, P, scratch, B);                \
+    k_box_finalize<W, TT><<<grid, CubeShape<W>::NT, 0, s>>>(M, scratch, n, pose[3], pose[7], pose[11], B); \
+  }
     switch (2 * M.m + 1) {
-#define AF_CASE(W)                                                                                    \
-  case W:                                                                                             \
-    k_box_integrate<W><<<grid, CubeShape<W>::NT, 0, s>>>(M, d_xyz, n, P, scratch, B);                \
-    k_box_finalize<W><<<grid, CubeShape<W>::NT, 0, s>>>(M, scratch, n, pose[3], pose[7], pose[11], B); \
+#define AF_CASE(W)                                \
+  case W:                                         \
+    if (T == kTileSmall) AF_TILE(W, kTileSmall)   \
+    else AF_TILE(W, kTileLarge)                   \
     break;
       AF_CASE(3) AF_CASE(5) AF_CASE(7) AF_CASE(9) AF_CASE(11) AF_CASE(13) AF_CASE(15) AF_CASE(17)
 #undef AF_CASE
+#undef AF_TILE
     }
   }
   const cudaError_t e = cudaGetLastError();
