@@ -515,7 +515,7 @@ af_status af_points_export(af_ctx *ctx, uint32_t cap, int32_t *h_ijk, float *h_n
  * launches (milliseconds) and, if `reset`, forgets them. launches[] counts
  * kernels: an af_score call with work sharing on is three (k_score,
  * k_score_split, k_score_finish) timed as one bracket, an af_soft_refine call
- * two (the pairs inside the view, then those that leave it).
+ * two (all pairs, then those whose samples lie very far from their point).
  */
 typedef struct {
     uint64_t launches[10];

@@ -258,16 +258,16 @@ __device__ inline bool sample_cell(const SoftView& S, const PointCell& pc, const
   return in;
 }
 
-// The same for a pair whose samples all lie inside the view and within 2^22
-// voxels of its point (samples_inside): no check is left, and the floor comes
-// from adding 1.5 2^23, which rounds to an integer kept in the low bits -- four
-// single-precision operations at full rate in the place of a rounding and a
-// conversion at a quarter of it. `cb` is the point's cell less the view's base
-// and that constant's bits. Same cell and same f.
+// The same cell and f for a sample within 2^22 voxels of its point: the floor
+// comes from adding 1.5 2^23, which rounds to an integer kept in the low bits --
+// four single-precision operations at full rate in the place of a rounding and a
+// conversion at a quarter of it. `cb` is the point's cell less the view's base and
+// that constant's bits. Whether the cell lies inside the view is known from the
+// sample's index (samples_near).
 constexpr float kRound = 12582912.0f;        // 1.5 2^23
 constexpr int kRoundBits = 0x4B400000;
-__device__ inline void sample_cell_inside(const PointCell& pc, const Dir& d, const int cb[3], float t,
-                                          float f[3], int c[3]) {
+__device__ inline void sample_cell_near(const PointCell& pc, const Dir& d, const int cb[3], float t,
+                                        float f[3], int c[3]) {
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     const float l = sample_pos(pc, d, t, i);
@@ -278,24 +278,48 @@ __device__ inline void sample_cell_inside(const PointCell& pc, const Dir& d, con
   }
 }
 
-// Whether every sample j0..J lies inside the view, and the constants of
-// sample_cell_inside. Rounding is monotone, so on each axis the samples' cells
-// lie between those of the first and the last sample.
+// Whether every sample j0..J lies within 2^22 voxels of the point and the first
+// one inside the view; then the constants of sample_cell_near and the last sample
+// inside the view. Rounding is monotone, so on each axis the samples' cells go one
+// way: a pair's samples inside the view are the first ones, up to one found by
+// bisection. (Pairs that leave the view are ordinary -- every third one where the
+// map box ends half a metre behind the surfaces.)
 template <bool SPARSE>
-__device__ inline bool samples_inside(const SoftView& S, const PointCell& pc, const Dir& d, int cb[3]) {
-  bool in = true;
+__device__ inline bool samples_near(const SoftView& S, const PointCell& pc, const Dir& d, int cb[3],
+                                    int* last) {
+  bool near = pc.ok;
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
     const float t = __fadd_rn(d.e, (float)(e ? S.J : S.j0));
-    float f[3];
-    int c[3];
-    in = in && sample_cell<SPARSE>(S, pc, d, t, f, c);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) in = in && fabsf(sample_pos(pc, d, t, i)) < 4.0e6f;
+    for (int i = 0; i < 3; ++i) near = near && fabsf(sample_pos(pc, d, t, i)) < 4.0e6f;
   }
 #pragma unroll
   for (int i = 0; i < 3; ++i) cb[i] = (int)pc.I[i] - (SPARSE ? S.glo[i] : S.lo[i]) - kRoundBits;
-  return in;
+  const auto inside = [&](int j) {
+    float f[3];
+    int c[3];
+    sample_cell_near(pc, d, cb, __fadd_rn(d.e, (float)j), f, c);
+    bool in = true;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) in = in && (unsigned)c[i] < (unsigned)(SPARSE ? 8 * S.gdim[i] : S.ncell[i]);
+    return in;
+  };
+  if (!near || !inside(S.j0)) return false;
+  int lo = S.j0, hi = S.J;
+  if (inside(hi)) {
+    lo = hi;
+  } else {
+    while (hi - lo > 1) {  // lo inside, hi outside
+      const int mid = (lo + hi) >> 1;
+      if (inside(mid))
+        lo = mid;
+      else
+        hi = mid;
+    }
+  }
+  *last = lo;
+  return true;
 }
 
 __device__ inline float lerp(float a, float b, float t) { return __fmaf_rn(t, b - a, a); }
@@ -445,20 +469,24 @@ __device__ inline float trilinear(const float4& lo, const float4& hi, const floa
 // 4; the refinement of 30k pairs 236 us with 3, 271 with 4 (spills), 263 with 2.
 constexpr int kInFlightField = 2;
 constexpr int kInFlightRefine = 3;
+constexpr int kInFlightRefineFew = 4;  // of few pairs, which wait for latency only
 
-// Folds lane g's samples j0 + g, j0 + g + kLanes, ... into sm. INSIDE: every
-// sample lies inside the view (samples_inside).
+// Folds lane g's samples j0 + g, j0 + g + kLanes, ... into sm. NEAR: every sample
+// lies near the point, those up to `last` inside the view (samples_near).
 //
 // Most samples of a 1.25 m axis read nothing but tau (78% of those of a finished
 // pine map), so the dense view's records are only read in blocks of cells that
 // hold anything else: one bit per 8^3 cells, 29 KB for the pine box, which stays
 // in L1. The records then read are a 27 MB part of the 3.7 GB view and stay in L2.
 // With the checks of the cells gone as well, the field of a finished map's 30k
-// points (1.9M pairs) went from 862 to 487 us, forward plus adjoint of 113k pairs
-// from 149 to 72 us, the refinement of 30k pairs from 315 to 236 us.
-template <bool INSIDE, bool GRAD, bool FIXED, bool SPARSE, int NF>
+// points (1.9M pairs) went from 862 to about 490 us, forward plus adjoint of 113k
+// pairs from 149 to 72 us, the refinement of 30k pairs from 315 to 235 us. In a
+// small box (0.17 GB of records, 350k pairs) the marks spare nothing and the field
+// takes 109 against 101 us; a switch at run time that drops them there cost more
+// everywhere (537 and 114 us).
+template <bool NEAR, bool GRAD, bool FIXED, bool SPARSE, int NF>
 __device__ inline void fold_samples(Softmin<GRAD, FIXED>& sm, const SoftView& S, const PointCell& pc,
-                                    const Dir& d, const int cb[3], int g) {
+                                    const Dir& d, const int cb[3], int last, int g) {
 #pragma unroll 1
   for (int j = S.j0 + g; j <= S.J; j += NF * kLanes) {
     float f[NF][3];
@@ -471,9 +499,9 @@ __device__ inline void fold_samples(Softmin<GRAD, FIXED>& sm, const SoftView& S,
       has[q] = j + q * kLanes <= S.J;
       const float t = __fadd_rn(d.e, (float)(j + q * kLanes));
       int c[3];
-      if (INSIDE) {
-        sample_cell_inside(pc, d, cb, t, f[q], c);
-        in[q] = has[q];
+      if (NEAR) {
+        sample_cell_near(pc, d, cb, t, f[q], c);
+        in[q] = j + q * kLanes <= last;
       } else {
         in[q] = has[q] && sample_cell<SPARSE>(S, pc, d, t, f[q], c);
       }
@@ -514,10 +542,10 @@ __device__ inline void fold_samples(Softmin<GRAD, FIXED>& sm, const SoftView& S,
   }
 }
 
-// How a kernel takes its samples: every pair whose samples lie inside the view
-// without checks and the others with them (kBoth), the others not at all
-// (kInside: *outside is set instead), every pair with checks (kChecked).
-enum Road { kBoth, kInside, kChecked };
+// How a kernel takes its samples: the short way for every pair whose samples lie
+// near its point and the general way for the others (kBoth), the others not at all
+// (kNear: *far is set instead), every pair the general way (kGeneral).
+enum Road { kBoth, kNear, kGeneral };
 
 // C of one pair and, with GRAD, dC / d(alpha, beta, h); *cmin = min_j phi_j.
 // Called by all kLanes lanes of the pair's group (lane g of it); with
@@ -525,16 +553,16 @@ enum Road { kBoth, kInside, kChecked };
 template <bool GRAD, bool FIXED, bool SPARSE, int NF, Road ROAD>
 __device__ inline float soft_eval(const SoftView& S, const PointCell& pc, const Dir& d,
                                   const float t1[3], const float t2[3], bool live, int g,
-                                  float* ga, float* gb, float* gh, float* cmin, bool* outside) {
+                                  float* ga, float* gb, float* gh, float* cmin, bool* far) {
   Softmin<GRAD, FIXED> sm;
   if (live) {
-    int cb[3] = {0, 0, 0};
-    if (ROAD != kChecked && samples_inside<SPARSE>(S, pc, d, cb))
-      fold_samples<true, GRAD, FIXED, SPARSE, NF>(sm, S, pc, d, cb, g);
-    else if (ROAD == kInside)
-      *outside = true;
+    int cb[3] = {0, 0, 0}, last = 0;
+    if (ROAD != kGeneral && samples_near<SPARSE>(S, pc, d, cb, &last))
+      fold_samples<true, GRAD, FIXED, SPARSE, NF>(sm, S, pc, d, cb, last, g);
+    else if (ROAD == kNear)
+      *far = true;
     else
-      fold_samples<false, GRAD, FIXED, SPARSE, ROAD == kChecked ? NF : 1>(sm, S, pc, d, cb, g);
+      fold_samples<false, GRAD, FIXED, SPARSE, ROAD == kGeneral ? NF : 1>(sm, S, pc, d, cb, 0, g);
   }
   sm.reduce(S.k2);
   const float C = (FIXED ? S.ref : sm.m) - S.ln2_tau_s * lg2(sm.Z);
@@ -636,8 +664,8 @@ __global__ void __launch_bounds__(128) k_soft(SoftView S, const float* __restric
 
 // `steps` ascent steps on C of pair i in registers, then C at the final state;
 // the group's lanes (`act`: the pair is taken) update identical copies of
-// (alpha, beta, h). False, with nothing written, if a step takes a sample out of
-// the view (ROAD == kInside).
+// (alpha, beta, h). False, with nothing written, if a step takes a sample far from
+// the point (ROAD == kNear).
 template <bool FIXED, bool SPARSE, int NF, Road ROAD>
 __device__ inline bool refine_pair(const SoftView& S, const RefineArgs& R, const float* __restrict__ pts,
                                    uint32_t per_point, const float* __restrict__ u0,
@@ -652,13 +680,13 @@ __device__ inline bool refine_pair(const SoftView& S, const RefineArgs& R, const
   float al = alpha[i], be = beta[i], h = hh[i];
   // a pair that is not finite (e.g. a point with no start) samples nothing
   const bool fin = pc.finite && make_dir(S, u, t1, t2, al, be, h).finite;
-  bool outside = false;
+  bool far = false;
 #pragma unroll 1
   for (int k = 0; k < R.steps; ++k) {
     const Dir d = make_dir(S, u, t1, t2, al, be, h);
-    const bool live = fin && act && d.finite && !outside;
+    const bool live = fin && act && d.finite && !far;
     float da, db, dh, mn;
-    soft_eval<true, FIXED, SPARSE, NF, ROAD>(S, pc, d, t1, t2, live, g, &da, &db, &dh, &mn, &outside);
+    soft_eval<true, FIXED, SPARSE, NF, ROAD>(S, pc, d, t1, t2, live, g, &da, &db, &dh, &mn, &far);
     if (live) {
       al = __fmaf_rn(R.lr_dir, da, al);
       be = __fmaf_rn(R.lr_dir, db, be);
@@ -668,9 +696,9 @@ __device__ inline bool refine_pair(const SoftView& S, const RefineArgs& R, const
   const Dir d = make_dir(S, u, t1, t2, al, be, h);
   const bool ok = fin && d.finite;
   float mn;
-  float C = soft_eval<false, FIXED, SPARSE, NF, ROAD>(S, pc, d, t1, t2, ok && act && !outside, g, nullptr,
-                                                      nullptr, nullptr, &mn, &outside);
-  if (!act || outside || g != 0) return !outside;
+  float C = soft_eval<false, FIXED, SPARSE, NF, ROAD>(S, pc, d, t1, t2, ok && act && !far, g, nullptr,
+                                                      nullptr, nullptr, &mn, &far);
+  if (!act || far || g != 0) return !far;
   if (!ok) C = mn = al = be = h = NAN;
   alpha[i] = al;
   beta[i] = be;
@@ -680,14 +708,14 @@ __device__ inline bool refine_pair(const SoftView& S, const RefineArgs& R, const
   return true;
 }
 
-// Two launches: the checks of the samples' cells would cost every pair 70
-// registers, so the first (ROAD kInside) leaves a pair that a step takes out of
-// the view as it was and marks its C with a NaN of its own, and the second takes
-// the marked pairs from their start again, with the checks.
+// Two launches: the general way beside the short one would cost every pair 70
+// registers, so the first (ROAD kNear) leaves a pair that it cannot take
+// (samples_near) as it was and marks its C with a NaN of its own, and the second
+// takes the marked pairs from their start again.
 constexpr unsigned kRedo = 0x7FC05EDDu;
 
-template <bool FIXED, bool SPARSE, Road ROAD>
-__global__ void __launch_bounds__(128, 4) k_soft_refine(SoftView S, RefineArgs R,
+template <bool FIXED, bool SPARSE, Road ROAD, int NF>
+__global__ void __launch_bounds__(128, ROAD == kBoth ? 2 : 4) k_soft_refine(SoftView S, RefineArgs R,
                                                      const float* __restrict__ pts,
                                                      uint32_t per_point,
                                                      const float* __restrict__ u0,
@@ -701,11 +729,11 @@ __global__ void __launch_bounds__(128, 4) k_soft_refine(SoftView S, RefineArgs R
     const size_t i0 = base + w.slot;
     bool act = i0 < n;
     const size_t i = act ? i0 : n - 1;
-    if (ROAD == kChecked) {
+    if (ROAD == kGeneral) {
       act = act && __float_as_uint(c[i]) == kRedo;
       if (!__any_sync(kFull, act)) continue;
     }
-    if (!refine_pair<FIXED, SPARSE, ROAD == kChecked ? 1 : kInFlightRefine, ROAD>(
+    if (!refine_pair<FIXED, SPARSE, NF, ROAD>(
             S, R, pts, per_point, u0, alpha, beta, hh, c, cmin, i, act, w.g) && act && w.g == 0)
       c[i] = __uint_as_float(kRedo);
   }
@@ -924,9 +952,19 @@ cudaError_t launch_soft_refine(const SoftView& S, const RefineArgs& R, const flo
                                cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
   const unsigned g = grid_for(n * kLanes, 128, num_sms, 16);
-#define AF_REFINE_LAUNCH(FX, SP)                                                                            \
-  (k_soft_refine<FX, SP, kInside><<<g, 128, 0, stream>>>(S, R, pts, per_point, u0, al, be, h, n, c, cmin), \
-   k_soft_refine<FX, SP, kChecked><<<g, 128, 0, stream>>>(S, R, pts, per_point, u0, al, be, h, n, c, cmin))
+  // fewer pairs than the wide kernel holds at once: latency is all that counts
+  const bool few = n <= (uint64_t)num_sms * 2 * (128 / kLanes);
+#define AF_REFINE_ROAD(FX, SP, RD, NF) \
+  k_soft_refine<FX, SP, RD, NF><<<g, 128, 0, stream>>>(S, R, pts, per_point, u0, al, be, h, n, c, cmin)
+#define AF_REFINE_LAUNCH(FX, SP)                            \
+  do {                                                      \
+    if (few) {                                              \
+      AF_REFINE_ROAD(FX, SP, kBoth, kInFlightRefineFew);    \
+    } else {                                                \
+      AF_REFINE_ROAD(FX, SP, kNear, kInFlightRefine);       \
+      AF_REFINE_ROAD(FX, SP, kGeneral, 1);                  \
+    }                                                       \
+  } while (0)
   if (S.fixed && S.sparse)
     AF_REFINE_LAUNCH(true, true);
   else if (S.fixed)
@@ -936,6 +974,7 @@ cudaError_t launch_soft_refine(const SoftView& S, const RefineArgs& R, const flo
   else
     AF_REFINE_LAUNCH(false, false);
 #undef AF_REFINE_LAUNCH
+#undef AF_REFINE_ROAD
   return cudaGetLastError();
 }
 
