@@ -481,9 +481,11 @@ constexpr int kInFlightRefineFew = 4;  // of few pairs, which wait for latency o
 // With the checks of the cells gone as well, the field of a finished map's 30k
 // points (1.9M pairs) went from 862 to about 490 us, forward plus adjoint of 113k
 // pairs from 149 to 72 us, the refinement of 30k pairs from 315 to 235 us. In a
-// small box (0.17 GB of records, 350k pairs) the marks spare nothing and the field
-// takes 109 against 101 us; a switch at run time that drops them there cost more
-// everywhere (537 and 114 us).
+// small box (0.17 GB of records, which the caches hold; 350k pairs, a third of
+// which leave the view) the field takes 109 against 101 us: the bisection is paid
+// once per evaluation. Without the marks there 112, with per-sample checks in its
+// place 105 (but 285 against 252 us for the refinement), by the general way for
+// the pairs that leave 142 to 147.
 template <bool NEAR, bool GRAD, bool FIXED, bool SPARSE, int NF>
 __device__ inline void fold_samples(Softmin<GRAD, FIXED>& sm, const SoftView& S, const PointCell& pc,
                                     const Dir& d, const int cb[3], int last, int g) {
