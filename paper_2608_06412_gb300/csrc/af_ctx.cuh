@@ -46,6 +46,9 @@ struct af_ctx {
   bool views_sparse = false;     // the view built is the sparse one
   bool views_valid = false;
   uint32_t views_frame = 0;
+  bool views_filled = false;             // the dense view's buffers hold tau or better
+  unsigned long long views_capture = 0;  // capture that updates the view, + 1 (0: none)
+  uint32_t views_capture_frame = 0;      // ... and the scan it updates it to
   float* d_table = nullptr;  // seed directions, and their host copy
   uint32_t table_cap = 0;
   std::vector<float> h_table;

@@ -908,7 +908,6 @@ static af_status ensure_views(af_ctx* ctx, cudaStream_t s) {
     ctx->views_sparse = ctx->soft_mode == 2 || (ctx->soft_mode == 0 && !dense_views_fit(ctx));
   const bool stale = !ctx->views_valid || ctx->views_frame != ctx->frame;
   if (!ctx->views_sparse) {
-    bool fill = false;
     if (!ctx->d_cells) {
       const size_t nd = (size_t)M.dim_vox[0] * M.dim_vox[1] * M.dim_vox[2];
       const size_t nc = ((size_t)M.dim_vox[0] + 1) * (M.dim_vox[1] + 1) * (M.dim_vox[2] + 1);
@@ -929,21 +928,31 @@ static af_status ensure_views(af_ctx* ctx, cudaStream_t s) {
                     "soft clearance: cannot allocate the SDF views (%zu + %zu bytes) of the map box",
                     nd * sizeof(float), nc * 2 * sizeof(float4));
       }
-      fill = true;
+      ctx->views_filled = false;
     }
-    if (fill || stale) {
-      // scan stamps wrap at 2^32 - 2: then every brick is taken
-      const bool all = fill || !ctx->views_valid || ctx->frame < ctx->views_frame;
-      AF_CUDA(ctx, timed(ctx, 4, s, [&] {
-        return af::launch_views(M, ctx->num_sms, fill, all, ctx->views_frame, ctx->d_dense,
-                                ctx->d_cells, ctx->d_vlist, ctx->d_vseen, s);
-      }));
-      // a captured update has not run yet: the next call updates from where
-      // the view is now
-      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-      if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
-      if (!fill && cap != cudaStreamCaptureStatusNone) return AF_OK;
+    if (!stale) return AF_OK;
+    // Launches under capture have not run yet, so they leave the view's state
+    // to eager calls: the next one fills and updates from where the view is
+    // now, and so does every replay. Within one capture the view is brought up
+    // to date once per scan.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(s, &cap, &id) != cudaSuccess) cudaGetLastError();
+    const bool captured = cap != cudaStreamCaptureStatusNone;
+    if (captured && ctx->views_capture == id + 1 && ctx->views_capture_frame == ctx->frame) return AF_OK;
+    const bool fill = !ctx->views_filled;
+    // scan stamps wrap at 2^32 - 2: then every brick is taken
+    const bool all = fill || !ctx->views_valid || ctx->frame < ctx->views_frame;
+    AF_CUDA(ctx, timed(ctx, 4, s, [&] {
+      return af::launch_views(M, ctx->num_sms, fill, all, ctx->views_frame, ctx->d_dense,
+                              ctx->d_cells, ctx->d_vlist, ctx->d_vseen, s);
+    }));
+    if (captured) {
+      ctx->views_capture = id + 1;
+      ctx->views_capture_frame = ctx->frame;
+      return AF_OK;
     }
+    ctx->views_filled = true;
   } else {
     const int gx = M.dim_vox[0] / 8 + 1, gy = M.dim_vox[1] / 8 + 1, gz = M.dim_vox[2] / 8 + 1;
     const size_t gcount = (size_t)gx * gy * gz;
@@ -1188,6 +1197,7 @@ extern "C" af_status af_soft_set_view(af_ctx* ctx, int32_t mode) {
   ctx->d_scells = nullptr;
   ctx->scells_cap = 0;
   ctx->views_valid = false;
+  ctx->views_capture = 0;
   ctx->soft_mode = mode;
   return AF_OK;
 }
