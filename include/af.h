@@ -153,6 +153,10 @@ af_status af_destroy(af_ctx *ctx);
  * end of the call weights above w_cap are capped with proportional rescaling
  * and the occupied / known view of every touched brick is rebuilt.
  * Asynchronous on `stream`; d_xyz must stay valid until the work completes.
+ * Under stream capture the pose and the scan's number are kept with the graph:
+ * a scan is one run of it, so replay such a graph once (a second run adds to
+ * the voxels, but finds its bricks marked as this scan's already and rebuilds
+ * none of their views).
  */
 af_status af_integrate_scan(af_ctx *ctx, const float *d_xyz, uint32_t n,
                             const float pose[16], void *stream);

@@ -35,7 +35,7 @@ struct af_ctx {
   // map has changed since)
   float* d_dense = nullptr;
   float4* d_cells = nullptr;
-  uint32_t* d_vlist = nullptr;   // bricks to update, then their count
+  uint32_t* d_vlist = nullptr;   // bricks to update, their count, the stamps they were taken at
   uint32_t* d_vseen = nullptr;   // a bit per block of 8^3 cells that reads anything but tau
   uint32_t* d_bgrid = nullptr;   // the brick-sparse view: slot per grid brick
   uint32_t* d_skeys = nullptr;   // grid brick of every slot

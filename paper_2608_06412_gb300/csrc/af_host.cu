@@ -31,9 +31,9 @@ cudaError_t launch_score(const MapView& M, const ToolView& T, const float* d_pts
                          const ScoreSplit& S, int num_sms, cudaStream_t stream);
 cudaError_t launch_export_flags(const MapView& M, uint32_t count, uint8_t* d_flags,
                                 cudaStream_t stream);
-cudaError_t launch_views(const MapView& M, int num_sms, bool fill, bool all, uint32_t since,
-                         float* dense, float4* cells, uint32_t* list, uint32_t* seen,
-                         cudaStream_t stream);
+cudaError_t launch_views(const MapView& M, int num_sms, bool fill, float* dense, float4* cells,
+                         uint32_t* list, uint32_t* seen, cudaStream_t stream);
+size_t view_list_words(const MapView& M);
 size_t seen_words(const MapView& M);
 cudaError_t launch_soft_seed(const float* d_nrm, uint32_t m, const float* d_table, uint32_t K,
                              float* d_u0, int num_sms, cudaStream_t stream);
@@ -915,7 +915,7 @@ static af_status ensure_views(af_ctx* ctx, cudaStream_t s) {
         return fail(ctx, AF_ERR_CAPACITY, "soft clearance: the map box has too many cells for the dense SDF view");
       if (cudaMalloc(&ctx->d_dense, nd * sizeof(float)) != cudaSuccess ||
           cudaMalloc(&ctx->d_cells, nc * 2 * sizeof(float4)) != cudaSuccess ||
-          cudaMalloc(&ctx->d_vlist, ((size_t)M.pool_blocks + 1) * sizeof(uint32_t)) != cudaSuccess ||
+          cudaMalloc(&ctx->d_vlist, af::view_list_words(M) * sizeof(uint32_t)) != cudaSuccess ||
           cudaMalloc(&ctx->d_vseen, af::seen_words(M) * sizeof(uint32_t)) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(ctx->d_dense);
@@ -941,11 +941,9 @@ static af_status ensure_views(af_ctx* ctx, cudaStream_t s) {
     const bool captured = cap != cudaStreamCaptureStatusNone;
     if (captured && ctx->views_capture == id + 1 && ctx->views_capture_frame == ctx->frame) return AF_OK;
     const bool fill = !ctx->views_filled;
-    // scan stamps wrap at 2^32 - 2: then every brick is taken
-    const bool all = fill || !ctx->views_valid || ctx->frame < ctx->views_frame;
     AF_CUDA(ctx, timed(ctx, 4, s, [&] {
-      return af::launch_views(M, ctx->num_sms, fill, all, ctx->views_frame, ctx->d_dense,
-                              ctx->d_cells, ctx->d_vlist, ctx->d_vseen, s);
+      return af::launch_views(M, ctx->num_sms, fill, ctx->d_dense, ctx->d_cells, ctx->d_vlist,
+                              ctx->d_vseen, s);
     }));
     if (captured) {
       ctx->views_capture = id + 1;

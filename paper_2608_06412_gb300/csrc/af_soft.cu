@@ -51,19 +51,21 @@ __global__ void __launch_bounds__(256) k_fill(float4* __restrict__ out, size_t n
     out[i] = v;
 }
 
-// Lists the pool bricks whose voxels changed after scan `since` (every brick
-// with `all`): each scan stamps the hash slot of every brick it touches, so
-// the slots say what a view built at an earlier scan lacks, however many scans
-// ago that was. A brick stamped by a scan later than the caller's is listed
-// too, so a replayed launch covers the scans since.
-__global__ void __launch_bounds__(256) k_view_list(MapView M, uint32_t since, int all,
+// Lists the pool bricks that a scan has touched since the view last took them:
+// each scan stamps the hash slot of every brick it touches, and `taken` keeps the
+// stamp at which the view took a brick (~0: never). Stamps are compared for
+// equality, not order, so scans that run late -- a captured scan replayed after
+// later ones keeps its older number -- and scan numbers that wrap are covered,
+// and a replayed update takes whatever changed before it.
+__global__ void __launch_bounds__(256) k_view_list(MapView M, uint32_t* __restrict__ taken,
                                                    uint32_t* __restrict__ list,
                                                    uint32_t* __restrict__ nlist) {
   const uint32_t count = min(__ldcg(&M.ctl->pool_count), M.pool_blocks);
   for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < count; b += gridDim.x * blockDim.x) {
-    uint32_t val, stamp = ~0u;
-    const bool found = all || find_slot(M, M.bkey[b], &val, &stamp) >= 0;
-    if (all || (found && stamp != ~0u && stamp > since)) list[atomicAdd(nlist, 1u)] = b;
+    uint32_t val, stamp;
+    if (find_slot(M, M.bkey[b], &val, &stamp) < 0 || stamp == taken[b]) continue;
+    taken[b] = stamp;
+    list[atomicAdd(nlist, 1u)] = b;
   }
 }
 
@@ -887,31 +889,34 @@ cudaError_t launch_sview_fill(const MapView& M, int num_sms, const uint32_t* key
   return cudaGetLastError();
 }
 
+// Words of the dense view's list: bricks to update, their count, and the stamp at
+// which the view took each brick.
+size_t view_list_words(const MapView& M) { return 2 * (size_t)M.pool_blocks + 1; }
+
 // Words of the dense view's block marks.
 size_t seen_words(const MapView& M) {
   const size_t n = ((size_t)M.dim_vox[0] / 8 + 1) * (M.dim_vox[1] / 8 + 1) * (M.dim_vox[2] / 8 + 1);
   return (n + 31) / 32;
 }
 
-// Brings the dense view up to date with the map: the bricks changed after scan
-// `since`, or every brick (`all`); with `fill` the buffers are new and every
-// value starts as tau.
-cudaError_t launch_views(const MapView& M, int num_sms, bool fill, bool all, uint32_t since,
-                         float* dense, float4* cells, uint32_t* list, uint32_t* seen,
-                         cudaStream_t stream) {
+// Brings the dense view up to date with the map; with `fill` the buffers are new,
+// every value starts as tau and every brick is taken. `list`: view_list_words(M).
+cudaError_t launch_views(const MapView& M, int num_sms, bool fill, float* dense, float4* cells,
+                         uint32_t* list, uint32_t* seen, cudaStream_t stream) {
   const size_t nd = (size_t)M.dim_vox[0] * M.dim_vox[1] * M.dim_vox[2];  // a multiple of 512
   const size_t nc = ((size_t)M.dim_vox[0] + 1) * (M.dim_vox[1] + 1) * (M.dim_vox[2] + 1);
+  uint32_t *nlist = list + M.pool_blocks, *taken = nlist + 1;
   if (fill) {
     k_fill<<<grid_for(nd / 4, 256, num_sms, 8), 256, 0, stream>>>(reinterpret_cast<float4*>(dense),
                                                                    nd / 4, M.tau);
     k_fill<<<grid_for(nc * 2, 256, num_sms, 8), 256, 0, stream>>>(cells, nc * 2, M.tau);
-    const cudaError_t z = cudaMemsetAsync(seen, 0, seen_words(M) * sizeof(uint32_t), stream);
+    cudaError_t z = cudaMemsetAsync(seen, 0, seen_words(M) * sizeof(uint32_t), stream);
+    if (z == cudaSuccess) z = cudaMemsetAsync(taken, 0xFF, M.pool_blocks * sizeof(uint32_t), stream);
     if (z != cudaSuccess) return z;
   }
-  uint32_t* nlist = list + M.pool_blocks;
   cudaError_t e = cudaMemsetAsync(nlist, 0, sizeof(uint32_t), stream);
   if (e != cudaSuccess) return e;
-  k_view_list<<<grid_for(M.pool_blocks, 256, num_sms, 8), 256, 0, stream>>>(M, since, all ? 1 : 0, list, nlist);
+  k_view_list<<<grid_for(M.pool_blocks, 256, num_sms, 8), 256, 0, stream>>>(M, taken, list, nlist);
   k_dense_view<<<(unsigned)num_sms * 8, 256, 0, stream>>>(M, list, nlist, dense);
   k_cell_view<<<(unsigned)num_sms * 8, 256, 0, stream>>>(M, list, nlist, dense, cells, seen);
   return cudaGetLastError();

@@ -110,3 +110,21 @@ def test_two_soft_calls_and_a_scan_in_one_capture():
     r.check([0, 1, 2])
     r.c.copy_(first)
     r.check([0, 1])
+
+
+def test_scan_captured_early_and_replayed_late():
+    """A captured scan keeps its scan number; replayed after later scans and a
+    soft call, the next scan's update still takes its bricks."""
+    r = Rig()
+    r.scan(0)
+    r.soft()
+    g = r.capture(lambda: r.scan(1))
+    for k in (2, 3):
+        r.scan(k)
+    r.soft()
+    r.check([0, 2, 3])
+    g.replay()
+    # an empty scan: nothing of its own, but the view is out of date
+    r.map.integrate_scan(r.scans[0][0][:0], r.scans[0][1])
+    r.soft()
+    r.check([0, 1, 2, 3])
