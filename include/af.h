@@ -206,9 +206,9 @@ af_status af_score(af_ctx *ctx, const float *d_pts, const float *d_normals, uint
 
 /*
  * Work sharing of af_score (and af_frame_host): a point whose search takes
- * more than `budget` candidate directions past the arm screen hands the rest
- * of its directions to a second kernel that searches them one warp per
- * (point, direction); the labels and best directions are identical to the
+ * more than `budget` candidate directions past the screen (arm samples; with
+ * strict corridors their nearest voxels too) hands the rest of its directions
+ * to a second kernel that searches them one warp per (point, direction); the labels and best directions are identical to the
  * single-pass search for every budget. budget = -1: single pass, one warp
  * per point (the default); 0 .. 4096: the hand-off threshold. The hand-off
  * records take 12 bytes per point, allocated for max_points at af_create and

@@ -131,7 +131,7 @@ struct ScoreSplit {
   int2* over;        // (point, first direction not yet searched)
   uint32_t* res;     // packed (score << 16 | direction) of the search so far
   uint32_t* count;   // points handed off
-  int budget;        // directions past the arm screen before a hand-off; < 0: never
+  int budget;        // directions past the screen before a hand-off; < 0: never
 };
 
 struct ToolView {

@@ -858,6 +858,7 @@ __device__ int nearest_resolved(const MapView& M, const PtView& V, const PtState
   return res;
 }
 
+template <bool STRICT>
 __global__ void __launch_bounds__(128) k_pts_eval(MapView M, ToolView T, PtView V) {
   __shared__ uint32_t s_c2f[4][kC2FTab];
   const int lane = threadIdx.x & 31;
@@ -975,21 +976,21 @@ __global__ void __launch_bounds__(128) k_pts_eval(MapView M, ToolView T, PtView 
     const bool fast = reach_inside(M, T, P);
     int2 res;
     if (V.c2f_stride == 0) {
-      res = fast ? best_direction<true>(M, T, P, F, lane) : best_direction<false>(M, T, P, F, lane);
+      res = fast ? best_direction<true, STRICT>(M, T, P, F, lane) : best_direction<false, STRICT>(M, T, P, F, lane);
     } else {
       // coarse set, then the window around the nearest resolved neighbour's
       // direction (else around the coarse best); lowest-index minimum of both
       const int nb = nearest_resolved(M, V, st, s_c2f[threadIdx.x >> 5], lane);
       if (nb >= 0) {  // one pass over the coarse set and the neighbour's window
         const WindowFilter Fu{F, nb, V.c2f_half, V.c2f_stride, true};
-        res = fast ? best_direction<true>(M, T, P, Fu, lane) : best_direction<false>(M, T, P, Fu, lane);
+        res = fast ? best_direction<true, STRICT>(M, T, P, Fu, lane) : best_direction<false, STRICT>(M, T, P, Fu, lane);
       } else {  // the coarse set, then the window around its best
         const CoarseFilter Fc{F, V.c2f_stride};
-        res = fast ? best_direction<true>(M, T, P, Fc, lane) : best_direction<false>(M, T, P, Fc, lane);
+        res = fast ? best_direction<true, STRICT>(M, T, P, Fc, lane) : best_direction<false, STRICT>(M, T, P, Fc, lane);
         if (res.y >= 0) {
           const WindowFilter Fw{F, res.y, V.c2f_half, V.c2f_stride, false};
-          res = better(res, fast ? best_direction<true>(M, T, P, Fw, lane)
-                                 : best_direction<false>(M, T, P, Fw, lane));
+          res = better(res, fast ? best_direction<true, STRICT>(M, T, P, Fw, lane)
+                                 : best_direction<false, STRICT>(M, T, P, Fw, lane));
         }
       }
     }
@@ -1100,7 +1101,10 @@ af_status select_and_eval(af_ctx* ctx, uint32_t budget, int trigger, int moved, 
   k_pts_trigger<<<grid, kSelBlock, 0, s>>>(ctx->M, V, ctx->frame, moved, trigger, budget);
   k_pts_select<<<grid, kSelBlock, 0, s>>>(V, budget);
   if (V.c2f_stride > 0) k_pts_snap<<<grid_cap(ctx->pcfg.capacity, 256, ctx->num_sms, 8), 256, 0, s>>>(V);
-  k_pts_eval<<<(unsigned)ctx->num_sms * 8, 128, 0, s>>>(ctx->M, ctx->T, V);
+  if (ctx->T.strict)
+    k_pts_eval<true><<<(unsigned)ctx->num_sms * 8, 128, 0, s>>>(ctx->M, ctx->T, V);
+  else
+    k_pts_eval<false><<<(unsigned)ctx->num_sms * 8, 128, 0, s>>>(ctx->M, ctx->T, V);
   PT_CUDA(ctx, cudaGetLastError());
   return AF_OK;
 }

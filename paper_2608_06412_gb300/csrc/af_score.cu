@@ -2,9 +2,10 @@
 //
 // One warp per surface point.
 // The lanes first evaluate the normal filter for
-// 32 directions at a time (ballot -> candidate mask), then the arm samples of
-// each candidate (three single-bit lookups: occupied or unknown blocks). The
-// arm-clear candidates are taken four at a time (kSide) in index order:
+// 32 directions at a time (ballot -> candidate mask), then the start of each
+// candidate (the three arm samples, single-bit lookups: occupied or unknown
+// blocks; with strict corridors their nearest entry too). The open candidates are
+// taken four at a time (kSide) in index order:
 //   * tool kernel: 8 lanes per direction fetch the kernel's entries (the same
 //     32 voxels of four rows in one or two 16-byte loads), AND with the masks
 //     and __popc; the count saturates at the score to beat, so it stops as
@@ -17,7 +18,7 @@
 // index).
 //
 // Work sharing (ScoreSplit): a point whose search takes more than `budget`
-// directions past the arm screen stops there and hands the rest of its
+// directions past the screen stops there and hands the rest of its
 // directions to k_score_split, where one warp takes each (point, direction)
 // item, prunes it against the point's packed best so far (read at the start
 // of the item; the best only ever decreases) and folds its exact score in
@@ -34,7 +35,7 @@
 namespace af {
 
 // Scores point pi with the whole warp (all 32 lanes call this together).
-template <bool SPLIT>
+template <bool SPLIT, bool STRICT>
 __device__ void score_point(const MapView& M, const ToolView& T, const float* __restrict__ pts,
                             const float* __restrict__ nrm, uint32_t pi,
                             uint8_t* __restrict__ label, int16_t* __restrict__ best_out,
@@ -79,13 +80,13 @@ __device__ void score_point(const MapView& M, const ToolView& T, const float* __
   int2 res;
   int next = -1;
   if (!SPLIT) {
-    res = fast ? best_direction<true>(M, T, P, F, lane, confident)
-               : best_direction<false>(M, T, P, F, lane, confident);
+    res = fast ? best_direction<true, STRICT>(M, T, P, F, lane, confident)
+               : best_direction<false, STRICT>(M, T, P, F, lane, confident);
   } else {
     res = make_int2(-1, -1);
     if (confident())
-      res = fast ? best_direction_budget<true>(M, T, P, F, lane, S.budget, &next)
-                 : best_direction_budget<false>(M, T, P, F, lane, S.budget, &next);
+      res = fast ? best_direction_budget<true, STRICT>(M, T, P, F, lane, S.budget, &next)
+                 : best_direction_budget<false, STRICT>(M, T, P, F, lane, S.budget, &next);
   }
   if (res.x < 0) {  // not confident
     if (lane == 0) {
@@ -114,28 +115,29 @@ __device__ void score_point(const MapView& M, const ToolView& T, const float* __
 // 61.8 us per pine frame, 1.50 / 1.34 / 1.38 / 1.48 ms on the 1 cm map.
 constexpr int kScoreThreads = 1280;
 
-template <int WARPS, bool SPLIT>
+template <int WARPS, bool SPLIT, bool STRICT>
 __global__ void __launch_bounds__(WARPS * 32, kScoreThreads / (WARPS * 32))
     k_score(MapView M, ToolView T, const float* __restrict__ pts, const float* __restrict__ nrm,
             uint32_t m, uint8_t* __restrict__ label, int16_t* __restrict__ best_out,
             ScoreSplit S) {
   const uint32_t pi = blockIdx.x * WARPS + (threadIdx.x >> 5);
   if (pi >= m) return;  // whole warp
-  score_point<SPLIT>(M, T, pts, nrm, pi, label, best_out, threadIdx.x & 31, S);
+  score_point<SPLIT, STRICT>(M, T, pts, nrm, pi, label, best_out, threadIdx.x & 31, S);
 }
 
 // One (point, direction) item of a handed-off search; the whole warp.
-template <bool FAST>
+template <bool FAST, bool STRICT>
 __device__ void split_item(const MapView& M, const ToolView& T, const Pt& P, int g, uint32_t* res,
                            int lane) {
   const int nc = T.n_c;
   const uint32_t cur = __ldcg(res);
   const int bs = (int)(cur >> 16), bg = (int)(cur & 0xFFFFu);  // bg 0xFFFF: none yet
-  bool arm_ok = false;
-  if (lane == 0) arm_ok = arm_clear<FAST>(M, T, g, P);
-  arm_ok = __shfl_sync(0xffffffffu, arm_ok, 0);
+  const int4 dt = __ldg(T.dtab + g);
+  bool open = false;
+  if (lane == 0) open = start_open<FAST, STRICT>(M, T, g, dt, P);
+  open = __shfl_sync(0xffffffffu, open, 0);
   uint32_t mine;
-  if (!arm_ok) {
+  if (!open) {
     if (bs <= nc) return;  // blocked (n_c + 1) cannot beat an unblocked best
     mine = pack_result(make_int2(nc + 1, g));
   } else {
@@ -145,12 +147,13 @@ __device__ void split_item(const MapView& M, const ToolView& T, const Pt& P, int
     if (!exact && sat == 0) return;
     const int c = tool_count<FAST>(M, T, g, P, sat, lane);
     if (!exact && c >= sat) return;
-    mine = corridor_blocked<FAST>(M, T, __ldg(T.dtab + g), P, lane) ? pack_result(make_int2(nc + 1, g))
-                                                   : pack_result(make_int2(min(c, nc), g));
+    mine = corridor_blocked<FAST, STRICT>(M, T, dt, P, lane) ? pack_result(make_int2(nc + 1, g))
+                                                             : pack_result(make_int2(min(c, nc), g));
   }
   if (lane == 0 && mine < cur) atomicMin(res, mine);
 }
 
+template <bool STRICT>
 __global__ void __launch_bounds__(128, kScoreThreads / 128)
     k_score_split(MapView M, ToolView T, const float* __restrict__ pts,
                   const float* __restrict__ nrm, ScoreSplit S) {
@@ -175,9 +178,9 @@ __global__ void __launch_bounds__(128, kScoreThreads / 128)
     P.pz = i2 - M.dom_vox[2];
     const bool fast = reach_inside(M, T, P);
     if (fast)
-      split_item<true>(M, T, P, g, S.res + o, lane);
+      split_item<true, STRICT>(M, T, P, g, S.res + o, lane);
     else
-      split_item<false>(M, T, P, g, S.res + o, lane);
+      split_item<false, STRICT>(M, T, P, g, S.res + o, lane);
   }
 }
 
@@ -194,28 +197,34 @@ __global__ void __launch_bounds__(256) k_score_finish(ScoreSplit S, int n_c,
   }
 }
 
+template <bool STRICT>
+static cudaError_t launch_score_form(const MapView& M, const ToolView& T, const float* d_pts,
+                                     const float* d_nrm, uint32_t m, uint8_t* d_label,
+                                     int16_t* d_best, const ScoreSplit& S, int num_sms,
+                                     cudaStream_t stream) {
+  constexpr int WARPS = 2;
+  const unsigned grid = (m + WARPS - 1) / WARPS;
+  if (S.budget < 0) {
+    k_score<WARPS, false, STRICT><<<grid, WARPS * 32, 0, stream>>>(M, T, d_pts, d_nrm, m, d_label,
+                                                                   d_best, S);
+    return cudaGetLastError();
+  }
+  const cudaError_t e = cudaMemsetAsync(S.count, 0, sizeof(uint32_t), stream);
+  if (e != cudaSuccess) return e;
+  k_score<WARPS, true, STRICT><<<grid, WARPS * 32, 0, stream>>>(M, T, d_pts, d_nrm, m, d_label,
+                                                                d_best, S);
+  k_score_split<STRICT><<<num_sms * (kScoreThreads / 128), 128, 0, stream>>>(M, T, d_pts, d_nrm, S);
+  k_score_finish<<<num_sms, 256, 0, stream>>>(S, T.n_c, d_label, d_best);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_score(const MapView& M, const ToolView& T, const float* d_pts,
                          const float* d_nrm, uint32_t m, uint8_t* d_label, int16_t* d_best,
                          const ScoreSplit& S, int num_sms, cudaStream_t stream) {
   if (m == 0) return cudaSuccess;
-  constexpr int WARPS = 2;
-  if (S.budget >= 0) {
-    cudaError_t e = cudaMemsetAsync(S.count, 0, sizeof(uint32_t), stream);
-    if (e != cudaSuccess) return e;
-  }
-  if (S.budget >= 0)
-    k_score<WARPS, true><<<(m + WARPS - 1) / WARPS, WARPS * 32, 0, stream>>>(M, T, d_pts, d_nrm,
-                                                                            m, d_label, d_best, S);
-  else
-    k_score<WARPS, false><<<(m + WARPS - 1) / WARPS, WARPS * 32, 0, stream>>>(M, T, d_pts, d_nrm,
-                                                                             m, d_label, d_best, S);
-  if (S.budget >= 0) {
-    k_score_split<<<num_sms * (kScoreThreads / 128), 128, 0, stream>>>(M, T, d_pts, d_nrm, S);
-    k_score_finish<<<num_sms, 256, 0, stream>>>(S, T.n_c, d_label, d_best);
-  }
-  return cudaGetLastError();
+  return T.strict ? launch_score_form<true>(M, T, d_pts, d_nrm, m, d_label, d_best, S, num_sms, stream)
+                  : launch_score_form<false>(M, T, d_pts, d_nrm, m, d_label, d_best, S, num_sms, stream);
 }
-
 
 // Batched ticks: every point of every map of the batch, one warp per point,
 // persistent grid (see af_batch.cu).
@@ -228,8 +237,13 @@ __global__ void __launch_bounds__(WARPS * 32, kScoreThreads / (WARPS * 32))
   for (uint32_t pg = blockIdx.x * WARPS + (threadIdx.x >> 5); pg < total; pg += nw) {
     const int s = scene_of<2>(D, count, pg);
     const SceneDesc& d = D[s];
-    score_point<false>(d.M, d.T, d.pts, d.nrm, pg - d.pt_off, d.label, d.best, threadIdx.x & 31,
-                       ScoreSplit{nullptr, nullptr, nullptr, -1});
+    const ScoreSplit S{nullptr, nullptr, nullptr, -1};
+    if (d.T.strict)
+      score_point<false, true>(d.M, d.T, d.pts, d.nrm, pg - d.pt_off, d.label, d.best,
+                               threadIdx.x & 31, S);
+    else
+      score_point<false, false>(d.M, d.T, d.pts, d.nrm, pg - d.pt_off, d.label, d.best,
+                                threadIdx.x & 31, S);
   }
 }
 

@@ -166,17 +166,17 @@ __device__ inline int tool_count(const MapView& M, const ToolView& T, int g, con
 // unknown) blocks. The whole warp, one entry per lane per step (most blocked
 // corridors are so by their nearest entries). Strict corridors run along x, the
 // known view's rows.
-template <bool FAST>
+template <bool FAST, bool STRICT>
 __device__ inline bool corridor_blocked(const MapView& M, const ToolView& T, int4 d, const Pt& P,
                                         int lane) {
-  const DirRows D = dir_rows(M, P, d, T.strict != 0);
+  const DirRows D = dir_rows(M, P, d, STRICT);
   for (int b = lane; b - lane < D.nc; b += 32) {
     bool h = false;
     if (b < D.nc) {
       uint4 m;
       const uint4 o = quad_bits<FAST>(M, T, D, D.view, D.c0 + b, &m);
       h = (o.x | o.y | o.z | o.w) != 0u;
-      if (T.strict) {
+      if (STRICT) {
         const uint4 n = quad_bits<FAST>(M, T, D, M.known, D.c0 + b, &m);
         h = h || ((n.x ^ m.x) | (n.y ^ m.y) | (n.z ^ m.z) | (n.w ^ m.w)) != 0u;
       }
@@ -211,6 +211,24 @@ __device__ inline bool arm_clear(const MapView& M, const ToolView& T, int g, con
     clear &= (kn & ~oc) >> (x & 31);
   }
   return clear & 1u;
+}
+
+// Whether direction g (table entry d; one lane) is open at its start: its arm
+// samples are clear and, in the strict form, its nearest corridor entry holds no
+// unknown voxel. Beyond the cleared band most of a map's space is unknown, so that
+// entry blocks most strict corridors, 32 directions at a time and before anything
+// is counted. Left to the corridor walk, a warp step for each direction after its
+// tool count, strict scoring took 213 us per pine frame (12k points, 128
+// directions) and 2.71 ms for the 1 cm map with 512; with it and the order of
+// best_direction 67 us and 0.35 ms.
+template <bool FAST, bool STRICT>
+__device__ inline bool start_open(const MapView& M, const ToolView& T, int g, int4 d, const Pt& P) {
+  if (!arm_clear<FAST>(M, T, g, P)) return false;
+  if (!STRICT || d.w == 0) return true;
+  const DirRows D = dir_rows(M, P, d, true);
+  uint4 m;
+  const uint4 n = quad_bits<FAST>(M, T, D, M.known, D.c0, &m);
+  return ((n.x ^ m.x) | (n.y ^ m.y) | (n.z ^ m.z) | (n.w ^ m.w)) == 0u;
 }
 
 __device__ inline bool candidate(const ToolView& T, int g, float n0, float n1, float n2) {
@@ -254,42 +272,58 @@ __device__ __forceinline__ int4 shfl4(int4 v, int from) {
 // `gate()` is asked once, after the first screen (so that a load it waits for
 // overlaps the screen's): if it says no, (-1, -1) is returned.
 //
-// The arm screen takes 32 directions at a time. The arm-clear ones are then
+// The screen (start_open) takes 32 directions at a time. The open ones are then
 // counted kSide at a time, all against the score to beat before them, and
 // decided in index order: a count that reaches that score cannot beat any later
 // one, so the result is the sequential one. A score of 0 ends the search.
-template <bool FAST, class Cand, class Gate = NoGate>
+//
+// STRICT: until a direction is found, the corridor comes before the count. Most
+// strict corridors are blocked, and a count is only needed of one that is not.
+// A template parameter, not a branch on the tool: both forms in one search cost the
+// usual one 2 to 3%.
+template <bool FAST, bool STRICT, class Cand, class Gate = NoGate>
 __device__ inline int2 best_direction(const MapView& M, const ToolView& T, const Pt& P,
                                       const Cand& cand_of, int lane, const Gate& gate = Gate()) {
   const int nc = T.n_c;
   int bscore = nc + 1, best = -1, first = -1;  // best: of the unblocked directions
   for (int gb = 0; gb < T.G; gb += 32) {
-    // lane-parallel screen: candidates, and the arm samples of each candidate
+    // lane-parallel screen: candidates, and the start of each candidate
     const bool cand = cand_of(T, gb + lane);
     const unsigned mask = __ballot_sync(0xffffffffu, cand);
     if (first < 0 && mask) first = gb + __ffs(mask) - 1;
     const int4 dt = cand ? __ldg(T.dtab + gb + lane) : make_int4(0, 0, 0, 0);
-    unsigned rest = __ballot_sync(0xffffffffu, cand && arm_clear<FAST>(M, T, gb + lane, P));
+    unsigned rest = __ballot_sync(0xffffffffu, cand && start_open<FAST, STRICT>(M, T, gb + lane, dt, P));
     if (gb == 0 && !gate()) return make_int2(-1, -1);
     while (rest) {
-      // the next kSide arm-clear directions, one per group of lanes
-      unsigned mine = rest;
-#pragma unroll
-      for (int k = 1; k < kSide; ++k) {
-        if (lane >= k * kDirLanes) mine &= mine - 1u;
+      int at, c = 0;
+      unsigned todo;
+      const bool one = STRICT && best < 0;
+      if (one) {  // the next open direction, not counted yet
+        at = __ffs(rest) - 1;
         rest &= rest - 1u;
+        todo = 1u;
+      } else {
+        // the next kSide open directions, one per group of lanes
+        unsigned mine = rest;
+#pragma unroll
+        for (int k = 1; k < kSide; ++k) {
+          if (lane >= k * kDirLanes) mine &= mine - 1u;
+          rest &= rest - 1u;
+        }
+        rest &= rest - 1u;
+        at = mine ? __ffs(mine) - 1 : 0;
+        c = tool_counts<FAST>(M, T, mine != 0u, shfl4(dt, at), P, min(bscore, nc), lane);
+        todo = __ballot_sync(0xffffffffu, mine != 0u && (best < 0 || c < bscore) &&
+                                              (lane & (kDirLanes - 1)) == 0);
       }
-      rest &= rest - 1u;
-      const int at = mine ? __ffs(mine) - 1 : 0;
-      const int c = tool_counts<FAST>(M, T, mine != 0u, shfl4(dt, at), P, min(bscore, nc), lane);
-      unsigned todo = __ballot_sync(0xffffffffu, mine != 0u && (best < 0 || c < bscore) &&
-                                                     (lane & (kDirLanes - 1)) == 0);
       while (todo) {
         const int from = __ffs(todo) - 1;
         todo &= todo - 1u;
-        const int k = __shfl_sync(0xffffffffu, at, from), ck = __shfl_sync(0xffffffffu, c, from);
+        const int k = __shfl_sync(0xffffffffu, at, from);
+        int ck = __shfl_sync(0xffffffffu, c, from);
         if (best >= 0 && ck >= bscore) continue;  // beaten by one before it
-        if (corridor_blocked<FAST>(M, T, shfl4(dt, k), P, lane)) continue;
+        if (corridor_blocked<FAST, STRICT>(M, T, shfl4(dt, k), P, lane)) continue;
+        if (one) ck = tool_count<FAST>(M, T, gb + k, P, nc, lane);
         bscore = ck;
         best = gb + k;
         if (bscore == 0) return make_int2(0, best);
@@ -301,10 +335,10 @@ __device__ inline int2 best_direction(const MapView& M, const ToolView& T, const
 }
 
 // best_direction with a budget: at most `budget` directions are taken past
-// the arm screen (tool count and corridor). If the search stops early,
+// the screen (tool count and corridor). If the search stops early,
 // *next receives the first direction index not searched and the result is
 // exact over the directions before it; *next = -1 when the search finished.
-template <bool FAST, class Cand>
+template <bool FAST, bool STRICT, class Cand>
 __device__ inline int2 best_direction_budget(const MapView& M, const ToolView& T, const Pt& P,
                                              const Cand& cand_of, int lane, int budget,
                                              int* next) {
@@ -314,12 +348,14 @@ __device__ inline int2 best_direction_budget(const MapView& M, const ToolView& T
   for (int gb = 0; gb < T.G && bscore != 0; gb += 32) {
     const bool cand = cand_of(T, gb + lane);
     unsigned mask = __ballot_sync(0xffffffffu, cand);
-    const unsigned arm_ok = __ballot_sync(0xffffffffu, cand && arm_clear<FAST>(M, T, gb + lane, P));
+    const int4 dt = cand ? __ldg(T.dtab + gb + lane) : make_int4(0, 0, 0, 0);
+    const unsigned open =
+        __ballot_sync(0xffffffffu, cand && start_open<FAST, STRICT>(M, T, gb + lane, dt, P));
     while (mask) {
       const int bit = __ffs(mask) - 1;
       const int g = gb + bit;
       mask &= mask - 1u;
-      if (!((arm_ok >> bit) & 1u)) {
+      if (!((open >> bit) & 1u)) {
         if (best < 0) {
           bscore = nc + 1;
           best = g;
@@ -334,11 +370,11 @@ __device__ inline int2 best_direction_budget(const MapView& M, const ToolView& T
       if (bscore <= nc) {
         const int cnt = tool_count<FAST>(M, T, g, P, bscore, lane);
         if (cnt >= bscore) continue;
-        if (corridor_blocked<FAST>(M, T, __ldg(T.dtab + g), P, lane)) continue;
+        if (corridor_blocked<FAST, STRICT>(M, T, __ldg(T.dtab + g), P, lane)) continue;
         bscore = cnt;
         best = g;
       } else {
-        if (corridor_blocked<FAST>(M, T, __ldg(T.dtab + g), P, lane)) {
+        if (corridor_blocked<FAST, STRICT>(M, T, __ldg(T.dtab + g), P, lane)) {
           if (best < 0) {
             bscore = nc + 1;
             best = g;
