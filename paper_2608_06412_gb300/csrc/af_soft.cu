@@ -264,11 +264,11 @@ __device__ inline bool sample_cell(const SoftView& S, const PointCell& pc, const
 // comes from adding 1.5 2^23, which rounds to an integer kept in the low bits --
 // four single-precision operations at full rate in the place of a rounding and a
 // conversion at a quarter of it. `cb` is the point's cell less the view's base and
-// that constant's bits. Whether the cell lies inside the view is known from the
+// that constant's bits, modulo 2^32 (a point may lie 1e9 cells from the view). Whether the cell lies inside the view is known from the
 // sample's index (samples_near).
 constexpr float kRound = 12582912.0f;        // 1.5 2^23
-constexpr int kRoundBits = 0x4B400000;
-__device__ inline void sample_cell_near(const PointCell& pc, const Dir& d, const int cb[3], float t,
+constexpr unsigned kRoundBits = 0x4B400000u;
+__device__ inline void sample_cell_near(const PointCell& pc, const Dir& d, const unsigned cb[3], float t,
                                         float f[3], int c[3]) {
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -276,7 +276,7 @@ __device__ inline void sample_cell_near(const PointCell& pc, const Dir& d, const
     const float y0 = __fadd_rn(l, kRound), y = __fsub_rn(y0, kRound);
     const bool up = y > l;  // rounded up: the floor is one below
     f[i] = l - (up ? y - 1.0f : y);
-    c[i] = __float_as_int(y0) + cb[i] - (up ? 1 : 0);
+    c[i] = (int)(__float_as_uint(y0) + cb[i] - (up ? 1u : 0u));
   }
 }
 
@@ -287,7 +287,7 @@ __device__ inline void sample_cell_near(const PointCell& pc, const Dir& d, const
 // bisection. (Pairs that leave the view are ordinary -- every third one where the
 // map box ends half a metre behind the surfaces.)
 template <bool SPARSE>
-__device__ inline bool samples_near(const SoftView& S, const PointCell& pc, const Dir& d, int cb[3],
+__device__ inline bool samples_near(const SoftView& S, const PointCell& pc, const Dir& d, unsigned cb[3],
                                     int* last) {
   bool near = pc.ok;
 #pragma unroll
@@ -297,7 +297,7 @@ __device__ inline bool samples_near(const SoftView& S, const PointCell& pc, cons
     for (int i = 0; i < 3; ++i) near = near && fabsf(sample_pos(pc, d, t, i)) < 4.0e6f;
   }
 #pragma unroll
-  for (int i = 0; i < 3; ++i) cb[i] = (int)pc.I[i] - (SPARSE ? S.glo[i] : S.lo[i]) - kRoundBits;
+  for (int i = 0; i < 3; ++i) cb[i] = (unsigned)(int)pc.I[i] - (unsigned)(SPARSE ? S.glo[i] : S.lo[i]) - kRoundBits;
   const auto inside = [&](int j) {
     float f[3];
     int c[3];
@@ -490,7 +490,7 @@ constexpr int kInFlightRefineFew = 4;  // of few pairs, which wait for latency o
 // the pairs that leave 142 to 147.
 template <bool NEAR, bool GRAD, bool FIXED, bool SPARSE, int NF>
 __device__ inline void fold_samples(Softmin<GRAD, FIXED>& sm, const SoftView& S, const PointCell& pc,
-                                    const Dir& d, const int cb[3], int last, int g) {
+                                    const Dir& d, const unsigned cb[3], int last, int g) {
 #pragma unroll 1
   for (int j = S.j0 + g; j <= S.J; j += NF * kLanes) {
     float f[NF][3];
@@ -560,7 +560,8 @@ __device__ inline float soft_eval(const SoftView& S, const PointCell& pc, const 
                                   float* ga, float* gb, float* gh, float* cmin, bool* far) {
   Softmin<GRAD, FIXED> sm;
   if (live) {
-    int cb[3] = {0, 0, 0}, last = 0;
+    unsigned cb[3] = {0u, 0u, 0u};
+    int last = 0;
     if (ROAD != kGeneral && samples_near<SPARSE>(S, pc, d, cb, &last))
       fold_samples<true, GRAD, FIXED, SPARSE, NF>(sm, S, pc, d, cb, last, g);
     else if (ROAD == kNear)

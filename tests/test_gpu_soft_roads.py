@@ -41,3 +41,28 @@ def test_refinement_does_not_depend_on_the_calls_size(view, tau_s, steps):
     for w, p in zip(whole, map(torch.cat, zip(*parts))):
         assert torch.equal(torch.nan_to_num(w, nan=1e9), torch.nan_to_num(p, nan=1e9))
     assert steps < 20 or (whole[0] != par[0]).sum() > N // 50
+
+
+@pytest.mark.parametrize("view", [1, 2])
+def test_points_far_beyond_the_view_read_tau(view):
+    """Cells up to 1e9 voxels from the box on either side: every sample reads
+    tau, as for a pair that just leaves the box."""
+    import torch
+    W = workload.single_frame()
+    m = af.Map(W.af_config(**CAPS))
+    m.set_tool(W.af_tool(), W.dirs)
+    m.soft_set_view(view)
+    f = synth.cone_frame(W.scene, 3000, 0.01, 51)
+    m.integrate_scan(torch.from_numpy(f.pts).cuda(), f.pose)
+    far = [s * k * W.params["v"] for k in (9.9e8, 8.9e8, 7.0e8, 1e6, 2e3) for s in (1.0, -1.0)]
+    pts = torch.tensor([[x if a == k else 1.0 for a in range(3)] for x in far for k in range(3)],
+                       dtype=torch.float32, device="cuda")
+    n = len(pts)
+    u0 = torch.tensor([0.0, 0.0, 1.0], device="cuda").repeat(n, 1).contiguous()
+    z = torch.zeros(n, device="cuda")
+    cmin = torch.empty(n, device="cuda")
+    c = m.soft_clearance_raw(pts, u0, z, z, z, 1, cmin=cmin)
+    tool = W.af_tool()
+    want = torch.tensor(W.params["tau"], dtype=torch.float32) - \
+        torch.tensor(max(tool.radius, tool.corr_radius), dtype=torch.float32)
+    assert (cmin == want.item()).all() and (c == c[0]).all()
