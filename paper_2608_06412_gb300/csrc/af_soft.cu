@@ -283,44 +283,57 @@ __device__ inline void sample_cell_near(const PointCell& pc, const Dir& d, const
 // Whether every sample j0..J lies within 2^22 voxels of the point and the first
 // one inside the view; then the constants of sample_cell_near and the last sample
 // inside the view. Rounding is monotone, so on each axis the samples' cells go one
-// way: a pair's samples inside the view are the first ones, up to one found by
-// bisection. (Pairs that leave the view are ordinary -- every third one where the
-// map box ends half a metre behind the surfaces.)
+// way: a pair's samples inside the view are the first ones. (Pairs that leave the
+// view are ordinary -- every third one where the map box ends half a metre behind
+// the surfaces.)
+//
+// A cell lies inside the view when the sample's position lies between the view's
+// faces in the point's frame, whole numbers of cells: two comparisons an axis. (A
+// face beyond 2^24 may be rounded; positions within 2^22 compare with it all the
+// same.) Where the axis crosses a face is one division for each face that the last
+// sample is beyond; the sample before it is then checked, and its neighbours until
+// one is inside and the next is not.
 template <bool SPARSE>
 __device__ inline bool samples_near(const SoftView& S, const PointCell& pc, const Dir& d, unsigned cb[3],
                                     int* last) {
-  bool near = pc.ok;
+  float face0[3], face1[3];
 #pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const float t = __fadd_rn(d.e, (float)(e ? S.J : S.j0));
-#pragma unroll
-    for (int i = 0; i < 3; ++i) near = near && fabsf(sample_pos(pc, d, t, i)) < 4.0e6f;
+  for (int i = 0; i < 3; ++i) {
+    const unsigned c0 = (unsigned)(int)pc.I[i] - (unsigned)(SPARSE ? S.glo[i] : S.lo[i]);
+    cb[i] = c0 - kRoundBits;
+    face0[i] = (float)(int)(0u - c0);
+    face1[i] = (float)(int)((unsigned)(SPARSE ? 8 * S.gdim[i] : S.ncell[i]) - c0);
   }
-#pragma unroll
-  for (int i = 0; i < 3; ++i) cb[i] = (unsigned)(int)pc.I[i] - (unsigned)(SPARSE ? S.glo[i] : S.lo[i]) - kRoundBits;
   const auto inside = [&](int j) {
-    float f[3];
-    int c[3];
-    sample_cell_near(pc, d, cb, __fadd_rn(d.e, (float)j), f, c);
+    const float t = __fadd_rn(d.e, (float)j);
     bool in = true;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) in = in && (unsigned)c[i] < (unsigned)(SPARSE ? 8 * S.gdim[i] : S.ncell[i]);
+    for (int i = 0; i < 3; ++i) {
+      const float l = sample_pos(pc, d, t, i);
+      in = in && l >= face0[i] && l < face1[i];
+    }
     return in;
   };
-  if (!near || !inside(S.j0)) return false;
-  int lo = S.j0, hi = S.J;
-  if (inside(hi)) {
-    lo = hi;
-  } else {
-    while (hi - lo > 1) {  // lo inside, hi outside
-      const int mid = (lo + hi) >> 1;
-      if (inside(mid))
-        lo = mid;
-      else
-        hi = mid;
+  bool ok = pc.ok, in = true;
+  float exit = (float)S.J;  // where the axis leaves the view, in samples
+  const float t0 = __fadd_rn(d.e, (float)S.j0), t1 = __fadd_rn(d.e, (float)S.J);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const float l0 = sample_pos(pc, d, t0, i), l1 = sample_pos(pc, d, t1, i);
+    ok = ok && fabsf(l0) < 4.0e6f && fabsf(l1) < 4.0e6f && l0 >= face0[i] && l0 < face1[i];
+    if (l1 < face0[i] || l1 >= face1[i]) {
+      in = false;
+      exit = fminf(exit, __fdividef((l1 < face0[i] ? face0[i] : face1[i]) - pc.r[i], d.u[i]) - d.e);
     }
   }
-  *last = lo;
+  if (!ok) return false;
+  int j = S.J;
+  if (!in) {
+    j = max(S.j0, min(S.J - 1, (int)exit));
+    while (j > S.j0 && !inside(j)) --j;
+    while (j + 1 < S.J && inside(j + 1)) ++j;
+  }
+  *last = j;
   return true;
 }
 
@@ -472,9 +485,13 @@ __device__ inline float trilinear(const float4& lo, const float4& hi, const floa
 constexpr int kInFlightField = 2;
 constexpr int kInFlightRefine = 3;
 constexpr int kInFlightRefineFew = 4;  // of few pairs, which wait for latency only
+constexpr int kInFlightRefineMid = 3;  // of as many as three CTAs per SM hold
+constexpr int kInFlightGeneral = 3;
+constexpr int kInFlightGeneralWide = 4;
 
 // Folds lane g's samples j0 + g, j0 + g + kLanes, ... into sm. NEAR: every sample
-// lies near the point, those up to `last` inside the view (samples_near).
+// lies near the point, those up to `last` inside the view (samples_near); otherwise
+// each sample is checked (launch_soft_form says when).
 //
 // Most samples of a 1.25 m axis read nothing but tau (78% of those of a finished
 // pine map), so the dense view's records are only read in blocks of cells that
@@ -483,11 +500,8 @@ constexpr int kInFlightRefineFew = 4;  // of few pairs, which wait for latency o
 // With the checks of the cells gone as well, the field of a finished map's 30k
 // points (1.9M pairs) went from 862 to about 490 us, forward plus adjoint of 113k
 // pairs from 149 to 72 us, the refinement of 30k pairs from 315 to 235 us. In a
-// small box (0.17 GB of records, which the caches hold; 350k pairs, a third of
-// which leave the view) the field takes 109 against 101 us: the bisection is paid
-// once per evaluation. Without the marks there 112, with per-sample checks in its
-// place 105 (but 285 against 252 us for the refinement), by the general way for
-// the pairs that leave 142 to 147.
+// small box (0.17 GB of records, which the caches hold) they gain nothing: 512k
+// pairs, a third of which leave the view, take 127 us either way.
 template <bool NEAR, bool GRAD, bool FIXED, bool SPARSE, int NF>
 __device__ inline void fold_samples(Softmin<GRAD, FIXED>& sm, const SoftView& S, const PointCell& pc,
                                     const Dir& d, const unsigned cb[3], int last, int g) {
@@ -511,7 +525,7 @@ __device__ inline void fold_samples(Softmin<GRAD, FIXED>& sm, const SoftView& S,
       }
       record_of<SPARSE>(S, c, &id[q], &loc[q]);
       rec[q] = id[q];
-      if (!SPARSE) {
+      if (!SPARSE && NEAR) {
         const uint32_t b = ((uint32_t)(c[2] >> 3) * (uint32_t)S.nblock[1] + (uint32_t)(c[1] >> 3)) *
                                (uint32_t)S.nblock[0] + (uint32_t)(c[0] >> 3);
         mark[q] = in[q] ? __ldg(S.seen + (b >> 5)) : 0u;
@@ -527,7 +541,7 @@ __device__ inline void fold_samples(Softmin<GRAD, FIXED>& sm, const SoftView& S,
         in[q] = in[q] && slot[q] != kNoBlock;
         rec[q] = (size_t)slot[q] * kBrickVox + loc[q];
       }
-    } else {
+    } else if (NEAR) {
 #pragma unroll
       for (int q = 0; q < NF; ++q) in[q] = (mark[q] >> (bit[q] & 31u)) & 1u;
     }
@@ -548,8 +562,9 @@ __device__ inline void fold_samples(Softmin<GRAD, FIXED>& sm, const SoftView& S,
 
 // How a kernel takes its samples: the short way for every pair whose samples lie
 // near its point and the general way for the others (kBoth), the others not at all
-// (kNear: *far is set instead), every pair the general way (kGeneral).
-enum Road { kBoth, kNear, kGeneral };
+// (kNear: *far is set instead), every pair the general way (kGeneral; kRedo: those
+// that a kNear launch has left).
+enum Road { kBoth, kNear, kGeneral, kRedo };
 
 // C of one pair and, with GRAD, dC / d(alpha, beta, h); *cmin = min_j phi_j.
 // Called by all kLanes lanes of the pair's group (lane g of it); with
@@ -562,12 +577,12 @@ __device__ inline float soft_eval(const SoftView& S, const PointCell& pc, const 
   if (live) {
     unsigned cb[3] = {0u, 0u, 0u};
     int last = 0;
-    if (ROAD != kGeneral && samples_near<SPARSE>(S, pc, d, cb, &last))
+    if ((ROAD == kBoth || ROAD == kNear) && samples_near<SPARSE>(S, pc, d, cb, &last))
       fold_samples<true, GRAD, FIXED, SPARSE, NF>(sm, S, pc, d, cb, last, g);
     else if (ROAD == kNear)
       *far = true;
     else
-      fold_samples<false, GRAD, FIXED, SPARSE, ROAD == kGeneral ? NF : 1>(sm, S, pc, d, cb, 0, g);
+      fold_samples<false, GRAD, FIXED, SPARSE, ROAD == kBoth ? 1 : NF>(sm, S, pc, d, cb, 0, g);
   }
   sm.reduce(S.k2);
   const float C = (FIXED ? S.ref : sm.m) - S.ln2_tau_s * lg2(sm.Z);
@@ -630,7 +645,7 @@ struct GroupWalk {
   }
 };
 
-template <bool GRAD, bool FIXED, bool SPARSE>
+template <bool GRAD, bool FIXED, bool SPARSE, Road ROAD, int NF>
 __global__ void __launch_bounds__(128) k_soft(SoftView S, const float* __restrict__ pts,
                                               uint32_t per_point, const float* __restrict__ u0,
                                               const float* __restrict__ alpha,
@@ -652,8 +667,8 @@ __global__ void __launch_bounds__(128) k_soft(SoftView S, const float* __restric
     const Dir d = make_dir(S, u, t1, t2, __ldg(alpha + i), __ldg(beta + i), __ldg(hh + i));
     const bool fin = pc.finite && d.finite;
     float da, db, dh, mn;
-    float C = soft_eval<GRAD, FIXED, SPARSE, kInFlightField, kBoth>(S, pc, d, t1, t2, fin && act, w.g,
-                                                                    &da, &db, &dh, &mn, nullptr);
+    float C = soft_eval<GRAD, FIXED, SPARSE, NF, ROAD>(S, pc, d, t1, t2, fin && act, w.g, &da, &db, &dh,
+                                                       &mn, nullptr);
     if (!act || w.g != 0) continue;
     if (!fin) C = mn = da = db = dh = NAN;
     if (c) c[i] = C;
@@ -717,10 +732,10 @@ __device__ inline bool refine_pair(const SoftView& S, const RefineArgs& R, const
 // registers, so the first (ROAD kNear) leaves a pair that it cannot take
 // (samples_near) as it was and marks its C with a NaN of its own, and the second
 // takes the marked pairs from their start again.
-constexpr unsigned kRedo = 0x7FC05EDDu;
+constexpr unsigned kRedoMark = 0x7FC05EDDu;
 
-template <bool FIXED, bool SPARSE, Road ROAD, int NF>
-__global__ void __launch_bounds__(128, ROAD == kBoth ? 2 : 4) k_soft_refine(SoftView S, RefineArgs R,
+template <bool FIXED, bool SPARSE, Road ROAD, int NF, int CTAS>
+__global__ void __launch_bounds__(128, CTAS) k_soft_refine(SoftView S, RefineArgs R,
                                                      const float* __restrict__ pts,
                                                      uint32_t per_point,
                                                      const float* __restrict__ u0,
@@ -734,13 +749,13 @@ __global__ void __launch_bounds__(128, ROAD == kBoth ? 2 : 4) k_soft_refine(Soft
     const size_t i0 = base + w.slot;
     bool act = i0 < n;
     const size_t i = act ? i0 : n - 1;
-    if (ROAD == kGeneral) {
-      act = act && __float_as_uint(c[i]) == kRedo;
+    if (ROAD == kRedo) {
+      act = act && __float_as_uint(c[i]) == kRedoMark;
       if (!__any_sync(kFull, act)) continue;
     }
     if (!refine_pair<FIXED, SPARSE, NF, ROAD>(
             S, R, pts, per_point, u0, alpha, beta, hh, c, cmin, i, act, w.g) && act && w.g == 0)
-      c[i] = __uint_as_float(kRedo);
+      c[i] = __uint_as_float(kRedoMark);
   }
 }
 
@@ -931,27 +946,96 @@ cudaError_t launch_soft_seed(const float* d_nrm, uint32_t m, const float* d_tabl
   return cudaGetLastError();
 }
 
+// Which way the samples go, by their number per pair. The short way costs each
+// evaluation about as much as four samples a lane (the view's faces, the last
+// sample inside) and spares a quarter of each sample's work, so few samples go the
+// general way. In a box whose records the caches hold the marks spare nothing as
+// well, and the line lies higher; without marks (sparse view) it lies lower, since
+// the general way has a slot to read for every sample. Field of 512k pairs with 8 / 12
+// / 20 / 28 / 36 / 62 samples, short against general way: in the pine's dense view
+// 49 / 59 / 74 / 88 / 102 / 137 us against 45 / 49 / 67 / 94 / 119 / 243; in a box of
+// 0.17 GB of records 49 / 59 / 70 / 81 / 92 / 127 against 46 / 50 / 63 / 77 / 86 / 127;
+// in the sparse view 50 / 61 / 77 / 93 / 108 / 153 against 51 / 58 / 78 / 97 / 110 / 160.
+constexpr int kGeneralBelow = 25, kGeneralBelowSmallBox = 49, kGeneralBelowSparse = 17;
+constexpr uint64_t kSmallBoxCells = 1ull << 23;  // 0.25 GB of records
+
+template <bool GRAD, bool FIXED, bool SPARSE>
+static void launch_soft_form(const SoftView& S, const float* pts, uint32_t per_point, const float* u0,
+                             const float* al, const float* be, const float* h, uint64_t n,
+                             const float* gc, float* c, float* cmin, float* ga, float* gb, float* gh,
+                             int num_sms, cudaStream_t stream) {
+  const int samples = S.J - S.j0 + 1;
+  const bool small = (uint64_t)S.ncell[0] * S.ncell[1] * S.ncell[2] <= kSmallBoxCells;
+  const unsigned g = grid_for(n * kLanes, 128, num_sms, 16);
+  const auto run = [&](auto kernel) {
+    kernel<<<g, 128, 0, stream>>>(S, pts, per_point, u0, al, be, h, n, gc, c, cmin, ga, gb, gh);
+  };
+  if (samples < (SPARSE ? kGeneralBelowSparse : small ? kGeneralBelowSmallBox : kGeneralBelow))
+    run(k_soft<GRAD, FIXED, SPARSE, kGeneral, kInFlightGeneral>);
+  else
+    run(k_soft<GRAD, FIXED, SPARSE, kBoth, kInFlightField>);
+}
+
 cudaError_t launch_soft(const SoftView& S, bool grad, const float* pts, uint32_t per_point,
                         const float* u0, const float* al, const float* be, const float* h,
                         uint64_t n, const float* gc, float* c, float* cmin, float* ga,
                         float* gb, float* gh, int num_sms, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
-  const unsigned g = grid_for(n * kLanes, 128, num_sms, 16);
-#define AF_SOFT_LAUNCH(GR, FX)                                                                  \
-  (S.sparse ? k_soft<GR, FX, true><<<g, 128, 0, stream>>>(S, pts, per_point, u0, al, be, h, n, gc, \
-                                                         c, cmin, ga, gb, gh)                    \
-            : k_soft<GR, FX, false><<<g, 128, 0, stream>>>(S, pts, per_point, u0, al, be, h, n,   \
-                                                          gc, c, cmin, ga, gb, gh))
-  if (grad && S.fixed)
-    AF_SOFT_LAUNCH(true, true);
-  else if (grad)
-    AF_SOFT_LAUNCH(true, false);
-  else if (S.fixed)
-    AF_SOFT_LAUNCH(false, true);
-  else
-    AF_SOFT_LAUNCH(false, false);
-#undef AF_SOFT_LAUNCH
+  decltype(&launch_soft_form<false, false, false>) form =
+      grad ? (S.fixed ? (S.sparse ? launch_soft_form<true, true, true> : launch_soft_form<true, true, false>)
+                      : (S.sparse ? launch_soft_form<true, false, true> : launch_soft_form<true, false, false>))
+           : (S.fixed ? (S.sparse ? launch_soft_form<false, true, true> : launch_soft_form<false, true, false>)
+                      : (S.sparse ? launch_soft_form<false, false, true>
+                                  : launch_soft_form<false, false, false>));
+  form(S, pts, per_point, u0, al, be, h, n, gc, c, cmin, ga, gb, gh, num_sms, stream);
   return cudaGetLastError();
+}
+
+// Refinement, by the samples per pair as above (its evaluations carry gradients, so
+// a sample spared counts for more) and by how many pairs the chip holds at once.
+//  * Few samples: the general way, four records in flight and three CTAs per SM, or
+//    three and four where that takes a wave less. 14k pairs with 8 / 12 / 20 samples:
+//    47 / 52 / 67 us, the short way in two launches 56 / 60 / 74; 15k pairs 52 / 57 /
+//    74, in two waves of three CTAs 69 / 75 / 99.
+//  * In the dense view up to 32 samples, two rounds of four a lane: the same, if it
+//    takes no wave more and the pairs are more than the next form holds (10k pairs
+//    with 28 samples 69 against 80 us).
+//  * As many pairs as two CTAs per SM hold: latency is all that counts, four records
+//    in flight, both ways in one kernel (220 registers).
+//  * As many as three CTAs per SM hold: both ways in one kernel of three records
+//    in flight (12k pairs of a small box with 62 samples 109 us, in two launches 113).
+//  * More: the short way in four CTAs per SM, and a second launch for what it left
+//    (25k pairs on the pine map 219 us).
+constexpr int kRefineGeneralBelow = 25, kRefineGeneralBelowSparse = 9, kRefineWideBelow = 33;
+
+template <bool FIXED, bool SPARSE>
+static void launch_refine_form(const SoftView& S, const RefineArgs& R, const float* pts,
+                               uint32_t per_point, const float* u0, float* al, float* be, float* h,
+                               uint64_t n, float* c, float* cmin, int num_sms, cudaStream_t stream) {
+  const int samples = S.J - S.j0 + 1;
+  const unsigned g = grid_for(n * kLanes, 128, num_sms, 16);
+  const auto waves = [&](int ctas) {
+    const uint64_t held = (uint64_t)num_sms * ctas * (128 / kLanes);
+    return (n + held - 1) / held;
+  };
+  const auto run = [&](auto kernel) {
+    kernel<<<g, 128, 0, stream>>>(S, R, pts, per_point, u0, al, be, h, n, c, cmin);
+  };
+  const int few_samples = SPARSE ? kRefineGeneralBelowSparse : kRefineGeneralBelow;
+  const bool wide = waves(3) == waves(4);
+  if (samples < few_samples && !wide) {
+    run(k_soft_refine<FIXED, SPARSE, kGeneral, kInFlightGeneral, 4>);
+  } else if (wide && (samples < few_samples ||
+                      (!SPARSE && samples < kRefineWideBelow && waves(2) > 1))) {
+    run(k_soft_refine<FIXED, SPARSE, kGeneral, kInFlightGeneralWide, 3>);
+  } else if (waves(2) == 1) {
+    run(k_soft_refine<FIXED, SPARSE, kBoth, kInFlightRefineFew, 2>);
+  } else if (waves(3) == 1) {
+    run(k_soft_refine<FIXED, SPARSE, kBoth, kInFlightRefineMid, 3>);
+  } else {
+    run(k_soft_refine<FIXED, SPARSE, kNear, kInFlightRefine, 4>);
+    run(k_soft_refine<FIXED, SPARSE, kRedo, 1, 4>);
+  }
 }
 
 cudaError_t launch_soft_refine(const SoftView& S, const RefineArgs& R, const float* pts,
@@ -959,30 +1043,10 @@ cudaError_t launch_soft_refine(const SoftView& S, const RefineArgs& R, const flo
                                float* h, uint64_t n, float* c, float* cmin, int num_sms,
                                cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
-  const unsigned g = grid_for(n * kLanes, 128, num_sms, 16);
-  // fewer pairs than the wide kernel holds at once: latency is all that counts
-  const bool few = n <= (uint64_t)num_sms * 2 * (128 / kLanes);
-#define AF_REFINE_ROAD(FX, SP, RD, NF) \
-  k_soft_refine<FX, SP, RD, NF><<<g, 128, 0, stream>>>(S, R, pts, per_point, u0, al, be, h, n, c, cmin)
-#define AF_REFINE_LAUNCH(FX, SP)                            \
-  do {                                                      \
-    if (few) {                                              \
-      AF_REFINE_ROAD(FX, SP, kBoth, kInFlightRefineFew);    \
-    } else {                                                \
-      AF_REFINE_ROAD(FX, SP, kNear, kInFlightRefine);       \
-      AF_REFINE_ROAD(FX, SP, kGeneral, 1);                  \
-    }                                                       \
-  } while (0)
-  if (S.fixed && S.sparse)
-    AF_REFINE_LAUNCH(true, true);
-  else if (S.fixed)
-    AF_REFINE_LAUNCH(true, false);
-  else if (S.sparse)
-    AF_REFINE_LAUNCH(false, true);
-  else
-    AF_REFINE_LAUNCH(false, false);
-#undef AF_REFINE_LAUNCH
-#undef AF_REFINE_ROAD
+  decltype(&launch_refine_form<false, false>) form =
+      S.fixed ? (S.sparse ? launch_refine_form<true, true> : launch_refine_form<true, false>)
+              : (S.sparse ? launch_refine_form<false, true> : launch_refine_form<false, false>);
+  form(S, R, pts, per_point, u0, al, be, h, n, c, cmin, num_sms, stream);
   return cudaGetLastError();
 }
 
