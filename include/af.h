@@ -43,7 +43,10 @@
  *  - Fault injection for tests: when the environment variable
  *    AF_FAIL_ALLOC_AT holds k >= 0, af_create's k-th device allocation
  *    (counting from 0) fails as if the device were out of memory: af_create
- *    frees what it allocated and returns AF_ERR_CUDA.
+ *    frees what it allocated and returns AF_ERR_CUDA. AF_DRAW_LIST, read by
+ *    af_points_enable, shortens the list that the draw of changed voxels goes
+ *    through (1 .. 32768, its length without the variable), so that ordinary
+ *    draws overflow it; the points are the same.
  */
 #ifndef AF_H
 #define AF_H

@@ -66,6 +66,7 @@ struct af_ctx {
   uint32_t* d_phist = nullptr;
   af::PtSample* d_psamp = nullptr;
   af::PtDrawn* d_pdrawn = nullptr;
+  uint32_t draw_list = 0;        // its length
   uint32_t pts_frames = 0;       // af_points_frame calls (the draw's salt)
   bool pts_snapshot = false;     // af_integrate_scan copies the dirty bricks after allocation
   uint32_t* d_psel = nullptr;

@@ -334,7 +334,8 @@ struct PtView {
   uint32_t* chgmask;          // per dirty brick: 512 bits, voxels whose state changed
   uint32_t* hist;             // 2048 bins of the draw's radix selection
   PtSample* samp;
-  PtDrawn* drawn;             // kDrawList candidates
+  PtDrawn* drawn;             // draw_list candidates
+  uint32_t draw_list;
   int trig_exact;             // 1: changed voxels within trig_radius; 0: touched bricks
   int trig_radius;
   uint32_t trig_sample;       // changed voxels drawn per frame (0: all)

@@ -44,6 +44,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <vector>
 
@@ -189,11 +190,7 @@ __device__ inline int draw_lo(int pass) { return max(0, 64 - kDrawBits * (pass +
 // itself).
 constexpr uint32_t kDrawSample = 4096;
 constexpr uint32_t kBinList = kDrawBins / 2;  // hashes of the bound's bin in shared memory
-#ifdef AF_CHECKED
-constexpr uint32_t kDrawList = 64;  // the checked build's draws of 256 overflow it
-#else
 constexpr uint32_t kDrawList = 32768;
-#endif
 
 // The digit of the bin that holds the `need`-th smallest of the histogrammed
 // hashes, and the count before it and in it (1024 threads, 2 bins each; the CTA
@@ -285,7 +282,7 @@ __global__ void __launch_bounds__(1024) k_pts_diff(MapView M, PtView V, int draw
     S->t = ~0ull;
     S->prefix = all ? kDrawBins - 1 : digit;
     S->below = before;
-    S->listed = all ? n <= kDrawList : before + cnt <= kDrawList && cnt <= kBinList;
+    S->listed = all ? n <= V.draw_list : before + cnt <= V.draw_list && cnt <= kBinList;
     V.C->ndrawn = 0;
   }
 }
@@ -313,13 +310,13 @@ __global__ void __launch_bounds__(1024) k_pts_collect(MapView M, PtView V) {
       const unsigned long long h = mix64(draw_key(M, x, y, z) ^ V.salt);
       if ((h >> draw_lo(0)) > prefix) continue;
       const uint32_t at = atomicAdd(&V.C->ndrawn, 1u);
-      if (at < kDrawList) V.drawn[at] = PtDrawn{h, d * (uint32_t)kBrickVox + (uint32_t)l, 0u};
+      if (at < V.draw_list) V.drawn[at] = PtDrawn{h, d * (uint32_t)kBrickVox + (uint32_t)l, 0u};
     }
   if (!last_cta(&V.C->ended) || done) return;
   const uint32_t need = V.trig_sample - S->below;
   if (listed) {
     // the bin's candidates, in shared memory
-    const uint32_t n = min(__ldcg(&V.C->ndrawn), kDrawList);
+    const uint32_t n = min(__ldcg(&V.C->ndrawn), V.draw_list);
     if (threadIdx.x == 0) s_bin = 0;
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < n; i += 1024) {
@@ -487,7 +484,7 @@ __global__ void __launch_bounds__(256) k_pts_scatter_list(MapView M, PtView V) {
   uint32_t w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (S->listed) {
     const unsigned long long t = S->t;
-    const uint32_t n = min(V.C->ndrawn, kDrawList);
+    const uint32_t n = min(V.C->ndrawn, V.draw_list);
     for (; w < n; w += warps) {
       const PtDrawn c = V.drawn[w];
       if (c.h > t) continue;
@@ -1074,6 +1071,7 @@ PtView pt_view(af_ctx* ctx) {
   V.hist = ctx->d_phist;
   V.samp = ctx->d_psamp;
   V.drawn = ctx->d_pdrawn;
+  V.draw_list = ctx->draw_list;
   V.trig_exact = c.trig_exact;
   V.trig_radius = c.trig_radius;
   V.trig_sample = c.trig_sample;
@@ -1190,7 +1188,11 @@ extern "C" af_status af_points_enable(af_ctx* ctx, const af_points_config* cfg) 
     if (e == cudaSuccess) e = alloc((void**)&ctx->d_pchgmask, B * 16 * 4, 0);
     if (e == cudaSuccess) e = alloc((void**)&ctx->d_phist, af::kDrawBins * 4, 0);
     if (e == cudaSuccess) e = alloc((void**)&ctx->d_psamp, sizeof(af::PtSample), 0);
-    if (e == cudaSuccess) e = alloc((void**)&ctx->d_pdrawn, af::kDrawList * sizeof(af::PtDrawn), 0);
+    // for tests: a shorter list (AF_DRAW_LIST), so that ordinary draws overflow it
+    ctx->draw_list = af::kDrawList;
+    if (const char* v = std::getenv("AF_DRAW_LIST"))
+      ctx->draw_list = (uint32_t)std::clamp<long>(std::strtol(v, nullptr, 10), 1, af::kDrawList);
+    if (e == cudaSuccess) e = alloc((void**)&ctx->d_pdrawn, ctx->draw_list * sizeof(af::PtDrawn), 0);
   }
   if (e == cudaSuccess) e = alloc((void**)&ctx->d_psel, P * 4, 0);
   if (e == cudaSuccess) e = alloc((void**)&ctx->d_pblock, nblocks * 4, 0);
