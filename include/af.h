@@ -388,7 +388,7 @@ af_status af_soft_clearance_adjoint(af_ctx *ctx, const float *d_pts, uint32_t pe
                                     float *d_c, float *d_ga, float *d_gb, float *d_gh,
                                     void *stream);
 
-/* R->steps gradient-ascent steps on C for every pair in one launch (alpha,
+/* R->steps gradient-ascent steps on C for every pair in one call (alpha,
  * beta, h updated in place), then C (and, if d_cmin is given, the hard
  * clearance) at the final state. */
 af_status af_soft_refine(af_ctx *ctx, const float *d_pts, uint32_t per_point, const float *d_u0,
@@ -520,9 +520,12 @@ af_status af_points_export(af_ctx *ctx, uint32_t cap, int32_t *h_ijk, float *h_n
  * 8 = seeding (af_soft_seed, af_soft_start), 9 = per-point best.
  * af_profile_read synchronises, sums the elapsed times of the recorded
  * launches (milliseconds) and, if `reset`, forgets them. launches[] counts
- * kernels: an af_score call with work sharing on is three (k_score,
- * k_score_split, k_score_finish) timed as one bracket, an af_soft_refine call
- * two (all pairs, then those whose samples lie very far from their point).
+ * kernels, one bracket may hold several: an af_score call with work sharing on
+ * is three (k_score, k_score_split, k_score_finish), a projective integration
+ * two, an update of the dense SDF view three (five with its first fill), an
+ * af_soft_refine call one, or two for more pairs than the chip holds at once
+ * (all pairs, then those of whose samples one step found the first outside the
+ * view or very far from its point).
  */
 typedef struct {
     uint64_t launches[10];

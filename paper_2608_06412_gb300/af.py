@@ -550,7 +550,7 @@ class Map:
 
     def soft_refine(self, pts, u0, alpha, beta, h, per_point=1, steps=20, lr_dir=0.05,
                     lr_h=0.005, h_max=0.05, tau_s=TAU_S, out=None, stream=None):
-        """af_soft_refine: `steps` ascent steps on every pair in one launch;
+        """af_soft_refine: `steps` ascent steps on every pair in one call;
         alpha, beta, h are updated in place. Returns (C, hard clearance)."""
         torch = _import_torch()
         n, ptr = self._pair_ptrs(pts, u0, alpha, beta, h, per_point)

@@ -5,7 +5,6 @@
 #include <af.h>
 
 #include <algorithm>
-#include <array>
 #include <climits>
 #include <cmath>
 #include <cstdarg>
@@ -32,7 +31,7 @@ cudaError_t launch_score(const MapView& M, const ToolView& T, const float* d_pts
 cudaError_t launch_export_flags(const MapView& M, uint32_t count, uint8_t* d_flags,
                                 cudaStream_t stream);
 cudaError_t launch_views(const MapView& M, int num_sms, bool fill, float* dense, float4* cells,
-                         uint32_t* list, uint32_t* seen, cudaStream_t stream);
+                         uint32_t* list, uint32_t* seen, int* kernels, cudaStream_t stream);
 size_t view_list_words(const MapView& M);
 size_t seen_words(const MapView& M);
 cudaError_t launch_soft_seed(const float* d_nrm, uint32_t m, const float* d_table, uint32_t K,
@@ -44,7 +43,7 @@ cudaError_t launch_soft(const SoftView& S, bool grad, const float* pts, uint32_t
 cudaError_t launch_soft_refine(const SoftView& S, const RefineArgs& R, const float* pts,
                                uint32_t per_point, const float* u0, float* al, float* be,
                                float* h, uint64_t n, float* c, float* cmin, int num_sms,
-                               cudaStream_t stream);
+                               int* kernels, cudaStream_t stream);
 cudaError_t launch_soft_best(const float* c, uint64_t n, uint32_t per_point, const float* u0,
                              int32_t* best_k, float* best_c, float* best_u0, int num_sms,
                              cudaStream_t stream);
@@ -74,14 +73,16 @@ cudaEvent_t take_event(af_ctx* c) {
   return e;
 }
 
-// Runs `launch` on `s`, bracketed by events when profiling is on.
+// Runs `launch` on `s`, bracketed by events when profiling is on. `kernels`: the
+// kernels it launches, as it says itself (null: one).
 template <class F>
-cudaError_t timed(af_ctx* c, int kernel, cudaStream_t s, F&& launch, int kernels = 1) {
+cudaError_t timed(af_ctx* c, int kernel, cudaStream_t s, F&& launch, const int* kernels = nullptr) {
   if (!c->prof_on) return launch();
-  af_ctx::ProfRec r{kernel, take_event(c), take_event(c), kernels};
+  af_ctx::ProfRec r{kernel, take_event(c), take_event(c), 1};
   cudaEventRecord(r.a, s);
   const cudaError_t e = launch();
   cudaEventRecord(r.b, s);
+  if (kernels) r.kernels = *kernels;
   c->prof.push_back(r);
   return e;
 }
@@ -574,7 +575,9 @@ extern "C" af_status af_integrate_scan(af_ctx* ctx, const float* d_xyz, uint32_t
   ctx->frame = ctx->frame + 1 >= 0xFFFFFFFFu ? 1 : ctx->frame + 1;
   cudaStream_t s = (cudaStream_t)stream;
   const MapView& M = ctx->M;
-  AF_CUDA(ctx, timed(ctx, 0, s, [&] { return af::launch_alloc(M, d_xyz, n, pose, ctx->d_ret, ctx->frame, s); }));
+  const int alloc_kernels = n > 0 ? 1 : 0;  // without returns the dirty list is only cleared
+  AF_CUDA(ctx, timed(ctx, 0, s, [&] { return af::launch_alloc(M, d_xyz, n, pose, ctx->d_ret, ctx->frame, s); },
+                     &alloc_kernels));
   // the point layer's neighbourhood trigger compares the touched bricks
   // after the scan with their state before it
   if (ctx->pts_snapshot) AF_CUDA(ctx, af::launch_pts_snapshot(ctx, s));
@@ -614,10 +617,13 @@ extern "C" af_status af_integrate_scan_projective(af_ctx* ctx, const float* d_xy
   cudaStream_t s = (cudaStream_t)stream;
   af::MapView M = ctx->M;
   M.ns = 0;  // no cleared band: the projective update has none
-  AF_CUDA(ctx, timed(ctx, 0, s, [&] { return af::launch_alloc(M, d_xyz, n, pose, ctx->d_ret, ctx->frame, s); }));
+  const int alloc_kernels = n > 0 ? 1 : 0;  // without returns the dirty list is only cleared
+  AF_CUDA(ctx, timed(ctx, 0, s, [&] { return af::launch_alloc(M, d_xyz, n, pose, ctx->d_ret, ctx->frame, s); },
+                     &alloc_kernels));
+  const int kernels = n > 0 ? 2 : 1;
   AF_CUDA(ctx, timed(ctx, 1, s, [&] {
             return af::launch_projective(M, d_xyz, n, pose, ctx->d_ret, ctx->d_img, bins, ctx->num_sms, s);
-          }, n > 0 ? 2 : 1));
+          }, &kernels));
   AF_CUDA(ctx, timed(ctx, 2, s, [&] { return af::launch_bitview(M, ctx->num_sms, s); }));
   ctx->last_stream = s;
   ctx->scans++;
@@ -737,11 +743,12 @@ extern "C" af_status af_score(af_ctx* ctx, const float* d_pts, const float* d_no
     ctx->split_cap = m;
   }
   const af::ScoreSplit S{ctx->d_over, ctx->d_sres, ctx->d_scount, ctx->score_budget};
+  const int kernels = S.budget >= 0 ? 3 : 1;
   if (m > 0)
     AF_CUDA(ctx, timed(ctx, 3, s, [&] {
               return af::launch_score(ctx->M, ctx->T, d_pts, d_normals, m, d_label, d_best, S,
                                       ctx->num_sms, s);
-            }, S.budget >= 0 ? 3 : 1));
+            }, &kernels));
   ctx->last_stream = s;
   ctx->points_in += m;
   return AF_OK;
@@ -941,10 +948,11 @@ static af_status ensure_views(af_ctx* ctx, cudaStream_t s) {
     const bool captured = cap != cudaStreamCaptureStatusNone;
     if (captured && ctx->views_capture == id + 1 && ctx->views_capture_frame == ctx->frame) return AF_OK;
     const bool fill = !ctx->views_filled;
+    int kernels = 0;
     AF_CUDA(ctx, timed(ctx, 4, s, [&] {
       return af::launch_views(M, ctx->num_sms, fill, ctx->d_dense, ctx->d_cells, ctx->d_vlist,
-                              ctx->d_vseen, s);
-    }));
+                              ctx->d_vseen, &kernels, s);
+    }, &kernels));
     if (captured) {
       ctx->views_capture = id + 1;
       ctx->views_capture_frame = ctx->frame;
@@ -1165,10 +1173,11 @@ extern "C" af_status af_soft_refine(af_ctx* ctx, const float* d_pts, uint32_t pe
   if ((st = ensure_views(ctx, s)) != AF_OK) return st;
   view_fields(ctx, &S);
   const af::RefineArgs A{(int)R->steps, R->lr_dir, R->lr_h, R->h_max};
+  int kernels = 0;
   AF_CUDA(ctx, timed(ctx, 7, s, [&] {
     return af::launch_soft_refine(S, A, d_pts, per_point, d_u0, d_alpha, d_beta, d_h, n, d_c,
-                                  d_cmin, ctx->num_sms, s);
-  }, 2));
+                                  d_cmin, ctx->num_sms, &kernels, s);
+  }, &kernels));
   ctx->last_stream = s;
   return AF_OK;
 }

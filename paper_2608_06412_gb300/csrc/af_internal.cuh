@@ -299,7 +299,7 @@ struct PtCounters {
   uint32_t nsnap;     // bricks whose state was copied before the frame's scan
   uint32_t nsel;      // points selected for evaluation
   uint32_t evals;     // evaluations of the last call
-  uint32_t ended;     // CTAs that have ended (count_ended; zero between kernels)
+  uint32_t ended;     // CTAs that have ended (last_cta; zero between kernels)
   uint32_t ndrawn;    // listed candidates of the draw
 };
 

@@ -917,8 +917,10 @@ size_t seen_words(const MapView& M) {
 
 // Brings the dense view up to date with the map; with `fill` the buffers are new,
 // every value starts as tau and every brick is taken. `list`: view_list_words(M).
+// *kernels: the kernels launched.
 cudaError_t launch_views(const MapView& M, int num_sms, bool fill, float* dense, float4* cells,
-                         uint32_t* list, uint32_t* seen, cudaStream_t stream) {
+                         uint32_t* list, uint32_t* seen, int* kernels, cudaStream_t stream) {
+  *kernels = fill ? 5 : 3;
   const size_t nd = (size_t)M.dim_vox[0] * M.dim_vox[1] * M.dim_vox[2];  // a multiple of 512
   const size_t nc = ((size_t)M.dim_vox[0] + 1) * (M.dim_vox[1] + 1) * (M.dim_vox[2] + 1);
   uint32_t *nlist = list + M.pool_blocks, *taken = nlist + 1;
@@ -1011,7 +1013,8 @@ constexpr int kRefineGeneralBelow = 25, kRefineGeneralBelowSparse = 9, kRefineWi
 template <bool FIXED, bool SPARSE>
 static void launch_refine_form(const SoftView& S, const RefineArgs& R, const float* pts,
                                uint32_t per_point, const float* u0, float* al, float* be, float* h,
-                               uint64_t n, float* c, float* cmin, int num_sms, cudaStream_t stream) {
+                               uint64_t n, float* c, float* cmin, int num_sms, int* kernels,
+                               cudaStream_t stream) {
   const int samples = S.J - S.j0 + 1;
   const unsigned g = grid_for(n * kLanes, 128, num_sms, 16);
   const auto waves = [&](int ctas) {
@@ -1020,6 +1023,7 @@ static void launch_refine_form(const SoftView& S, const RefineArgs& R, const flo
   };
   const auto run = [&](auto kernel) {
     kernel<<<g, 128, 0, stream>>>(S, R, pts, per_point, u0, al, be, h, n, c, cmin);
+    ++*kernels;
   };
   const int few_samples = SPARSE ? kRefineGeneralBelowSparse : kRefineGeneralBelow;
   const bool wide = waves(3) == waves(4);
@@ -1041,12 +1045,13 @@ static void launch_refine_form(const SoftView& S, const RefineArgs& R, const flo
 cudaError_t launch_soft_refine(const SoftView& S, const RefineArgs& R, const float* pts,
                                uint32_t per_point, const float* u0, float* al, float* be,
                                float* h, uint64_t n, float* c, float* cmin, int num_sms,
-                               cudaStream_t stream) {
+                               int* kernels, cudaStream_t stream) {
+  *kernels = 0;
   if (n == 0) return cudaSuccess;
   decltype(&launch_refine_form<false, false>) form =
       S.fixed ? (S.sparse ? launch_refine_form<true, true> : launch_refine_form<true, false>)
               : (S.sparse ? launch_refine_form<false, true> : launch_refine_form<false, false>);
-  form(S, R, pts, per_point, u0, al, be, h, n, c, cmin, num_sms, stream);
+  form(S, R, pts, per_point, u0, al, be, h, n, c, cmin, num_sms, kernels, stream);
   return cudaGetLastError();
 }
 
