@@ -34,14 +34,41 @@ struct CubeShape {
   static constexpr int MR = W / 2;
 };
 
-// Returns per CTA ("tile") of one scan's integration, by the scan's size. A tile's
-// setup (brick table or box offsets, per-axis terms) is spread over its pairs, so
-// larger tiles cost less a return as long as enough CTAs are left to overlap: with
-// tiles of 8 / 12 / 16 the map's kernel takes 26.9 / 25.5 / 26.7 us for 20,000
-// returns and 68.5 / 63.9 / 60.8 us for 60,000, the box's 27.6 / 27.0 / 26.3 us for
-// 20,000. Small scans take small tiles, so that every SM has one.
-constexpr int kTileSmall = 4, kTile = 12, kTileLarge = 16;
-constexpr uint32_t kTileSmallBelow = 4000, kTileLargeFrom = 40000;
+// Returns per CTA ("tile") of one scan's integration: 4, 8, 12 or 16, the one that
+// should take least time. An SM holds as many CTAs at once as their threads and
+// registers allow (five of the cube of 7, one of 17) and takes the rest in turn; a
+// CTA costs its pairs (offsets per thread times returns) and a setup (tables, per-axis
+// terms) worth about six returns of one offset in the map's kernel, eight in the
+// box's two. So small scans take the tile that spreads them over the chip in one go,
+// large ones the tile that pays the setup least often without a last round for a few.
+// Cubes of 3 and 5 have one and four warps per CTA, which a tile's setup keeps busy
+// longer than its pairs: they stay with 4 and 8.
+// Map's kernel, tiles of 4 / 8 / 12 / 16 (us): cube of 3, 6,000 returns 10.3 / 12.3 /
+// 14.4 / 16.6; of 7, 6,000 returns 16.4 / 14.3 / 15.3 / 15.6, 12,000 25.0 / 21.1 /
+// 22.0 / 20.2, 20,000 36.5 / 30.5 / 28.8 / 28.5, 60,000 90 / 72 / 67 / 63; of 9, 2,000
+// returns 16.1 / 13.0 / 14.5 / 13.8, 4,000 24.4 / 19.6 / 20.1 / 17.4; of 17, 2,000
+// returns 43 / 37 / 49 / 35, 20,000 308 / 270 / 248 / 260.
+constexpr int kSetupMap = 6, kSetupBox = 8;
+constexpr uint32_t kChipSMs = 152;
+
+template <int W>
+inline int tile_of(uint32_t n, int setup) {
+  using S = CubeShape<W>;
+  constexpr int most = W == 3 ? 4 : (W == 5 ? 8 : 16);
+  constexpr uint32_t held = S::OPT > 3 ? 1 : (2048 / S::NT < 32 ? 2048 / S::NT : 32);
+  int best = 0;
+  uint64_t least = ~0ull;
+  for (const int T : {8, 4, 12, 16}) {  // a tie keeps the one before
+    if (T > most) continue;
+    const uint32_t ctas = (n + T - 1) / T, turns = (ctas + kChipSMs - 1) / kChipSMs;
+    const uint64_t cost = (uint64_t)(turns > held ? turns : held) * (uint64_t)(T * S::OPT + setup);
+    if (cost < least) {
+      least = cost;
+      best = T;
+    }
+  }
+  return best;
+}
 
 // What a pair reads of its return: x = range |p - q|, y = RN(1 / range) (for the
 // approximate cone test), w = valid flag.

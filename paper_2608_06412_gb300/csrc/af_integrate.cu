@@ -430,23 +430,31 @@ cudaError_t launch_alloc(const MapView& M, const float* d_xyz, uint32_t n, const
   return cudaGetLastError();
 }
 
+template <int W>
+static void launch_cube_tiled(const MapView& M, uint32_t n, const float pose[16], const float4* d_ret,
+                              uint32_t frame, cudaStream_t stream) {
+  const int T = tile_of<W>(n, kSetupMap);
+  const auto run = [&](auto kernel) {
+    kernel<<<(n + T - 1) / T, CubeShape<W>::NT, 0, stream>>>(M, d_ret, n, pose[3], pose[7], pose[11], frame);
+  };
+  if constexpr (W > 5) {
+    if (T == 16) return run(k_integrate<W, 16>);
+    if (T == 12) return run(k_integrate<W, 12>);
+  }
+  if constexpr (W > 3) {
+    if (T == 8) return run(k_integrate<W, 8>);
+  }
+  run(k_integrate<W, 4>);
+}
+
 cudaError_t launch_cube(const MapView& M, uint32_t n, const float pose[16], const float4* d_ret,
                         uint32_t frame, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
-  const int T = n < kTileSmallBelow ? kTileSmall : (n < kTileLargeFrom ? kTile : kTileLarge);
-  const unsigned grid = (n + T - 1) / T;
-#define AF_TILE(W, TT) \
-  k_integrate<W, TT><<<grid, CubeShape<W>::NT, 0, stream>>>(M, d_ret, n, pose[3], pose[7], pose[11], frame)
   switch (2 * M.m + 1) {
-#define AF_CASE(W)                                   \
-  case W:                                            \
-    if (T == kTileSmall) AF_TILE(W, kTileSmall);     \
-    else if (T == kTile) AF_TILE(W, kTile);          \
-    else AF_TILE(W, kTileLarge);                     \
-    break;
+#define AF_CASE(W) \
+  case W: launch_cube_tiled<W>(M, n, pose, d_ret, frame, stream); break;
     AF_CASE(3) AF_CASE(5) AF_CASE(7) AF_CASE(9) AF_CASE(11) AF_CASE(13) AF_CASE(15) AF_CASE(17)
 #undef AF_CASE
-#undef AF_TILE
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

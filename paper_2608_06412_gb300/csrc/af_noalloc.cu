@@ -243,6 +243,28 @@ __global__ void __launch_bounds__(CubeShape<W>::NT) k_box_finalize(MapView M,
   }
 }
 
+template <int W, int T>
+void launch_box_tile(const MapView& M, const float* xyz, uint32_t n, const Pose& P, float4* scratch,
+                     const Box& B, cudaStream_t s) {
+  const unsigned grid = (n + T - 1) / T;
+  k_box_integrate<W, T><<<grid, CubeShape<W>::NT, 0, s>>>(M, xyz, n, P, scratch, B);
+  k_box_finalize<W, T><<<grid, CubeShape<W>::NT, 0, s>>>(M, scratch, n, P.r[0][3], P.r[1][3], P.r[2][3], B);
+}
+
+template <int W>
+void launch_box(const MapView& M, const float* xyz, uint32_t n, const Pose& P, float4* scratch,
+                const Box& B, cudaStream_t s) {
+  const int T = tile_of<W>(n, kSetupBox);
+  if constexpr (W > 5) {
+    if (T == 16) return launch_box_tile<W, 16>(M, xyz, n, P, scratch, B, s);
+    if (T == 12) return launch_box_tile<W, 12>(M, xyz, n, P, scratch, B, s);
+  }
+  if constexpr (W > 3) {
+    if (T == 8) return launch_box_tile<W, 8>(M, xyz, n, P, scratch, B, s);
+  }
+  launch_box_tile<W, 4>(M, xyz, n, P, scratch, B, s);
+}
+
 bool finite_f(float x) { return std::isfinite(x); }
 
 }  // namespace
@@ -325,23 +347,11 @@ extern "C" af_status af_integrate_scan_noalloc(const af_config* cfg, const float
 
   cudaStream_t s = (cudaStream_t)stream;
   if (n > 0) {
-    // the box's kernels take the large tile from the middle range on
-    const int T = n < kTileSmallBelow ? kTileSmall : kTileLarge;
-    const unsigned grid = (n + T - 1) / T;
-#define AF_TILE(W, TT)                                                                                    \
-  {                                                                                                       \
-    k_box_integrate<W, TT><<<grid, CubeShape<W>::NT, 0, s>>>(M, d_xyz, n, P, scratch, B);                \
-    k_box_finalize<W, TT><<<grid, CubeShape<W>::NT, 0, s>>>(M, scratch, n, pose[3], pose[7], pose[11], B); \
-  }
     switch (2 * M.m + 1) {
-#define AF_CASE(W)                                \
-  case W:                                         \
-    if (T == kTileSmall) AF_TILE(W, kTileSmall)   \
-    else AF_TILE(W, kTileLarge)                   \
-    break;
+#define AF_CASE(W) \
+  case W: launch_box<W>(M, d_xyz, n, P, scratch, B, s); break;
       AF_CASE(3) AF_CASE(5) AF_CASE(7) AF_CASE(9) AF_CASE(11) AF_CASE(13) AF_CASE(15) AF_CASE(17)
 #undef AF_CASE
-#undef AF_TILE
     }
   }
   const cudaError_t e = cudaGetLastError();
