@@ -132,8 +132,7 @@ struct Offset {
   int x, y, z;
 };
 
-bool member(const af_tool& t, double v, const double u[3], int ox, int oy, int oz, int which) {
-  const double ex = (double)ox * v, ey = (double)oy * v, ez = (double)oz * v;
+inline bool member_at(const af_tool& t, double ex, double ey, double ez, const double u[3], int which) {
   const double a = (ex * u[0] + ey * u[1]) + ez * u[2];
   const double rx = ex - a * u[0], ry = ey - a * u[1], rz = ez - a * u[2];
   const double rho2 = (rx * rx + ry * ry) + rz * rz;
@@ -141,10 +140,14 @@ bool member(const af_tool& t, double v, const double u[3], int ox, int oy, int o
   if (which == AF_KERNEL_TOOL) {
     const double e2 = (ex * ex + ey * ey) + ez * ez;
     const double r = (double)t.radius, rs = (double)t.self_excl;
-    return a >= 0.0 && a <= L && rho2 <= r * r && e2 > rs * rs;
+    return (a >= 0.0) & (a <= L) & (rho2 <= r * r) & (e2 > rs * rs);
   }
   const double r = (double)t.corr_radius;
-  return a > L && a <= L + (double)t.corr_length && rho2 <= r * r;
+  return (a > L) & (a <= L + (double)t.corr_length) & (rho2 <= r * r);
+}
+
+bool member(const af_tool& t, double v, const double u[3], int ox, int oy, int oz, int which) {
+  return member_at(t, (double)ox * v, (double)oy * v, (double)oz * v, u, which);
 }
 
 // The axis-aligned box that holds the cylinder (with one voxel of margin);
@@ -182,31 +185,51 @@ struct Run {
   double a;
 };
 
+template <int AXIS, int WHICH>
+void rasterise_rows(const af_tool& t, double v, const double u[3], const int lo[3], const int hi[3],
+                    std::vector<Run>* out) {
+  constexpr int o1 = AXIS == 0 ? 1 : 0, o2 = AXIS == 2 ? 1 : 2;
+  const int n = hi[AXIS] - lo[AXIS] + 1;
+  std::vector<uint8_t> in(n + 1, 0);  // ends outside
+  double e[3];
+  auto axial = [&](int k) {
+    double x[3] = {e[0], e[1], e[2]};
+    x[AXIS] = (double)k * v;
+    return (x[0] * u[0] + x[1] * u[1]) + x[2] * u[2];
+  };
+  for (int c2 = lo[o2]; c2 <= hi[o2]; ++c2)
+    for (int c1 = lo[o1]; c1 <= hi[o1]; ++c1) {
+      e[o1] = (double)c1 * v;
+      e[o2] = (double)c2 * v;
+      unsigned any = 0;
+      for (int k = 0; k < n; ++k) {
+        const double x = (double)(lo[AXIS] + k) * v;
+        in[k] = member_at(t, AXIS == 0 ? x : e[0], AXIS == 1 ? x : e[1], AXIS == 2 ? x : e[2], u, WHICH);
+        any |= in[k];
+      }
+      for (int k = 0; any && k < n; ++k) {
+        if (!in[k]) continue;
+        const int s = k;
+        while (in[k]) ++k;
+        out->push_back({c1, c2, lo[AXIS] + s, lo[AXIS] + k,
+                        std::min(axial(lo[AXIS] + s), axial(lo[AXIS] + k - 1))});
+      }
+    }
+}
+
 std::vector<Run> rasterise_runs(const af_tool& t, double v, const double u[3], int which, int axis) {
   std::vector<Run> out;
-  int lo[3], hi[3], o[3];
+  int lo[3], hi[3];
   if (!kernel_box(t, v, u, which, lo, hi)) return out;
-  const int o1 = axis == 0 ? 1 : 0, o2 = axis == 2 ? 1 : 2;
-  auto axial = [&](int k) {
-    o[axis] = k;
-    return ((double)o[0] * v * u[0] + (double)o[1] * v * u[1]) + (double)o[2] * v * u[2];
+  const auto rows = [&](auto tool, auto corridor) {
+    (which == AF_KERNEL_TOOL ? tool : corridor)(t, v, u, lo, hi, &out);
   };
-  for (o[o2] = lo[o2]; o[o2] <= hi[o2]; ++o[o2])
-    for (o[o1] = lo[o1]; o[o1] <= hi[o1]; ++o[o1])
-      for (int k = lo[axis]; k <= hi[axis];) {
-        auto in = [&](int i) {
-          o[axis] = i;
-          return member(t, v, u, o[0], o[1], o[2], which);
-        };
-        if (!in(k)) {
-          ++k;
-          continue;
-        }
-        int e = k + 1;
-        while (e <= hi[axis] && in(e)) ++e;
-        out.push_back({o[o1], o[o2], k, e, std::min(axial(k), axial(e - 1))});
-        k = e + 1;
-      }
+  if (axis == 0)
+    rows(rasterise_rows<0, AF_KERNEL_TOOL>, rasterise_rows<0, AF_KERNEL_CORRIDOR>);
+  else if (axis == 1)
+    rows(rasterise_rows<1, AF_KERNEL_TOOL>, rasterise_rows<1, AF_KERNEL_CORRIDOR>);
+  else
+    rows(rasterise_rows<2, AF_KERNEL_TOOL>, rasterise_rows<2, AF_KERNEL_CORRIDOR>);
   return out;
 }
 
@@ -231,51 +254,66 @@ struct Quad {
 // ordered by axial distance (near ones first: blocking geometry next to the
 // surface is met early).
 void to_quads(const std::vector<Run>& runs, std::vector<Quad> out[4]) {
-  struct Piece {
-    int q1, q2, s, e, row;
-    double a;
-  };
-  std::vector<Piece> pieces(runs.size());
+  if (runs.empty()) return;
+  int d1lo = INT_MAX, d1hi = INT_MIN, d2lo = INT_MAX, d2hi = INT_MIN;
+  for (const Run& r : runs) {
+    d1lo = std::min(d1lo, r.d1);
+    d1hi = std::max(d1hi, r.d1);
+    d2lo = std::min(d2lo, r.d2);
+    d2hi = std::max(d2hi, r.d2);
+  }
+  std::vector<uint32_t> first, order(runs.size());
+  std::vector<Quad> q;
   for (int p = 0; p < 4; ++p) {
     const int p1 = p & 1, p2 = p >> 1;
-    for (size_t k = 0; k < runs.size(); ++k) {
-      const Run& r = runs[k];
-      pieces[k] = {(p1 + r.d1) >> 1, (p2 + r.d2) >> 1, r.s, r.e,
-                   ((p1 + r.d1) & 1) | (((p2 + r.d2) & 1) << 1), r.a};
-    }
-    std::sort(pieces.begin(), pieces.end(), [](const Piece& x, const Piece& y) {
-      if (x.q2 != y.q2) return x.q2 < y.q2;
-      if (x.q1 != y.q1) return x.q1 < y.q1;
-      if (x.s != y.s) return x.s < y.s;
-      return x.row < y.row;
-    });
-    std::vector<Quad>& q = out[p];
-    for (size_t i = 0; i < pieces.size();) {
-      size_t j = i;
-      while (j < pieces.size() && pieces[j].q1 == pieces[i].q1 && pieces[j].q2 == pieces[i].q2) ++j;
-      // windows of 32 over the group's pieces, from the lowest voxel not yet taken
-      int from = pieces[i].s;
+    // runs by group, (q2, q1) ascending: a counting sort
+    const int q1lo = (p1 + d1lo) >> 1, n1 = ((p1 + d1hi) >> 1) - q1lo + 1;
+    const int q2lo = (p2 + d2lo) >> 1, n2 = ((p2 + d2hi) >> 1) - q2lo + 1;
+    const auto group = [&](const Run& r) {
+      return (size_t)(((p2 + r.d2) >> 1) - q2lo) * n1 + (size_t)(((p1 + r.d1) >> 1) - q1lo);
+    };
+    const size_t groups = (size_t)n1 * n2;
+    first.assign(groups + 1, 0);
+    for (const Run& r : runs) ++first[group(r) + 1];
+    for (size_t g = 0; g < groups; ++g) first[g + 1] += first[g];
+    for (size_t k = 0; k < runs.size(); ++k) order[first[group(runs[k])]++] = (uint32_t)k;
+    // first[g] is now the end of group g
+    q.clear();
+    size_t i = 0;
+    for (size_t g = 0; g < groups; i = first[g++]) {
+      const size_t j = first[g];
+      if (i == j) continue;
+      // windows of 32 over the group's runs, from the lowest voxel not yet taken
+      int from = INT_MIN;
       while (true) {
         int lo = INT_MAX;
-        for (size_t k = i; k < j; ++k)
-          if (pieces[k].e > from) lo = std::min(lo, std::max(pieces[k].s, from));
+        for (size_t k = i; k < j; ++k) {
+          const Run& r = runs[order[k]];
+          if (r.e > from) lo = std::min(lo, std::max(r.s, from));
+        }
         if (lo == INT_MAX) break;
         int hi = lo;
-        Quad w{1e300, pieces[i].q1, pieces[i].q2, lo, 0, {0, 0, 0, 0}};
+        Quad w{1e300, q1lo + (int)(g % n1), q2lo + (int)(g / n1), lo, 0, {0, 0, 0, 0}};
         for (size_t k = i; k < j; ++k) {
-          const int s = std::max(pieces[k].s, lo), e = std::min(pieces[k].e, lo + 32);
+          const Run& r = runs[order[k]];
+          const int s = std::max(r.s, lo), e = std::min(r.e, lo + 32);
           if (s >= e) continue;
-          w.mask[pieces[k].row] |= (uint32_t)(((1ull << (e - s)) - 1ull) << (s - lo));
-          w.a = std::min(w.a, pieces[k].a);
+          w.mask[((p1 + r.d1) & 1) | (((p2 + r.d2) & 1) << 1)] |=
+              (uint32_t)(((1ull << (e - s)) - 1ull) << (s - lo));
+          w.a = std::min(w.a, r.a);
           hi = std::max(hi, e);
         }
         w.spare = 32 - (hi - lo);
         q.push_back(w);
         from = lo + 32;
       }
-      i = j;
     }
-    std::stable_sort(q.begin(), q.end(), [](const Quad& x, const Quad& y) { return x.a < y.a; });
+    // order by distance through indices: an entry is 48 bytes
+    std::vector<std::pair<double, uint32_t>> by(q.size());
+    for (size_t k = 0; k < q.size(); ++k) by[k] = {q[k].a, (uint32_t)k};
+    std::sort(by.begin(), by.end());  // equal distances in the order above
+    out[p].resize(q.size());
+    for (size_t k = 0; k < q.size(); ++k) out[p][k] = q[by[k].second];
   }
 }
 
