@@ -211,7 +211,11 @@ def _stream_ptr(stream) -> int:
     if stream is not None:
         return stream.cuda_stream
     torch = _import_torch()
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    try:
+        raw = torch._C._cuda_getCurrentRawStream
+    except AttributeError:   # torch's own, not in its documented interface
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 @dataclass
