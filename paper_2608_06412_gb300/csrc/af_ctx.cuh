@@ -33,7 +33,7 @@ struct af_ctx {
   af_tool tool{};
   // views of the differentiable form (built on first use, rebuilt when the
   // map has changed since)
-  float* d_dense = nullptr;
+  float* d_dense = nullptr;      // the dense view's one allocation: values, then the next three
   float4* d_cells = nullptr;
   uint32_t* d_vlist = nullptr;   // bricks to update, their count, the stamps they were taken at
   uint32_t* d_vseen = nullptr;   // a bit per block of 8^3 cells that reads anything but tau

@@ -439,9 +439,6 @@ static void free_all(af_ctx* c) {
   cudaFree(c->d_sres);
   cudaFree(c->d_scount);
   cudaFree(c->d_dense);
-  cudaFree(c->d_cells);
-  cudaFree(c->d_vlist);
-  cudaFree(c->d_vseen);
   cudaFree(c->d_bgrid);
   cudaFree(c->d_skeys);
   cudaFree(c->d_nslots);
@@ -958,21 +955,22 @@ static af_status ensure_views(af_ctx* ctx, cudaStream_t s) {
       const size_t nc = ((size_t)M.dim_vox[0] + 1) * (M.dim_vox[1] + 1) * (M.dim_vox[2] + 1);
       if (nc >= (1ull << 31))
         return fail(ctx, AF_ERR_CAPACITY, "soft clearance: the map box has too many cells for the dense SDF view");
-      if (cudaMalloc(&ctx->d_dense, nd * sizeof(float)) != cudaSuccess ||
-          cudaMalloc(&ctx->d_cells, nc * 2 * sizeof(float4)) != cudaSuccess ||
-          cudaMalloc(&ctx->d_vlist, af::view_list_words(M) * sizeof(uint32_t)) != cudaSuccess ||
-          cudaMalloc(&ctx->d_vseen, af::seen_words(M) * sizeof(uint32_t)) != cudaSuccess) {
+      // one allocation (dense values, records, list, marks): the first call of a map
+      // waits for it
+      const size_t dense_b = nd * sizeof(float), cells_b = nc * 2 * sizeof(float4);
+      const size_t list_b = af::view_list_words(M) * sizeof(uint32_t);
+      unsigned char* base = nullptr;
+      if (cudaMalloc((void**)&base, dense_b + cells_b + list_b + af::seen_words(M) * sizeof(uint32_t)) !=
+          cudaSuccess) {
         cudaGetLastError();
-        cudaFree(ctx->d_dense);
-        cudaFree(ctx->d_cells);
-        cudaFree(ctx->d_vlist);
-        ctx->d_dense = nullptr;
-        ctx->d_cells = nullptr;
-        ctx->d_vlist = nullptr;
         return fail(ctx, AF_ERR_CAPACITY,
                     "soft clearance: cannot allocate the SDF views (%zu + %zu bytes) of the map box",
-                    nd * sizeof(float), nc * 2 * sizeof(float4));
+                    dense_b, cells_b);
       }
+      ctx->d_dense = (float*)base;  // a multiple of 2 KB: the records stay aligned
+      ctx->d_cells = (float4*)(base + dense_b);
+      ctx->d_vlist = (uint32_t*)(base + dense_b + cells_b);
+      ctx->d_vseen = (uint32_t*)(base + dense_b + cells_b + list_b);
       ctx->views_filled = false;
     }
     if (!stale) return AF_OK;
@@ -1225,9 +1223,6 @@ extern "C" af_status af_soft_set_view(af_ctx* ctx, int32_t mode) {
   if (mode < 0 || mode > 2) return fail(ctx, AF_ERR_INVALID_ARG, "af_soft_set_view: mode must be 0, 1 or 2");
   AF_CUDA(ctx, cudaDeviceSynchronize());
   cudaFree(ctx->d_dense);
-  cudaFree(ctx->d_cells);
-  cudaFree(ctx->d_vlist);
-  cudaFree(ctx->d_vseen);
   cudaFree(ctx->d_bgrid);
   cudaFree(ctx->d_skeys);
   cudaFree(ctx->d_nslots);
