@@ -31,8 +31,8 @@ struct af_ctx {
   int4* d_dtab = nullptr;
   short4* d_arm = nullptr;
   af_tool tool{};
-  // views of the differentiable form (built on first use, rebuilt when the
-  // map has changed since)
+  // views of the differentiable form (built on first use, brought up to date
+  // when the map has changed since)
   float* d_dense = nullptr;      // the dense view's one allocation: values, then the next three
   float4* d_cells = nullptr;
   uint32_t* d_vlist = nullptr;   // bricks to update, their count, the stamps they were taken at

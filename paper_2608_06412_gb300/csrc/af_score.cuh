@@ -20,8 +20,8 @@
 // in two steps instead of five. Against runs with their tables staged in
 // shared memory: 72.5 -> 53 us per pine frame (12k points, 128 directions), 489
 // -> 282 us for 40k points of three pines with the 6 cm tool and 256 directions,
-// 2.5 -> 1.34 ms for 83k points of a 1 cm map with 512. The latter two are bound
-// by L1 wavefronts (80% of their peak on the 1 cm map: a gather of 16-byte words
+// 2.5 -> 1.28 ms for 83k points of a 1 cm map with 512. The latter two are bound
+// by L1 wavefronts (82% of their peak on the 1 cm map: a gather of 16-byte words
 // takes a wavefront per lane), the pine frame by the chain and its tail.
 //
 // A point whose whole kernel reach lies inside the map box takes the FAST path,

@@ -498,8 +498,8 @@ constexpr int kInFlightGeneralWide = 4;
 // hold anything else: one bit per 8^3 cells, 29 KB for the pine box, which stays
 // in L1. The records then read are a 27 MB part of the 3.7 GB view and stay in L2.
 // With the checks of the cells gone as well, the field of a finished map's 30k
-// points (1.9M pairs) went from 862 to about 490 us, forward plus adjoint of 113k
-// pairs from 149 to 72 us, the refinement of 30k pairs from 315 to 235 us. In a
+// points (1.9M pairs) went from 862 to about 485 us, forward plus adjoint of 113k
+// pairs from 149 to 71 us, the refinement of 30k pairs from 315 to 232 us. In a
 // small box (0.17 GB of records, which the caches hold) they gain nothing: 512k
 // pairs, a third of which leave the view, take 127 us either way.
 template <bool NEAR, bool GRAD, bool FIXED, bool SPARSE, int NF>
