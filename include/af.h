@@ -522,7 +522,7 @@ af_status af_points_export(af_ctx *ctx, uint32_t cap, int32_t *h_ijk, float *h_n
  * launches (milliseconds) and, if `reset`, forgets them. launches[] counts
  * kernels, one bracket may hold several: an af_score call with work sharing on
  * is three (k_score, k_score_split, k_score_finish), a projective integration
- * two, an update of the dense SDF view three (five with its first fill), an
+ * two, an update of the dense SDF view two (four with its first fill), an
  * af_soft_refine call one, or two for more pairs than the chip holds at once
  * (all pairs, then those of whose samples one step found the first outside the
  * view or very far from its point).

@@ -984,6 +984,7 @@ static af_status ensure_views(af_ctx* ctx, cudaStream_t s) {
     const bool captured = cap != cudaStreamCaptureStatusNone;
     if (captured && ctx->views_capture == id + 1 && ctx->views_capture_frame == ctx->frame) return AF_OK;
     const bool fill = !ctx->views_filled;
+    if (!captured) ctx->views_filled = false;  // a launch that fails leaves the list as it is
     int kernels = 0;
     AF_CUDA(ctx, timed(ctx, 4, s, [&] {
       return af::launch_views(M, ctx->num_sms, fill, ctx->d_dense, ctx->d_cells, ctx->d_vlist,

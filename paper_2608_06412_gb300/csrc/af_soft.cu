@@ -51,43 +51,62 @@ __global__ void __launch_bounds__(256) k_fill(float4* __restrict__ out, size_t n
     out[i] = v;
 }
 
-// Lists the pool bricks that a scan has touched since the view last took them:
-// each scan stamps the hash slot of every brick it touches, and `taken` keeps the
-// stamp at which the view took a brick (~0: never). Stamps are compared for
-// equality, not order, so scans that run late -- a captured scan replayed after
-// later ones keeps its older number -- and scan numbers that wrap are covered,
-// and a replayed update takes whatever changed before it.
-__global__ void __launch_bounds__(256) k_view_list(MapView M, uint32_t* __restrict__ taken,
-                                                   uint32_t* __restrict__ list,
-                                                   uint32_t* __restrict__ nlist) {
-  const uint32_t count = min(__ldcg(&M.ctl->pool_count), M.pool_blocks);
-  for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < count; b += gridDim.x * blockDim.x) {
-    uint32_t val, stamp;
-    if (find_slot(M, M.bkey[b], &val, &stamp) < 0 || stamp == taken[b]) continue;
-    taken[b] = stamp;
-    list[atomicAdd(nlist, 1u)] = b;
+// The pool bricks that a scan has touched since the view last took them: their
+// dense SDF (S / (w 2^20) divided in double and rounded to single precision, tau
+// where w = 0), and a list of them for k_cell_view. Each scan stamps the hash slot of
+// every brick it touches, and `taken` keeps the stamp at which the view took a brick
+// (~0: never). Stamps are compared for equality, not order, so scans that run late --
+// a captured scan replayed after later ones keeps its older number -- and scan
+// numbers that wrap are covered, and a replayed update takes whatever changed
+// before it.
+//
+// A CTA looks at 256 bricks at a time, far apart in the pool (a scan's new bricks
+// are neighbours there), and takes each changed one with all its threads: the
+// divisions are what a brick costs (a warp to a brick took 2.2 times as long). In a
+// small box (`whole`, launch_views) every brick is taken without a look at its
+// stamp: the probes and the list would cost more than its few bricks.
+__device__ inline void dense_brick(const MapView& M, uint32_t b, float* __restrict__ dense) {
+  const size_t X = (size_t)M.dim_vox[0], Y = (size_t)M.dim_vox[1];
+  const uint64_t key = M.bkey[b];
+  const size_t bx = (size_t)(key & 0x1FFFFF) * 8, by = (size_t)((key >> 21) & 0x1FFFFF) * 8,
+               bz = (size_t)(key >> 42) * 8;
+  for (int l = threadIdx.x; l < kBrickVox; l += 256) {
+    const unsigned long long word = __ldcg(M.vox + (size_t)b * kBrickVox + l);
+    const unsigned long long w = word & kWMask;
+    const float d = w ? __double2float_rn((double)word_S(word) / ((double)w * 1048576.0)) : M.tau;
+    dense[((bz + (l >> 6)) * Y + by + ((l >> 3) & 7)) * X + bx + (l & 7)] = d;
   }
 }
 
-// Dense SDF of the listed bricks: S / (w 2^20) divided in double and rounded to
-// single precision; tau where w = 0.
-__global__ void __launch_bounds__(256) k_dense_view(MapView M, const uint32_t* __restrict__ list,
-                                                    const uint32_t* __restrict__ nlist,
+__global__ void __launch_bounds__(256) k_dense_view(MapView M, int whole, uint32_t* __restrict__ taken,
+                                                    uint32_t* __restrict__ list,
+                                                    uint32_t* __restrict__ nlist,
                                                     float* __restrict__ dense) {
-  const uint32_t count = __ldcg(nlist);
-  const size_t X = (size_t)M.dim_vox[0], Y = (size_t)M.dim_vox[1];
-  for (uint32_t k = blockIdx.x; k < count; k += gridDim.x) {
-    const uint32_t b = list[k];
-    const uint64_t key = M.bkey[b];
-    const size_t bx = (size_t)(key & 0x1FFFFF) * 8, by = (size_t)((key >> 21) & 0x1FFFFF) * 8,
-                 bz = (size_t)(key >> 42) * 8;
-    for (int l = threadIdx.x; l < kBrickVox; l += blockDim.x) {
-      const unsigned long long word = __ldcg(M.vox + (size_t)b * kBrickVox + l);
-      const unsigned long long w = word & kWMask;
-      const long long S = word_S(word);
-      const float d = w ? __double2float_rn((double)S / ((double)w * 1048576.0)) : M.tau;
-      dense[((bz + (l >> 6)) * Y + by + ((l >> 3) & 7)) * X + bx + (l & 7)] = d;
+  __shared__ uint32_t s_brick[256], s_n, s_first;
+  const uint32_t count = min(__ldcg(&M.ctl->pool_count), M.pool_blocks);
+  if (whole) {
+    for (uint32_t b = blockIdx.x; b < count; b += gridDim.x) dense_brick(M, b, dense);
+    return;
+  }
+  for (uint64_t base = blockIdx.x; base < count; base += 256ull * gridDim.x) {
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    const uint64_t at = base + (uint64_t)threadIdx.x * gridDim.x;
+    if (at < count) {
+      uint32_t val, stamp;
+      if (find_slot(M, M.bkey[at], &val, &stamp) >= 0 && stamp != taken[at]) {
+        taken[at] = stamp;
+        s_brick[atomicAdd(&s_n, 1u)] = (uint32_t)at;
+      }
     }
+    __syncthreads();
+    const uint32_t n = s_n;
+    if (threadIdx.x == 0 && n) s_first = atomicAdd(nlist, n);
+    for (uint32_t i = 0; i < n; ++i) dense_brick(M, s_brick[i], dense);
+    __syncthreads();
+    if (threadIdx.x < n && s_first + threadIdx.x < M.pool_blocks)
+      list[s_first + threadIdx.x] = s_brick[threadIdx.x];
+    __syncthreads();  // s_brick and s_n are written again
   }
 }
 
@@ -104,17 +123,21 @@ __global__ void __launch_bounds__(256) k_dense_view(MapView M, const uint32_t* _
 // 0.35 ms.
 constexpr int kCellEdge = kBrick + 1, kCornerEdge = kBrick + 2;
 
-__global__ void __launch_bounds__(256) k_cell_view(MapView M, const uint32_t* __restrict__ list,
-                                                   const uint32_t* __restrict__ nlist,
+// The last CTA to end empties the list for the next update (`ended`: zero between
+// launches). `whole`: every brick of the box, without a list.
+__global__ void __launch_bounds__(256) k_cell_view(MapView M, int whole, const uint32_t* __restrict__ list,
+                                                   uint32_t* __restrict__ nlist,
+                                                   uint32_t* __restrict__ ended,
                                                    const float* __restrict__ dense,
                                                    float4* __restrict__ cells,
                                                    uint32_t* __restrict__ seen) {
   __shared__ float s_d[kCornerEdge * kCornerEdge * kCornerEdge];
   __shared__ uint32_t s_seen;  // of the 8 blocks the brick's cells lie in
-  const uint32_t count = __ldcg(nlist);
   const int X = M.dim_vox[0], Y = M.dim_vox[1], Z = M.dim_vox[2];
+  const uint32_t count = whole ? (uint32_t)((X / 8) * (Y / 8) * (Z / 8)) : min(__ldcg(nlist), M.pool_blocks);
   for (uint32_t k = blockIdx.x; k < count; k += gridDim.x) {
-    const uint64_t key = M.bkey[list[k]];
+    const uint64_t key = whole ? pack_brick(k % (X / 8), k / (X / 8) % (Y / 8), k / ((X / 8) * (Y / 8)))
+                               : M.bkey[list[k]];
     const int bx = (int)(key & 0x1FFFFF) * 8, by = (int)((key >> 21) & 0x1FFFFF) * 8,
               bz = (int)(key >> 42) * 8;
     __syncthreads();  // the previous brick's voxels and marks are no longer read
@@ -149,6 +172,15 @@ __global__ void __launch_bounds__(256) k_cell_view(MapView M, const uint32_t* __
                         (size_t)((by >> 3) + ((threadIdx.x >> 1) & 1))) * (X / 8 + 1) +
                        (size_t)((bx >> 3) + (threadIdx.x & 1));
       atomicOr(seen + (b >> 5), 1u << (b & 31));
+    }
+  }
+  if (whole) return;
+  __syncthreads();  // every thread has read the count
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(ended, 1u) == gridDim.x - 1u) {
+      *nlist = 0u;
+      *ended = 0u;
     }
   }
 }
@@ -905,9 +937,9 @@ cudaError_t launch_sview_fill(const MapView& M, int num_sms, const uint32_t* key
   return cudaGetLastError();
 }
 
-// Words of the dense view's list: bricks to update, their count, and the stamp at
-// which the view took each brick.
-size_t view_list_words(const MapView& M) { return 2 * (size_t)M.pool_blocks + 1; }
+// Words of the dense view's list: the bricks of an update, their count, its ended
+// CTAs, and the stamp at which the view took each brick.
+size_t view_list_words(const MapView& M) { return 2 * (size_t)M.pool_blocks + 2; }
 
 // Words of the dense view's block marks.
 size_t seen_words(const MapView& M) {
@@ -920,23 +952,27 @@ size_t seen_words(const MapView& M) {
 // *kernels: the kernels launched.
 cudaError_t launch_views(const MapView& M, int num_sms, bool fill, float* dense, float4* cells,
                          uint32_t* list, uint32_t* seen, int* kernels, cudaStream_t stream) {
-  *kernels = fill ? 5 : 3;
+  *kernels = fill ? 4 : 2;
   const size_t nd = (size_t)M.dim_vox[0] * M.dim_vox[1] * M.dim_vox[2];  // a multiple of 512
   const size_t nc = ((size_t)M.dim_vox[0] + 1) * (M.dim_vox[1] + 1) * (M.dim_vox[2] + 1);
-  uint32_t *nlist = list + M.pool_blocks, *taken = nlist + 1;
+  uint32_t *nlist = list + M.pool_blocks, *ended = nlist + 1, *taken = nlist + 2;
   if (fill) {
     k_fill<<<grid_for(nd / 4, 256, num_sms, 8), 256, 0, stream>>>(reinterpret_cast<float4*>(dense),
                                                                    nd / 4, M.tau);
     k_fill<<<grid_for(nc * 2, 256, num_sms, 8), 256, 0, stream>>>(cells, nc * 2, M.tau);
     cudaError_t z = cudaMemsetAsync(seen, 0, seen_words(M) * sizeof(uint32_t), stream);
+    if (z == cudaSuccess) z = cudaMemsetAsync(nlist, 0, 2 * sizeof(uint32_t), stream);
     if (z == cudaSuccess) z = cudaMemsetAsync(taken, 0xFF, M.pool_blocks * sizeof(uint32_t), stream);
     if (z != cudaSuccess) return z;
   }
-  cudaError_t e = cudaMemsetAsync(nlist, 0, sizeof(uint32_t), stream);
-  if (e != cudaSuccess) return e;
-  k_view_list<<<grid_for(M.pool_blocks, 256, num_sms, 8), 256, 0, stream>>>(M, taken, list, nlist);
-  k_dense_view<<<(unsigned)num_sms * 8, 256, 0, stream>>>(M, list, nlist, dense);
-  k_cell_view<<<(unsigned)num_sms * 8, 256, 0, stream>>>(M, list, nlist, dense, cells, seen);
+  // A CTA for each brick that there can be, up to a chip full of them. Boxes of up to
+  // four bricks per SM are taken whole: 8^3 bricks 20 us a scan, by their stamps 22 (26
+  // with the list in a launch of its own and a memset); 12^3 bricks by stamps 21, whole 25.
+  const size_t bricks = nd / kBrickVox;
+  const int whole = bricks <= (size_t)num_sms * 4;
+  const unsigned grid = (unsigned)std::min<size_t>(bricks, (size_t)num_sms * 8);
+  k_dense_view<<<grid, 256, 0, stream>>>(M, whole, taken, list, nlist, dense);
+  k_cell_view<<<grid, 256, 0, stream>>>(M, whole, list, nlist, ended, dense, cells, seen);
   return cudaGetLastError();
 }
 
